@@ -100,186 +100,328 @@ __device__ __forceinline__ void psp_select_kernel_body(const DavProb *__restrict
 
 __global__ void __launch_bounds__(kSelThreads) psp_select_kernel(const DavProb *__restrict__ probs, long long *__restrict__ pidx, int *__restrict__ pcount, int nprob_) {
     for (int w = blockIdx.x; w < nprob_; w += gridDim.x) {
+        if (probs[w].seed) continue;   // started from its own vector: no P-space
         psp_select_kernel_body(probs, pidx, pcount, w);
         __syncthreads();   // shared memory is reused by the next body
     }
 }
 
-// Per problem (kPsp threads): H in the pair functions, its lowest eigenvectors
-// by cyclic Jacobi (rotations applied by all threads), written to the start
-// slots 0..nv-1; the random start vector is cleared on the P-space determinants.
-__device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict__ probs, const HdiagDesc *__restrict__ hdd, const long long *__restrict__ pidx,
-                 const int *__restrict__ pcount, const DavState *__restrict__ st, int max_space,
-                 double *__restrict__ blk_energy, int w_) {
-    extern __shared__ double psm[];
-    double *A = psm;                       // [kPsp][kPsp]
-    double *V = psm + kPsp * kPsp;         // [kPsp][kPsp]
-    __shared__ double red[kPsp], red2[kPsp];
-    const DavProb p = probs[w_];
-    const HdiagDesc d = hdd[w_];
-    const int P = pcount[w_];
-    const int t = threadIdx.x;
-    const int n = p.nb;
-    const double rs2 = 0.7071067811865476;
-    // row t of A: <u_t|H|u_c>, every term of the pair functions written out (in
-    // an off-diagonal block, whose spin-flip image is not iterated, u_K = |K>)
-    if (t < P) {
-        const long long K = pidx[w_ * kPsp + t];
-        const int ka = (int)(K / n), kb = (int)(K % n);
-        for (int c = 0; c < P; c++) {
-            const long long L = pidx[w_ * kPsp + c];
-            const int la = (int)(L / n), lb = (int)(L % n);
-            const int nbra = (ka == kb || !p.sym) ? 1 : 2, nket = (la == lb || !p.sym) ? 1 : 2;
-            const double f = (nbra == 2 ? rs2 : 1.0) * (nket == 2 ? rs2 : 1.0);
-            double v = 0.0;
-            for (int x = 0; x < nbra; x++)
-                for (int y = 0; y < nket; y++) {
-                    // (row, column) local indices of the bra and ket determinants
-                    const int ba = x ? kb : ka, bb = x ? ka : kb, ca = y ? lb : la, cb = y ? la : lb;
-                    v += h_element(d.n, d.h1, d.eri, (uint32_t)d.strings[blk_row(p, ba)],
-                                   (uint32_t)d.strings[blk_col(p, bb)], (uint32_t)d.strings[blk_row(p, ca)],
-                                   (uint32_t)d.strings[blk_col(p, cb)]);
-                }
-            A[t * kPsp + c] = f * v;
-            V[t * kPsp + c] = t == c ? 1.0 : 0.0;
-        }
-    }
-    // blocks of the P-space: connected components of the coupling graph
-    // (|A_ij| above 1e-12 of the largest element); distant bodies make H split
-    // into (nearly) decoupled sectors, and the start block takes the lowest
-    // eigenvector of each of the lowest blocks first
-    __shared__ int comp[kPsp];
-    if (t == 0) {
-        double amax = 0.0;
-        for (int i = 0; i < P; i++)
-            for (int c = 0; c < P; c++) amax = fmax(amax, fabs(A[i * kPsp + c]));
-        const double thr = 1e-12 * amax;
-        for (int i = 0; i < P; i++) comp[i] = -1;
-        int ncomp = 0;
-        int stack[kPsp];
-        for (int i = 0; i < P; i++) {
-            if (comp[i] >= 0) continue;
-            int top = 0;
-            stack[top++] = i;
-            comp[i] = ncomp;
-            while (top > 0) {
-                const int u = stack[--top];
-                for (int v = 0; v < P; v++)
-                    if (comp[v] < 0 && fabs(A[u * kPsp + v]) > thr) {
-                        comp[v] = ncomp;
-                        stack[top++] = v;
-                    }
-            }
-            ncomp++;
-        }
-    }
-    __syncthreads();
-    // sweeps until the off-diagonal part is below 1e-26 of |A|_F^2 (a start
-    // guess needs no more); a rotation whose A_pq is below 1e-18 (|A_pp| +
-    // |A_qq|) only sets A_pq = A_qp = 0
+// Row-cyclic Jacobi on the symmetric P x P matrix A (shared memory, row
+// stride LD) by one warp: every lane derives the same rotation from the
+// settled entries, then rotates the columns of its rows, and after a warp
+// barrier its columns' rows and V.  Sweeps end once the off-diagonal part is
+// below 1e-26 of |A|_F^2 (a start guess needs no more); a rotation whose A_pq
+// is below 1e-18 (|A_pp| + |A_qq|) only sets A_pq = A_qp = 0.  Zero couplings
+// (other sectors, pair functions beyond a double excitation apart) are skipped.
+// The chain of dependent FP64 operations of one rotation bounds it; one warp
+// pays that chain once where a block of two warps paid it twice and three
+// block barriers with it.
+template <int MAXP>
+__device__ __forceinline__ void psp_jacobi_cyclic(double *A, double *V, int P, double *red, double *red2) {
+    constexpr int LD = MAXP + 1, R = (MAXP + 31) / 32;
+    const int lane = threadIdx.x;
     for (int sweep = 0; sweep < 40; sweep++) {
-        double off = 0.0, all = 0.0;
-        if (t < P)
+#pragma unroll
+        for (int u = 0; u < R; u++) {
+            const int t = lane + 32 * u;
+            if (t >= P) continue;
+            double off = 0.0, all = 0.0;
             for (int c = 0; c < P; c++) {
-                const double a2 = A[t * kPsp + c] * A[t * kPsp + c];
+                const double a2 = A[t * LD + c] * A[t * LD + c];
                 all += a2;
                 if (c != t) off += a2;
             }
-        red[t] = off;
-        red2[t] = all;
-        __syncthreads();
+            red[t] = off;
+            red2[t] = all;
+        }
+        __syncwarp();
         double tot = 0.0, fro = 0.0;
         for (int i = 0; i < P; i++) {
             tot += red[i];
             fro += red2[i];
         }
-        __syncthreads();
+        __syncwarp();
         if (tot <= 1e-26 * fro || tot == 0.0) break;
         for (int pp = 0; pp < P - 1; pp++)
             for (int q = pp + 1; q < P; q++) {
-                // every thread reads the same settled entries and derives the same
-                // rotation (no barrier); zero couplings (other sectors, pair
-                // functions beyond a double excitation apart) are skipped
-                const double apq = A[pp * kPsp + q];
+                const double apq = A[pp * LD + q];
                 if (fabs(apq) < 1e-300) continue;
-                const double app = A[pp * kPsp + pp], aqq = A[q * kPsp + q];
+                const double app = A[pp * LD + pp], aqq = A[q * LD + q];
+                __syncwarp();   // every lane has read the rotation's entries
                 if (fabs(apq) <= 1e-18 * (fabs(app) + fabs(aqq))) {
-                    __syncthreads();   // every thread has read A[pp][q]
-                    if (t == 0) A[pp * kPsp + q] = A[q * kPsp + pp] = 0.0;
-                    __syncthreads();
+                    if (lane == 0) A[pp * LD + q] = A[q * LD + pp] = 0.0;
+                    __syncwarp();
                     continue;
                 }
                 double c, sn;
                 jacobi_rotation(app, aqq, apq, c, sn);
-                __syncthreads();   // every thread has read A[pp][q], A[pp][pp], A[q][q]
-                if (t < P) {
-                    const double arp = A[t * kPsp + pp], arq = A[t * kPsp + q];
-                    A[t * kPsp + pp] = c * arp - sn * arq;
-                    A[t * kPsp + q] = sn * arp + c * arq;
+#pragma unroll
+                for (int u = 0; u < R; u++) {
+                    const int t = lane + 32 * u;
+                    if (t >= P) continue;
+                    const double arp = A[t * LD + pp], arq = A[t * LD + q];
+                    A[t * LD + pp] = c * arp - sn * arq;
+                    A[t * LD + q] = sn * arp + c * arq;
                 }
-                __syncthreads();
-                if (t < P) {
-                    const double apr = A[pp * kPsp + t], aqr = A[q * kPsp + t];
-                    A[pp * kPsp + t] = c * apr - sn * aqr;
-                    A[q * kPsp + t] = sn * apr + c * aqr;
-                    const double vrp = V[t * kPsp + pp], vrq = V[t * kPsp + q];
-                    V[t * kPsp + pp] = c * vrp - sn * vrq;
-                    V[t * kPsp + q] = sn * vrp + c * vrq;
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < R; u++) {
+                    const int t = lane + 32 * u;
+                    if (t >= P) continue;
+                    const double apr = A[pp * LD + t], aqr = A[q * LD + t];
+                    A[pp * LD + t] = c * apr - sn * aqr;
+                    A[q * LD + t] = sn * apr + c * aqr;
+                    const double vrp = V[t * LD + pp], vrq = V[t * LD + q];
+                    V[t * LD + pp] = c * vrp - sn * vrq;
+                    V[t * LD + q] = sn * vrp + c * vrq;
                 }
-                __syncthreads();
+                __syncwarp();
             }
     }
-    // the nv lowest eigenvalues' columns, each sign fixed by its largest component
-    int nv, ns;
-    start_block(p.ndim, max_space, p.seed != nullptr, &nv, &ns);
-    if (p.seed) return;   // started from its own vector: no P-space guess
-    __shared__ int cols[kStartP];
-    if (t == 0) {
-        // eigenvalues in ascending order; each eigenvector's block is the block
-        // of its largest component
-        int order[kPsp], blk[kPsp];
-        bool used[kPsp];
-        for (int i = 0; i < P; i++) used[i] = false;
-        for (int r = 0; r < P; r++) {
-            int b = -1;
-            for (int i = 0; i < P; i++)
-                if (!used[i] && (b < 0 || A[i * kPsp + i] < A[b * kPsp + b])) b = i;
-            used[b] = true;
-            order[r] = b;
-            int g = 0;
-            for (int i = 1; i < P; i++)
-                if (fabs(V[i * kPsp + b]) > fabs(V[g * kPsp + b])) g = i;
-            blk[r] = comp[g];
+}
+
+// The same by NT threads in round-robin order: a step rotates n / 2 disjoint
+// index pairs at once, so every 2 x 2 block (pair i, pair j) of A changes on
+// its own, A' = R_i^T A_ij R_j, and a sweep is n - 1 steps of two barriers
+// instead of n (n - 1) / 2 dependent rotations.  The FP64 pipe (~1.8 FMA per
+// clock and SM on this part) bounds it: per step 16 operations per block above
+// the diagonal (the other half is its mirror image) and 4 per element pair of
+// V.  n4 = P rounded up to a multiple of 4; the padding rows are zero and never
+// rotate.
+template <int MAXP, int NT>
+__device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, double *red, double *red2) {
+    static_assert(MAXP % 4 == 0 && NT >= MAXP && NT / 32 <= MAXP, "P-space sizes");
+    constexpr int LD = MAXP + 1;
+    __shared__ double rc[MAXP / 2], rsn[MAXP / 2];
+    __shared__ int rp[MAXP / 2], rq[MAXP / 2];       // the step's index pairs; rq < 0: no rotation
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int n4 = (P + 3) & ~3, npr = n4 / 2;
+    for (int e = t; e < n4 * n4; e += NT) {
+        const int r = e / n4, c = e % n4;
+        if (r >= P || c >= P) A[r * LD + c] = 0.0;
+    }
+    __syncthreads();
+    for (int sweep = 0; sweep < 40; sweep++) {
+        double off = 0.0, all = 0.0;
+        for (int e = t; e < P * P; e += NT) {
+            const int r = e / P, c = e % P;
+            const double a = A[r * LD + c];
+            all += a * a;
+            if (c != r) off += a * a;
         }
+        for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        __syncthreads();   // red is free again
+        if (lane == 0) {
+            red[warp] = off;
+            red2[warp] = all;
+        }
+        __syncthreads();
+        off = all = 0.0;
+        for (int w = 0; w < NT / 32; w++) {
+            off += red[w];
+            all += red2[w];
+        }
+        if (off <= 1e-26 * all || off == 0.0) break;
+        for (int step = 0; step < n4 - 1; step++) {
+            if (t < npr) {
+                // index n4 - 1 stays, the others turn
+                const int a = t == 0 ? n4 - 1 : (step + t) % (n4 - 1), b = t == 0 ? step : (step + n4 - 1 - t) % (n4 - 1);
+                const int pp = min(a, b), q = max(a, b);
+                const double apq = A[pp * LD + q];
+                int rot = 0;
+                if (!(fabs(apq) < 1e-300)) {
+                    const double app = A[pp * LD + pp], aqq = A[q * LD + q];
+                    if (fabs(apq) <= 1e-18 * (fabs(app) + fabs(aqq))) {
+                        A[pp * LD + q] = A[q * LD + pp] = 0.0;
+                    } else {
+                        double c, sn;
+                        jacobi_rotation(app, aqq, apq, c, sn);
+                        const double xp = c * app - sn * apq, xq = sn * app + c * apq;   // columns of row p
+                        const double yp = c * apq - sn * aqq, yq = sn * apq + c * aqq;   // columns of row q
+                        A[pp * LD + pp] = c * xp - sn * yp;
+                        A[q * LD + q] = sn * xq + c * yq;
+                        A[pp * LD + q] = A[q * LD + pp] = c * xq - sn * yq;
+                        rc[t] = c;
+                        rsn[t] = sn;
+                        rot = 1;
+                    }
+                }
+                rp[t] = pp;
+                rq[t] = rot ? q : -1 - q;
+            }
+            __syncthreads();
+            // blocks (i, j), i < j, of the npr pairs (npr is even): row r of the
+            // folded triangle holds pair row r and pair row npr - 1 - r
+            for (int e = t; e < npr / 2 * (npr - 1); e += NT) {
+                const int r = e / (npr - 1), c = e % (npr - 1);
+                const int i = c >= r ? r : npr - 1 - r, j = c >= r ? c + 1 : npr - 1 - c;
+                int qi = rq[i], qj = rq[j];
+                if (qi < 0 && qj < 0) continue;
+                const double ci = qi >= 0 ? rc[i] : 1.0, si = qi >= 0 ? rsn[i] : 0.0;
+                const double cj = qj >= 0 ? rc[j] : 1.0, sj = qj >= 0 ? rsn[j] : 0.0;
+                const int pi = rp[i], pj = rp[j];
+                if (qi < 0) qi = -1 - qi;
+                if (qj < 0) qj = -1 - qj;
+                const double a00 = A[pi * LD + pj], a01 = A[pi * LD + qj], a10 = A[qi * LD + pj], a11 = A[qi * LD + qj];
+                const double x00 = cj * a00 - sj * a01, x01 = sj * a00 + cj * a01;
+                const double x10 = cj * a10 - sj * a11, x11 = sj * a10 + cj * a11;
+                const double b00 = ci * x00 - si * x10, b10 = si * x00 + ci * x10;
+                const double b01 = ci * x01 - si * x11, b11 = si * x01 + ci * x11;
+                A[pi * LD + pj] = A[pj * LD + pi] = b00;
+                A[pi * LD + qj] = A[qj * LD + pi] = b01;
+                A[qi * LD + pj] = A[pj * LD + qi] = b10;
+                A[qi * LD + qj] = A[qj * LD + qi] = b11;
+            }
+            for (int e = t; e < npr * P; e += NT) {
+                const int i = e / P, r = e % P, q = rq[i];
+                if (q < 0) continue;
+                const double c = rc[i], sn = rsn[i], vp = V[r * LD + rp[i]], vq = V[r * LD + q];
+                V[r * LD + rp[i]] = c * vp - sn * vq;
+                V[r * LD + q] = sn * vp + c * vq;
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// Per problem (one block of NT threads): H in the pair functions, its lowest
+// eigenvectors, written to the start slots 0..nv-1; the random start vector is
+// cleared on the P-space determinants.
+//
+// NT = 256 runs the round-robin sweeps, NT = 32 the cyclic ones.  The round-robin
+// order is the faster one for a 64-function problem (21.8 ms with one rotation at
+// a time on 64 threads, 3.5 ms) and serves the whole spaces of an FP64 solve,
+// where a last-bit change of the start vector stays one.  With a quantised
+// contraction (FP64E and the mixed modes that end on it) such a change turns up
+// at the contraction's own level, ~5e-11 Eh, so those solves keep the order of
+// rotations, and with it every bit of their start vectors (an expansion of 298
+// sets: 68.6 ms of P-space solves before, 64.0 ms on one warp each).  So do the blocks of sectored spaces (MAXP = 24), which come by the
+// hundred thousand and share an SM sixteen at a time.
+template <int MAXP, int NT>
+__device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict__ probs, const HdiagDesc *__restrict__ hdd, const long long *__restrict__ pidx,
+                 const int *__restrict__ pcount, int max_space, double *__restrict__ blk_energy, int w_) {
+    constexpr int LD = MAXP + 1;
+    extern __shared__ double psm[];
+    double *A = psm;                       // [MAXP][LD]
+    double *V = psm + MAXP * LD;           // [MAXP][LD]
+    __shared__ double red[MAXP], red2[MAXP];
+    __shared__ unsigned long long adj[MAXP];
+    __shared__ int comp[MAXP], order[MAXP], blk[MAXP], cols[kStartP];
+    const DavProb p = probs[w_];
+    const HdiagDesc d = hdd[w_];
+    const int P = pcount[w_];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int n = p.nb;
+    const double rs2 = 0.7071067811865476;
+    // <u_r|H|u_c>, every term of the pair functions written out (in an
+    // off-diagonal block, whose spin-flip image is not iterated, u_K = |K>)
+    for (int e = t; e < P * P; e += NT) {
+        const int r = e / P, c = e % P;
+        const long long K = pidx[w_ * kPsp + r], L = pidx[w_ * kPsp + c];
+        const int ka = (int)(K / n), kb = (int)(K % n), la = (int)(L / n), lb = (int)(L % n);
+        const int nbra = (ka == kb || !p.sym) ? 1 : 2, nket = (la == lb || !p.sym) ? 1 : 2;
+        const double f = (nbra == 2 ? rs2 : 1.0) * (nket == 2 ? rs2 : 1.0);
+        double v = 0.0;
+        for (int x = 0; x < nbra; x++)
+            for (int y = 0; y < nket; y++) {
+                // (row, column) local indices of the bra and ket determinants
+                const int ba = x ? kb : ka, bb = x ? ka : kb, ca = y ? lb : la, cb = y ? la : lb;
+                v += h_element(d.n, d.h1, d.eri, (uint32_t)d.strings[blk_row(p, ba)],
+                               (uint32_t)d.strings[blk_col(p, bb)], (uint32_t)d.strings[blk_row(p, ca)],
+                               (uint32_t)d.strings[blk_col(p, cb)]);
+            }
+        A[r * LD + c] = f * v;
+        V[r * LD + c] = r == c ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    // blocks of the P-space: connected components of the coupling graph
+    // (|A_ij| above 1e-12 of the largest element); distant bodies make H split
+    // into (nearly) decoupled sectors, and the start block takes the lowest
+    // eigenvector of each of the lowest blocks first
+    {
+        double amax = 0.0;
+        for (int e = t; e < P * P; e += NT) amax = fmax(amax, fabs(A[(e / P) * LD + e % P]));
+        for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        if (lane == 0) red[warp] = amax;   // NT / 32 <= MAXP
+        __syncthreads();
+        for (int w = 0; w < NT / 32; w++) amax = fmax(amax, red[w]);
+        for (int r = t; r < P; r += NT) {
+            unsigned long long m = 0ull;
+            for (int c = 0; c < P; c++)
+                if (fabs(A[r * LD + c]) > 1e-12 * amax) m |= 1ull << c;
+            adj[r] = m;
+        }
+        __syncthreads();
+        if (t == 0) {
+            unsigned long long left = P == 64 ? ~0ull : (1ull << P) - 1ull;
+            for (int ncomp = 0; left; ncomp++) {
+                unsigned long long front = left & (~left + 1ull), members = 0ull;
+                while (front) {
+                    const int u = __ffsll((long long)front) - 1;
+                    members |= 1ull << u;
+                    comp[u] = ncomp;
+                    front = (front | (adj[u] & left)) & ~members;
+                }
+                left &= ~members;
+            }
+        }
+    }
+    __syncthreads();
+    if constexpr (NT == 32) psp_jacobi_cyclic<MAXP>(A, V, P, red, red2);
+    else psp_jacobi_pairs<MAXP, NT>(A, V, P, red, red2);
+    __syncthreads();
+    int nv, ns;
+    start_block(p.ndim, max_space, false, &nv, &ns);
+    // eigenvalues in ascending order; each eigenvector's block is the block of
+    // its largest component (entries that are not numbers keep their own place)
+    for (int r = t; r < P; r += NT) {
+        order[r] = r;
+        blk[r] = comp[r];
+    }
+    __syncthreads();
+    for (int r = t; r < P; r += NT) {
+        const double ev = A[r * LD + r];
+        int rank = 0, g = 0;
+        for (int i = 0; i < P; i++) {
+            const double o = A[i * LD + i];
+            if (o < ev || (o == ev && i < r)) rank++;
+            if (fabs(V[i * LD + r]) > fabs(V[g * LD + r])) g = i;
+        }
+        order[rank] = r;
+        blk[rank] = comp[g];
+    }
+    __syncthreads();
+    if (t == 0) {
         // rank of each block by its lowest eigenvalue: first[] = the eigenpair
         // index (in ascending order) that opens block rank 0, 1, ...
-        int first[kPsp], nb = 0;
-        for (int r = 0; r < P; r++) {
-            bool opens = true;
-            for (int q = 0; q < r; q++)
-                if (blk[q] == blk[r]) opens = false;
-            if (opens) first[nb++] = r;
-        }
+        int first[MAXP], nb = 0;
+        unsigned long long seen = 0ull, taken = 0ull;
+        for (int r = 0; r < P; r++)
+            if (!(seen >> blk[r] & 1ull)) {
+                seen |= 1ull << blk[r];
+                first[nb++] = r;
+            }
         if (blk_energy) {
-            blk_energy[2 * w_] = A[order[first[0]] * kPsp + order[first[0]]];
-            blk_energy[2 * w_ + 1] = nb > 1 ? A[order[first[1]] * kPsp + order[first[1]]] : 1e300;
+            blk_energy[2 * w_] = A[order[first[0]] * LD + order[first[0]]];
+            blk_energy[2 * w_ + 1] = nb > 1 ? A[order[first[1]] * LD + order[first[1]]] : 1e300;
         }
-        bool taken[kPsp];
-        for (int r = 0; r < P; r++) taken[r] = false;
         int nc = 0;
         const int seed = p.seed_block;
         if (seed > 0 && seed < nb) {
             // second pass: that block's lowest vector first, then the lowest
             // eigenvectors outside the blocks ranked below it
             cols[nc++] = order[first[seed]];
-            taken[first[seed]] = true;
+            taken |= 1ull << first[seed];
             for (int r = 0; r < P && nc < nv; r++) {
                 bool lower = false;
                 for (int q = 0; q < seed; q++)
                     if (blk[r] == blk[first[q]]) lower = true;
-                if (!taken[r] && !lower) {
+                if (!(taken >> r & 1ull) && !lower) {
                     cols[nc++] = order[r];
-                    taken[r] = true;
+                    taken |= 1ull << r;
                 }
             }
         } else {
@@ -287,26 +429,27 @@ __device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict_
             // eigenvalues), then the next lowest eigenvectors
             for (int k = 0; k < nb && nc < nv; k++) {
                 cols[nc++] = order[first[k]];
-                taken[first[k]] = true;
+                taken |= 1ull << first[k];
             }
         }
         for (int r = 0; r < P && nc < nv; r++)
-            if (!taken[r]) {
+            if (!(taken >> r & 1ull)) {
                 cols[nc++] = order[r];
-                taken[r] = true;
+                taken |= 1ull << r;
             }
     }
     __syncthreads();
-    if (t < P) {
-        const long long K = pidx[w_ * kPsp + t];
+    // the nv chosen columns, each sign fixed by its largest component
+    for (int u = t; u < P; u += NT) {
+        const long long K = pidx[w_ * kPsp + u];
         const int ka = (int)(K / n), kb = (int)(K % n);
         const long long KT = (long long)kb * n + ka;
         for (int r = 0; r < nv; r++) {
             const int col = cols[r];
             int g = 0;
             for (int i = 1; i < P; i++)
-                if (fabs(V[i * kPsp + col]) > fabs(V[g * kPsp + col])) g = i;
-            const double y = (V[g * kPsp + col] < 0 ? -1.0 : 1.0) * V[t * kPsp + col];
+                if (fabs(V[i * LD + col]) > fabs(V[g * LD + col])) g = i;
+            const double y = (V[g * LD + col] < 0 ? -1.0 : 1.0) * V[u * LD + col];
             double *Br = p.B + (long long)r * p.ndet;
             if (ka == kb || !p.sym) {
                 Br[K] = y;
@@ -323,11 +466,14 @@ __device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict_
     }
 }
 
-__global__ void __launch_bounds__(kPsp) psp_solve_kernel(const DavProb *__restrict__ probs, const HdiagDesc *__restrict__ hdd, const long long *__restrict__ pidx,
-                 const int *__restrict__ pcount, const DavState *__restrict__ st, int max_space,
-                 double *__restrict__ blk_energy, int nprob_) {
+// Whole spaces (MAXP = 64) or blocks of sectored spaces (MAXP = 24); a problem
+// started from its own vector needs no P-space guess.
+template <int MAXP, int NT>
+__global__ void __launch_bounds__(NT) psp_solve_kernel(const DavProb *__restrict__ probs, const HdiagDesc *__restrict__ hdd, const long long *__restrict__ pidx,
+                 const int *__restrict__ pcount, int max_space, double *__restrict__ blk_energy, int nprob_) {
     for (int w = blockIdx.x; w < nprob_; w += gridDim.x) {
-        psp_solve_kernel_body(probs, hdd, pidx, pcount, st, max_space, blk_energy, w);
+        if (probs[w].seed || (probs[w].gc != nullptr) != (MAXP < kPsp)) continue;
+        psp_solve_kernel_body<MAXP, NT>(probs, hdd, pidx, pcount, max_space, blk_energy, w);
         __syncthreads();   // shared memory is reused by the next body
     }
 }
@@ -395,14 +541,32 @@ int launch_pspace_start(ifci_handle_t h, const DavBatch &b, const HdiagDesc *d_h
         psp_select_kernel<<<stride_grid(h->device, b.nprob, 8), kSelThreads, 0, s>>>(b.d_probs, pidx, pcount, b.nprob);
         IFCI_LAUNCH_CHECK(h);
     }
-    const int smem = 2 * kPsp * kPsp * (int)sizeof(double);   // 64 KB
-    static SmemOptIn opt;
-    IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel, smem));
-    {
+    bool whole = false, sector = false;
+    for (const DavProb &p : b.probs) {
+        whole = whole || (!p.gc && !p.seed);
+        sector = sector || (p.gc && !p.seed);
+    }
+    constexpr int smem = 2 * kPsp * (kPsp + 1) * (int)sizeof(double);   // 65 KB
+    if (whole && b.precision == IFCI_FP64) {
+        static SmemOptIn opt;
+        IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel<kPsp, 256>, smem));
         ProfScope ps(h, s, PK_PSPACE);
-        psp_solve_kernel<<<stride_grid(h->device, b.nprob, 3), kPsp, smem, s>>>(b.d_probs, d_hd, pidx, pcount,
-                                                                                 b.d_state, b.max_space,
-                                                                                 b.d_blk_energy, b.nprob);
+        psp_solve_kernel<kPsp, 256><<<stride_grid(h->device, b.nprob, 3), 256, smem, s>>>(
+            b.d_probs, d_hd, pidx, pcount, b.max_space, b.d_blk_energy, b.nprob);
+        IFCI_LAUNCH_CHECK(h);
+    } else if (whole) {
+        static SmemOptIn opt;
+        IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel<kPsp, 32>, smem));
+        ProfScope ps(h, s, PK_PSPACE);
+        psp_solve_kernel<kPsp, 32><<<stride_grid(h->device, b.nprob, 3), 32, smem, s>>>(
+            b.d_probs, d_hd, pidx, pcount, b.max_space, b.d_blk_energy, b.nprob);
+        IFCI_LAUNCH_CHECK(h);
+    }
+    if (sector) {
+        constexpr int smem24 = 2 * kPspBlock * (kPspBlock + 1) * (int)sizeof(double);   // 9.6 KB
+        ProfScope ps(h, s, PK_PSPACE);
+        psp_solve_kernel<kPspBlock, 32><<<stride_grid(h->device, b.nprob, 16), 32, smem24, s>>>(
+            b.d_probs, d_hd, pidx, pcount, b.max_space, b.d_blk_energy, b.nprob);
         IFCI_LAUNCH_CHECK(h);
     }
     ProfScope ps(h, s, PK_SETUP);
