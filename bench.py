@@ -37,11 +37,10 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "iFCI increments/s & sigma TFLOP/s, 1 GB300, batched+mixed vs plain FP64 @1µEh"
-# dram__bytes_read.sum + dram__bytes_write.sum of one oz_contract_kernel launch
-# on CAS(6e,18o) (45.65 + 850.18 MB, 171 x 665,856 G elements; ncu capture of
-# `bench.py --case sigma --precision fp64e`); set to None whenever that kernel
-# changes until it is captured again
-OZ_DRAM_BYTES_PER_G_ELEMENT = (45.652992e6 + 850.175232e6) / (171 * 665856)
+# dram__bytes_read.sum + dram__bytes_write.sum of one oz_sigma_kernel launch on
+# CAS(6e,18o) per determinant (ncu capture of one FP64E sigma); set to None
+# whenever that kernel changes until it is captured again
+OZ_DRAM_BYTES_PER_DET = None
 UNIT = "increments/s"
 
 
@@ -438,15 +437,15 @@ def main():
     flops_full = 0.0
     flops_step = 0.0
     exec_step = 0.0
-    gelems_step = 0.0
+    dets_step = 0.0
     for (X, n, k), it in zip(subs, its):
         nd, fl = cost_of(n, k)
         npc = contracted_pairs(X, chain.body_sizes, Cb) if k > 1 else n * (n + 1) // 2
         it = float(it)
         flops_full += it * fl
-        flops_step += it * 2.0 * nd * npc * npc
-        exec_step += it * executed_oz_flops(n, k, npc)
-        gelems_step += it * nd * npc
+        flops_step += it * 2.0 * nd * npc * (oz_string_pairs(n, k, npc) if args.precision == "fp64e" else npc)
+        exec_step += it * issued_oz_flops(n, k, npc)
+        dets_step += it * nd
     sig_ms = sum(prof[k][0] for k in ("gather", "contract", "contract_hi", "scatter"))
     peaks = {}
     try:
@@ -470,12 +469,12 @@ def main():
         nlaunch = max(1, prof["contract_hi"][1])
         ach = flops_step / (c_ms / 1000.0) / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": bf, "unit": "TFLOP/s", "frac": ach / bf,
-                "traffic": (OZ_DRAM_BYTES_PER_G_ELEMENT * gelems_step / nlaunch
-                            if OZ_DRAM_BYTES_PER_G_ELEMENT else None),
-                "kernel": "oz_contract_kernel", "peak_source": bf_src,
-                "achieved_note": "FP64-equivalent FLOPs of the contraction (2 ndet npc^2 per sigma, npc the pairs "
-                                 "contracted: all pairs, or the intra-group pairs of a set of decoupled body "
-                                 "groups) / event-timed oz_contract_kernel time of one profiled step",
+                "traffic": (OZ_DRAM_BYTES_PER_DET * dets_step / nlaunch if OZ_DRAM_BYTES_PER_DET else None),
+                "kernel": "oz_sigma_kernel", "peak_source": bf_src,
+                "achieved_note": "FP64-equivalent FLOPs of the contraction (2 ndet npc k per sigma: npc output "
+                                 "pairs, all of them or the intra-group pairs of a set of decoupled body groups, "
+                                 "k of them with an excitation of the determinant's alpha string) / event-timed "
+                                 "oz_sigma_kernel time of one profiled step (its alpha and beta sums included)",
                 "achieved_full_npair": flops_full / (c_ms / 1000.0) / 1e12,
                 "full_npair_note": "2 ndet npair^2 per sigma over every pair (the contraction without the "
                                    "block structure of decoupled groups)",
@@ -563,9 +562,9 @@ def class_rooflines(subs, iters, kernel_ms, steps, hbm_gbs, fp64_tflops, max_spa
     """Achieved rates of the per-step kernel classes other than the contraction,
     from their CUDA-event times and algorithmic work:
 
-    * scatter (+ quantise, symmetrisation): per determinant and sigma, the G
-      values its alpha and beta lists read (2 nexc x 8 B), the quantised
-      copy read and written (16 B) and sigma read and written (16 B); HBM-bound.
+    * scatter (+ quantise): per determinant and sigma, c read (8 B), its digit
+      planes and the cleared integer sigma written (28 B), the integer sigma
+      read and sigma written (16 B); HBM-bound.
     * Davidson vector kernels: per determinant and iteration ~(5k + 8) x 8 B
       and ~9k FP64 FMAs at an average subspace size k = (max_space + 4) / 2
       (thick restarts keep 4 vectors); bound by the FP64 ALU on this GPU."""
@@ -575,9 +574,8 @@ def class_rooflines(subs, iters, kernel_ms, steps, hbm_gbs, fp64_tflops, max_spa
     kbar = (max_space + 4) / 2.0
     for (X, n, k), it in zip(subs, iters):
         nd = math.comb(n, k) ** 2
-        nexc = k * (n - k + 1)
         it = float(it)
-        sbytes += it * nd * (16.0 * nexc + 32.0)
+        sbytes += it * nd * 52.0
         vbytes += it * nd * (5.0 * kbar + 8.0) * 8.0
         vflops += it * nd * 9.0 * kbar * 2.0
     out = {}
@@ -642,7 +640,7 @@ def sigma_case(args, torch, ifci):
     if args.precision == "fp64e":
         c_ms = prof["contract_hi"][0] / steps
         line["contract_hi_tflops_algorithmic"] = fl / (c_ms / 1000.0) / 1e12
-        line["contract_hi_executed_fp16_tflops"] = executed_oz_flops(n, m) / (c_ms / 1000.0) / 1e12
+        line["contract_hi_executed_fp16_tflops"] = issued_oz_flops(n, m) / (c_ms / 1000.0) / 1e12
     print(json.dumps(line), flush=True)
     return 0
 
@@ -823,10 +821,17 @@ def fourbody_case(args, torch, ifci):
     return 0
 
 
+def oz_string_pairs(n: int, m: int, npc: int = 0) -> float:
+    """Pairs one string has an excitation on: m (n - m + 1) of the npair, in the
+    mean over the strings its share of them when only npc are contracted."""
+    return m * (n - m + 1) * ((npc or n * (n + 1) // 2) / (n * (n + 1) / 2))
+
+
 def executed_oz_flops(n: int, m: int, npc: int = 0) -> float:
-    """FP16 MMA FLOPs the FP64-emulating contraction issues for one sigma of one
-    problem: row-aligned tiles of 128 determinants x 96-pair output tiles x
-    the contracted pairs (npc, default all) rounded to 16, 15 slice products."""
+    """FP16 MMA FLOPs of one FP64-emulating sigma that contracts every pair of
+    npc (default all) for each determinant: row-aligned tiles of 128 determinants
+    x 96-pair output tiles x the pairs rounded to 16, 15 slice products.  The
+    yardstick that issued_oz_flops is set against."""
     nstr = math.comb(n, m)
     np_ = npc if npc else n * (n + 1) // 2
     if nstr >= 128:
@@ -839,6 +844,16 @@ def executed_oz_flops(n: int, m: int, npc: int = 0) -> float:
     for n0 in range(0, np_, 96):
         npad += (min(96, np_ - n0) + 15) // 16 * 16
     return 15.0 * 2.0 * tiles * 128 * npad * kpad
+
+
+def issued_oz_flops(n: int, m: int, npc: int = 0) -> float:
+    """FP16 MMA FLOPs the FP64-emulating sigma issues for one problem: per alpha
+    string tiles of 128 determinants x the output pairs (npc, default all)
+    rounded to 16 x the string's own pairs rounded to 16, 15 slice products."""
+    nstr = math.comb(n, m)
+    npad = ((npc or n * (n + 1) // 2) + 15) // 16 * 16
+    kpad = (math.ceil(oz_string_pairs(n, m, npc)) + 15) // 16 * 16
+    return 15.0 * 2.0 * nstr * ((nstr + 127) // 128) * 128 * npad * kpad
 
 
 def _dgemm_peak(dev):

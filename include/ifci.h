@@ -151,13 +151,12 @@ typedef struct {
  *   precision : ifci_precision_t of the contraction (FP64 exact path;
  *               the others round the contraction inputs, FP32 accumulate).
  * Sizes: BF16 and TF32 take npair <= 256 (norb <= 22), FP64E npair <= 304
- * (norb <= 24; above 204 pairs in K chunks of 192 whose exact int64 partial
- * sums are added), else UNSUPPORTED.  The intermediates take
- * 2 * npair * nstr^2 elements of the precision's storage type; a
- * spin-symmetric FP64E call above 2^31 G elements runs in row slabs of at
- * most 2^31 (16 GB), the scatter adding each slab's contribution into an
- * int64 accumulator, with the same result bit for bit.  Workspace beyond the
- * device's memory fails with OOM.
+ * (norb <= 24) and nstr <= 32767, else UNSUPPORTED (OOM for more strings).  The
+ * intermediates take 2 * npair * nstr^2 elements of the precision's storage
+ * type; FP64E takes 28 bytes per determinant instead (digit planes of c and
+ * -c, and the integer sigma), 56 without IFCI_SIGMA_SPIN_SYMMETRIC.  Its sums
+ * are integer sums: the result does not depend on their order.  Workspace
+ * beyond the device's memory fails with OOM.
  * Asynchronous on `stream`; uses handle workspace (grows it if needed). */
 int ifci_sigma(ifci_handle_t handle, const ifci_strings_t *str,
                const double *h1, const double *eri, const double *c, double *sigma,
@@ -256,10 +255,11 @@ typedef struct {
                             precision always finishes on exact sigmas. */
     int hi_precision;    /* mixed mode: sigma of restart vectors, IFCI_FP64 or IFCI_FP64E
                             (default IFCI_FP64E) */
-    long long det_budget;/* D elements (npair x determinants) per sigma wave; 0 = 2^31.
-                            A problem above it alone runs in row slabs of G on the
-                            FP64E path (bit-identical result); on the other paths it
-                            fails with OOM */
+    long long det_budget;/* D elements (npair x determinants) per sigma wave, on the FP64E path
+                            8-byte elements of its intermediates (~3.5 per determinant);
+                            0 = 2^31.  A problem above it alone takes a wave of its own on the
+                            FP64E path; on the other paths it fails with OOM.  The result does
+                            not depend on it */
     int graph_iters;     /* > 0: Davidson iterations are captured in blocks of this
                             many into one CUDA graph, replayed on a stream of the
                             handle (event-ordered with `stream`); 0 = launched one

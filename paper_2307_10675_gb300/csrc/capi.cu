@@ -43,16 +43,15 @@ int ifci_sigma(ifci_handle_t h, const ifci_strings_t *str, const double *h1, con
     const bool sym = sym_req && (tc || oz) && 2 * ndet < (1ll << 31);
     p.sym = sym ? 1 : 0;   // the pair map is placed below, before the plan is uploaded
     plan.probs.push_back(p);
-    // one wave; a spin-symmetric FP64E problem above 2^31 G elements runs in row slabs
-    const long long whole = sigma_elems(np, ndet);
-    IFCI_TRY(plan_sigma(h, plan, (oz && sym) ? std::min(whole, kSigmaSlabBudget) : whole, precision));
+    IFCI_TRY(plan_sigma(h, plan, sigma_elems(np, ndet), precision));   // one wave
     const size_t eb = sigma_elem_bytes(precision);
-    const long long delems_D = std::max(plan.max_delems, plan.max_qelems);
+    const long long delems_D = oz ? plan.max_qelems : std::max(plan.max_delems, plan.max_qelems);
+    const int ldj = oz ? oz_map_ld(nstr) : 0;
     size_t need = ws_round(sizeof(FoldDesc)) + ws_round((size_t)ld * ld * 8) + ws_round((size_t)ld * ld * 4) +
                   (tc ? ws_round((size_t)tc_operand_bytes(np, precision)) : 0) +
                   (oz ? ws_round((size_t)oz_operand_bytes(np)) + ws_round(8) : 0) +
-                  ((tc || oz) ? ws_round((size_t)nstr * kBlk16Stride) : 0) +
-                  (sym ? ws_round((size_t)nstr * pmap_ld(np) * 4) : 0) + plan_device_bytes(plan) +
+                  (oz ? ws_round(oz_map_elems(np, nstr) * 2) : 0) + (tc ? ws_round((size_t)nstr * kBlk16Stride) : 0) +
+                  (sym && tc ? ws_round((size_t)nstr * pmap_ld(np) * 4) : 0) + plan_device_bytes(plan) +
                   ws_round((size_t)delems_D * eb) + ws_round((size_t)plan.max_delems * eb);
     IFCI_TRY(ws_reserve(h, need));
     auto *fd = ws_take<FoldDesc>(h, 1);
@@ -64,22 +63,26 @@ int ifci_sigma(ifci_handle_t h, const ifci_strings_t *str, const double *h1, con
     plan.probs[0].Wf = Wf;
     plan.probs[0].Wtc = Wtc;
     plan.probs[0].Woz = Woz;
-    plan.probs[0].Wexp = oz ? (double *)(Woz + (oz_operand_bytes(np) - np * 8 - 256)) : nullptr;
+    plan.probs[0].Wexp = oz ? (double *)(Woz + (oz_operand_bytes(np) - 256)) : nullptr;
     plan.probs[0].dscale = 2.0;
-    uint8_t *blk = (tc || oz) ? ws_take<uint8_t>(h, (size_t)nstr * kBlk16Stride) : nullptr;
+    uint16_t *jmap = oz ? ws_take<uint16_t>(h, oz_map_elems(np, nstr)) : nullptr;
+    plan.probs[0].jmap = jmap;
+    plan.probs[0].ldj = ldj;
+    uint8_t *blk = tc ? ws_take<uint8_t>(h, (size_t)nstr * kBlk16Stride) : nullptr;
     plan.probs[0].blk = blk;
-    int32_t *pmap = sym ? ws_take<int32_t>(h, (size_t)nstr * pmap_ld(np)) : nullptr;
+    int32_t *pmap = sym && tc ? ws_take<int32_t>(h, (size_t)nstr * pmap_ld(np)) : nullptr;
     plan.probs[0].pmap = pmap;
     FoldDesc f{n, 2 * str->nelec_spin, ld, h1, eri, W};
     IFCI_CUDA_TRY(h, cudaMemcpyAsync(fd, &f, sizeof(f), cudaMemcpyHostToDevice, s));
     IFCI_TRY(launch_fold(h, 1, fd, np, s));
     if (blk) IFCI_TRY(launch_exc_blocks(h, nstr, nexc, str->exc, blk, s));
     if (pmap) IFCI_TRY(launch_pair_map(h, nstr, nexc, np, str->exc, pmap, s));
+    if (jmap) IFCI_TRY(launch_oz_map(h, nstr, nexc, np, str->exc, jmap, s));
     IFCI_TRY(upload_plan(h, plan, s));
     if (precision == IFCI_FP32) IFCI_TRY(launch_convert_w(h, 1, plan.d_probs, s));
     if (tc) IFCI_TRY(launch_tc_pack_w(h, 1, plan.d_probs, precision, s));
     if (oz) {
-        IFCI_TRY(launch_oz_pack_w(h, 1, plan.d_probs, s));
+        IFCI_TRY(launch_oz_pack_w(h, 1, plan.d_probs, np, s));
         IFCI_TRY(launch_oz_dscale(h, plan.d_probs, c, ndet, s));
     }
     void *D = ws_take<char>(h, (size_t)delems_D * eb);

@@ -17,7 +17,6 @@
 
 #include "dav_driver.cuh"
 #include "hamiltonian.cuh"
-#include "tc_gather.cuh"
 
 namespace ifci {
 
@@ -125,41 +124,37 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         sp.n = p.n; sp.nstr = nstr; sp.nexc = nexc; sp.np = np; sp.ld = np;
         sp.ndet = ndet; sp.stride = ndet;
         sp.sym = ((tc || oz) && 2ll * nstr * nstr < (1ll << 31)) ? 1 : 0;   // plan_sigma keeps it for tensor cores
-        // a spin-symmetric FP64E problem above the budget runs in row slabs of
-        // G; any other must fit one wave whole
-        if (!(oz && !lo && sp.sym)) max_pd = std::max(max_pd, sigma_elems(np, ndet));
+        if (lo || !oz) max_pd = std::max(max_pd, sigma_elems(np, ndet));   // D and G of a problem stay whole there
         sum_pd += sigma_elems(np, ndet);
         sp.dscale = 2.0;   // basis vectors are normalised: |D| <= 2
         hi.probs.push_back(sp);
         lop.probs.push_back(sp);
     }
-    // FP64E contraction of a sectored unit over its intra-group pairs
+    // FP64E sigma of a sectored unit over its intra-group pairs
     std::vector<std::vector<int32_t>> act(nu);
-    std::vector<std::vector<uint8_t>> pact(nu);
+    std::vector<std::vector<int16_t>> pinv(nu);
     for (int u = 0; u < nu; u++) {
         const Unit &U = units[u];
         if (!oz || !U.sector || U.label.empty() || !hi.probs[u].sym) continue;
         const int n = U.spec.n, np = n * (n + 1) / 2;
-        pact[u].assign(np, 0);
+        pinv[u].assign(np, -1);
         for (int P = 0; P < n; P++)
             for (int Q = 0; Q <= P; Q++)
                 if (U.label[P] == U.label[Q]) {
+                    pinv[u][P * (P + 1) / 2 + Q] = (int16_t)act[u].size();
                     act[u].push_back(P * (P + 1) / 2 + Q);
-                    pact[u][P * (P + 1) / 2 + Q] = 1;
                 }
         hi.probs[u].npc = (int)act[u].size();
     }
-    std::vector<size_t> act_off(nu + 1, 0), pact_off(nu + 1, 0);
-    int ncompact = 0;
+    std::vector<size_t> act_off(nu + 1, 0), pinv_off(nu + 1, 0);
     for (int u = 0; u < nu; u++) {
         act_off[u + 1] = act_off[u] + act[u].size();
-        pact_off[u + 1] = pact_off[u] + pact[u].size();
-        if (!act[u].empty()) ncompact++;
+        pinv_off[u + 1] = pinv_off[u] + pinv[u].size();
     }
     long long budget = o.det_budget > 0 ? o.det_budget : (1ll << 31);   // two 16 GB intermediates
     budget = std::max(budget, max_pd);
     budget = std::min(budget, std::max(sum_pd, max_pd));
-    for (int u = 0; u < nu; u++)   // placeholder until the device copy exists: plan_sigma tiles over npc
+    for (int u = 0; u < nu; u++)   // placeholder until the device copy exists: plan_sigma takes npc
         if (!act[u].empty()) hi.probs[u].act = act[u].data();
     IFCI_TRY(plan_sigma(h, hi, budget, hi_prec));
     if (lo) IFCI_TRY(plan_sigma(h, lop, budget * 8 / (long long)sigma_elem_bytes(o.precision), o.precision));
@@ -175,11 +170,11 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         std::vector<void *> Wtc;
         std::vector<char *> Woz;
         std::vector<double *> hd, B, S, cblk;
-        std::vector<int32_t *> act, pmapc;
-        std::vector<uint8_t *> pact;
+        std::vector<uint16_t *> jm, jmc;
+        OzMapDesc *mdesc = nullptr;
+        std::vector<uint8_t *> kcnt;
         int32_t *act_all = nullptr;
-        uint8_t *pact_all = nullptr;
-        CompactDesc *cdesc = nullptr;
+        int16_t *pinv_all = nullptr;
         int *sidx = nullptr;
         DavProb *probs = nullptr;
         DavState *state = nullptr;
@@ -201,32 +196,29 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
     };
     auto carve = [&](Carver &c, Mem &m) {
         const int nc = (int)cls_keys.size();
-        m.st.resize(nc); m.ex.resize(nc); m.bl.resize(nc); m.pm.assign(nc, nullptr);
+        m.st.resize(nc); m.ex.resize(nc); m.bl.assign(nc, nullptr); m.pm.assign(nc, nullptr); m.jm.assign(nc, nullptr);
         for (int k = 0; k < nc; k++) {
             const int nn = cls_keys[k].first, mm = cls_keys[k].second;
             const int nstr = (int)binom(nn, mm), nexc = mm * (nn - mm + 1), np = nn * (nn + 1) / 2;
             m.st[k] = c.take<uint64_t>(nstr);
             m.ex[k] = c.take<int32_t>((size_t)nstr * nexc);
-            m.bl[k] = c.take<uint8_t>((size_t)nstr * kBlk16Stride);
-            // Davidson vectors are spin-flip symmetric: the tensor-core sigmas use
+            // Davidson vectors are spin-flip symmetric: the BF16 and TF32 sigmas use
             // the alpha-only gathers where the pair map's offsets fit in int32
-            if ((tc || oz) && 2ll * nstr * nstr < (1ll << 31)) m.pm[k] = c.take<int32_t>((size_t)nstr * pmap_ld(np));
+            if (tc) m.bl[k] = c.take<uint8_t>((size_t)nstr * kBlk16Stride);
+            if (tc && 2ll * nstr * nstr < (1ll << 31)) m.pm[k] = c.take<int32_t>((size_t)nstr * pmap_ld(np));
+            if (oz) m.jm[k] = c.take<uint16_t>(oz_map_elems(np, nstr));
         }
-        // active pairs of every sectored unit in one array each (one copy, one
-        // compaction launch for all units)
-        m.act.assign(nu, nullptr); m.pmapc.assign(nu, nullptr); m.pact.assign(nu, nullptr);
+        // active pairs of every sectored unit in one array each (one copy for all units)
         m.act_all = c.take<int32_t>(act_off.back());
-        m.pact_all = c.take<uint8_t>(pact_off.back());
-        m.cdesc = c.take<CompactDesc>(ncompact);
-        for (int u = 0; u < nu; u++) {
-            if (act[u].empty()) continue;
-            const int nstr = (int)binom(units[u].spec.n, units[u].spec.m);
-            if (!c.count) {
-                m.act[u] = m.act_all + act_off[u];
-                m.pact[u] = m.pact_all + pact_off[u];
-            }
-            m.pmapc[u] = c.take<int32_t>((size_t)nstr * pmap_ld((int)act[u].size()));
-        }
+        m.pinv_all = c.take<int16_t>(pinv_off.back());
+        m.mdesc = c.take<OzMapDesc>(nu);
+        m.jmc.assign(nu, nullptr);
+        for (int u = 0; u < nu; u++)
+            if (!act[u].empty())
+                m.jmc[u] = c.take<uint16_t>(oz_map_elems((int)act[u].size(), (int)binom(units[u].spec.n, units[u].spec.m)));
+        m.kcnt.assign(nu, nullptr);
+        for (int u = 0; u < nu; u++)
+            if (!act[u].empty()) m.kcnt[u] = c.take<uint8_t>((size_t)binom(units[u].spec.n, units[u].spec.m));
         m.W.resize(nu); m.Wf.assign(nu, nullptr); m.Wtc.assign(nu, nullptr); m.Woz.assign(nu, nullptr);
         m.gc.assign(nu, nullptr); m.gs.assign(nu, nullptr);
         for (int u = 0; u < nu; u++) {
@@ -271,11 +263,12 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         m.hwp = c.take<int>(hw_prob.size());
         m.hws = c.take<long long>(hw_start.size());
         m.dst = c.take<double *>(n);
-        // D holds the gathered intermediate on the CUDA-core paths, only the
-        // quantised copies of c on the FP64-emulating one
-        m.D = c.take<char>((size_t)((hi_prec == IFCI_FP64E && !lo) ? std::max(hi.max_qelems, 1ll)
-                                                                     : std::max(budget, hi.max_qelems)) * 8);
-        m.G = c.take<char>((size_t)budget * 8);
+        // D holds the gathered intermediate on the CUDA-core paths and the quantised
+        // copies of c on the tensor-core ones, G the other intermediate or, on the
+        // FP64-emulating path, the integer sigma
+        const long long whole = (oz && !lo) ? 1 : budget;
+        m.D = c.take<char>((size_t)std::max(whole, oz ? hi.max_qelems : 0ll) * 8);
+        m.G = c.take<char>((size_t)std::max(whole, oz ? hi.max_delems : 0ll) * 8);
         m.hi_p = c.take<SigmaProb>(hi.probs.size());
         m.hi_i = c.take<WorkItem>(hi.items.size());
         m.hi_t = c.take<WorkItem>(hi.tiles.size());
@@ -304,8 +297,9 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         const int nn = cls_keys[k].first, mm = cls_keys[k].second;
         const int nstr = (int)binom(nn, mm), nexc = mm * (nn - mm + 1), np = nn * (nn + 1) / 2;
         IFCI_TRY(ifci_build_strings(h, nn, mm, mem.st[k], mem.ex[k], (ifci_stream_t)s));
-        IFCI_TRY(launch_exc_blocks(h, nstr, nexc, mem.ex[k], mem.bl[k], s));
+        if (mem.bl[k]) IFCI_TRY(launch_exc_blocks(h, nstr, nexc, mem.ex[k], mem.bl[k], s));
         if (mem.pm[k]) IFCI_TRY(launch_pair_map(h, nstr, nexc, np, mem.ex[k], mem.pm[k], s));
+        if (mem.jm[k]) IFCI_TRY(launch_oz_map(h, nstr, nexc, np, mem.ex[k], mem.jm[k], s));
     }
 
     // ---- descriptors
@@ -328,10 +322,12 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
             sp.exc = mem.ex[k];
             sp.blk = mem.bl[k];
             sp.pmap = mem.pm[k];
-            if (!sp.pmap) sp.sym = 0;
+            sp.jmap = mem.jm[k];
+            sp.ldj = oz_map_ld(nstr);
+            if (pl == &lop && !sp.pmap) sp.sym = 0;
             sp.W = mem.W[u]; sp.Wf = mem.Wf[u]; sp.Wtc = mem.Wtc[u];
             sp.Woz = mem.Woz[u];
-            sp.Wexp = oz ? (double *)(mem.Woz[u] + (oz_operand_bytes(np) - np * 8 - 256)) : nullptr;
+            sp.Wexp = oz ? (double *)(mem.Woz[u] + (oz_operand_bytes(np) - 256)) : nullptr;
             if (U.sector) {
                 sp.cbase = mem.gc[u]; sp.sbase = mem.gs[u];
                 sp.cslot = nullptr; sp.sslot = nullptr;
@@ -341,16 +337,12 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
                 sp.sslot = &mem.state[U.prob0].newest;
             }
             sp.active = (pl == &hi ? mem.uhi : mem.ulo) + u;
-            if (pl == &hi && mem.act[u]) {
-                sp.act = mem.act[u];
-                sp.pact = mem.pact[u];
-                sp.pmapc = mem.pmapc[u];
-            } else {
-                sp.act = nullptr;
-                sp.pact = nullptr;
-                sp.pmapc = nullptr;
-                sp.npc = sp.np;
-            }
+            const bool part = pl == &hi && !act[u].empty();
+            sp.act = part ? mem.act_all + act_off[u] : nullptr;
+            sp.kcnt = part ? mem.kcnt[u] : nullptr;
+            if (part) sp.jmap = mem.jmc[u];
+            sp.pinv = part ? mem.pinv_all + pinv_off[u] : nullptr;
+            if (!part) sp.npc = sp.np;
         }
     }
     for (int i = 0; i < n; i++) {
@@ -420,23 +412,22 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
                                      cudaMemcpyHostToDevice, s));
     IFCI_CUDA_TRY(h, cudaMemsetAsync(b.d_gs, 0, (size_t)n * kMaxSpace * kMaxSpace * 8, s));
     IFCI_CUDA_TRY(h, cudaMemsetAsync(b.d_y, 0, (size_t)n * kYStride * 8, s));
-    if (ncompact > 0) {
-        std::vector<int32_t> act_h(act_off.back());
-        std::vector<uint8_t> pact_h(pact_off.back());
-        std::vector<CompactDesc> cd;
+    if (act_off.back() > 0) {
+        std::vector<int32_t> act_h;
+        std::vector<int16_t> pinv_h;
         for (int u = 0; u < nu; u++) {
-            if (!mem.act[u]) continue;
-            std::copy(act[u].begin(), act[u].end(), act_h.begin() + act_off[u]);
-            std::copy(pact[u].begin(), pact[u].end(), pact_h.begin() + pact_off[u]);
-            const int k = cls[{units[u].spec.n, units[u].spec.m}];
-            const int nstr = (int)binom(units[u].spec.n, units[u].spec.m), np = units[u].spec.n * (units[u].spec.n + 1) / 2;
-            cd.push_back(CompactDesc{nstr, pmap_ld(np), (int)act[u].size(), pmap_ld((int)act[u].size()), mem.pm[k],
-                                     mem.act[u], mem.pmapc[u]});
+            act_h.insert(act_h.end(), act[u].begin(), act[u].end());
+            pinv_h.insert(pinv_h.end(), pinv[u].begin(), pinv[u].end());
         }
         IFCI_CUDA_TRY(h, cudaMemcpyAsync(mem.act_all, act_h.data(), act_h.size() * 4, cudaMemcpyHostToDevice, s));
-        IFCI_CUDA_TRY(h, cudaMemcpyAsync(mem.pact_all, pact_h.data(), pact_h.size(), cudaMemcpyHostToDevice, s));
-        IFCI_CUDA_TRY(h, cudaMemcpyAsync(mem.cdesc, cd.data(), cd.size() * sizeof(CompactDesc), cudaMemcpyHostToDevice, s));
-        IFCI_TRY(launch_compact_pair_maps(h, (int)cd.size(), mem.cdesc, s));
+        IFCI_CUDA_TRY(h, cudaMemcpyAsync(mem.pinv_all, pinv_h.data(), pinv_h.size() * 2, cudaMemcpyHostToDevice, s));
+        std::vector<OzMapDesc> md;
+        for (int u = 0; u < nu; u++)
+            if (mem.jmc[u])
+                md.push_back(OzMapDesc{(int)act[u].size(), hi.probs[u].ldj, hi.probs[u].nstr, mem.act_all + act_off[u],
+                                       mem.jm[cls[{units[u].spec.n, units[u].spec.m}]], mem.jmc[u], mem.kcnt[u]});
+        IFCI_CUDA_TRY(h, cudaMemcpyAsync(mem.mdesc, md.data(), md.size() * sizeof(OzMapDesc), cudaMemcpyHostToDevice, s));
+        IFCI_TRY(launch_oz_compact_maps(h, (int)md.size(), mem.mdesc, s));
     }
     {
         ProfScope ps(h, s, PK_SETUP);
@@ -445,7 +436,7 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         IFCI_TRY(launch_fold(h, nu, mem.fold, maxnp, s));
         if (lo) IFCI_TRY(launch_convert_w(h, nu, lop.d_probs, s));
         if (tc) IFCI_TRY(launch_tc_pack_w(h, nu, lop.d_probs, o.precision, s));
-        if (oz) IFCI_TRY(launch_oz_pack_w(h, nu, hi.d_probs, s));
+        if (oz) IFCI_TRY(launch_oz_pack_w(h, nu, hi.d_probs, maxnp, s));
         IFCI_TRY(launch_hdiag(h, mem.hdu, mem.hwp, mem.hws, (int)hw_prob.size(), kVecChunk, s));
         if (b.any_sector) IFCI_TRY(launch_sector_hd(h, b, s));
         b.d_pidx = mem.pidx;

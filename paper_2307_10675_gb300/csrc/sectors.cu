@@ -208,27 +208,7 @@ __global__ void __launch_bounds__(256) sector_expand_kernel(const DavProb *__res
     for (int w = blockIdx.x; w < nitem_; w += gridDim.x) sector_expand_kernel_body(probs, items, dst, w);
 }
 
-// pair map of a sectored unit restricted to its active pairs
-__global__ void __launch_bounds__(256) compact_pmaps_kernel(const CompactDesc *__restrict__ desc, int n) {
-    for (int u = blockIdx.x; u < n; u += gridDim.x) {
-        const CompactDesc d = desc[u];
-        const long long tot = (long long)d.nstr * d.ldc;
-        for (long long t = threadIdx.x; t < tot; t += blockDim.x) {
-            const long long r = t / d.ldc;
-            const int k = (int)(t % d.ldc);
-            d.pmapc[t] = k < d.npc ? d.pmap[r * d.ld + d.act[k]] : -1;
-        }
-    }
-}
-
 }  // namespace
-
-int launch_compact_pair_maps(ifci_handle_t h, int n, const CompactDesc *d_desc, cudaStream_t s) {
-    if (n <= 0) return IFCI_OK;
-    compact_pmaps_kernel<<<stride_grid(h->device, n, 8), 256, 0, s>>>(d_desc, n);
-    IFCI_LAUNCH_CHECK(h);
-    return IFCI_OK;
-}
 
 int launch_coupling(ifci_handle_t h, int nprob, const CoupDesc *d_desc, double tau, uint32_t *d_adj, cudaStream_t s) {
     coupling_kernel<<<nprob, 256, 0, s>>>(d_desc, tau, d_adj);

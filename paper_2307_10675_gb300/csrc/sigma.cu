@@ -16,9 +16,10 @@
 // part of D is the transpose of the alpha part, D_beta[A] = C X_A = (X_A C)^T,
 // so G = G_a + G_a^T with G_a = W D_alpha, and
 //   sigma = sum_A X_A G[A] + G[A] X_A = S + S^T,  S = sum_A X_A G_a[A] + G_a[A] X_A.
-// The tensor-core paths then gather alpha excitations only (every thread of
+// The BF16 and TF32 paths then gather alpha excitations only (every thread of
 // a tile row shares one alpha list, read from a dense pair map), run the
-// unchanged scatter on G_a to get S, and add the transpose of S.
+// unchanged scatter on G_a to get S, and add the transpose of S.  The FP64E
+// path (sigma_oz.cu) builds S in one kernel without D and G.
 #include <algorithm>
 
 #include "sigma.cuh"
@@ -152,31 +153,21 @@ scatter_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__
     s[I] = v;
 }
 
-// Quantised copy of c for the tensor-core gathers, written into the D buffer
-// (which those paths do not need): FP32 for BF16, and for FP64E the fixed
-// point integer X = round(c * 2^38 / dscale), so that their gathers run in FP32
-// or integer arithmetic (GB300 issues FP64 at a small fraction of FP32).
-template <int KIND>
+// FP32 copy of c for the tensor-core gathers, written into the D buffer
+// (which those paths do not need): their gathers then run in FP32 arithmetic
+// (GB300 issues FP64 at a small fraction of FP32).
 __global__ void __launch_bounds__(kGatherChunk)
-quantise_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items, char *__restrict__ qbuf) {
+quantise_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items, float *__restrict__ qbuf) {
     const WorkItem it = items[blockIdx.x];
     const SigmaProb &p = probs[it.prob];
     if (p.active && !*p.active) return;
     const long long I = it.start + threadIdx.x;
     if (I >= p.ndet) return;
     const double *c = p.cbase + (p.cslot ? (long long)*p.cslot : 0ll) * p.stride;
-    const long long off = p.qoff;
+    const float v = (float)c[I];
+    qbuf[p.qoff + I] = v;
     // symmetric gathers read the negated copy at off + ndet (sign by address)
-    if (KIND == 0) {
-        const float v = (float)c[I];
-        reinterpret_cast<float *>(qbuf)[off + I] = v;
-        if (p.sym) reinterpret_cast<float *>(qbuf)[off + p.ndet + I] = -v;
-    } else {
-        const double sc = 274877906944.0 / p.dscale;   // 2^38 / dscale
-        const long long v = __double2ll_rn(c[I] * sc);
-        reinterpret_cast<long long *>(qbuf)[off + I] = v;
-        if (p.sym) reinterpret_cast<long long *>(qbuf)[off + p.ndet + I] = -v;
-    }
+    if (p.sym) qbuf[p.qoff + p.ndet + I] = -v;
 }
 
 // sigma = S + S^T in place for the spin-flip-symmetric problems (each
@@ -196,42 +187,6 @@ sym_sum_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__
     const double v = s[K] + s[T];
     s[K] = v;
     s[T] = v;
-}
-
-// Scatter of the FP64-emulating path: G is int64 fixed point with one scale
-// per problem (2^-45 Wscale dscale), so sigma_I sums integers exactly and
-// converts once.
-__global__ void __launch_bounds__(kGatherChunk)
-scatter_fixed_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items,
-                     const long long *__restrict__ G) {
-    const WorkItem it = items[blockIdx.x];
-    const SigmaProb &p = probs[it.prob];
-    if (p.active && !*p.active) return;
-    const long long I = it.start + threadIdx.x;
-    if (I >= p.ndet) return;
-    const int nstr = p.nstr, nexc = p.nexc;
-    const long long ndet = p.ndet;
-    const int ia = (int)(I / nstr), ib = (int)(I % nstr);
-    const int32_t *__restrict__ ea = p.exc + (size_t)ia * nexc;
-    const int32_t *__restrict__ eb = p.exc + (size_t)ib * nexc;
-    const long long *__restrict__ Gp = G + p.doff;
-    const uint8_t *__restrict__ pact = p.pact;   // G rows of other pairs are not written (their W is zero)
-    long long acc = 0;
-    for (int e = 0; e < nexc; e++) {
-        const int32_t x = ea[e];
-        if (pact && !pact[exc_pair(x)]) continue;
-        const long long gv = Gp[(long long)exc_pair(x) * ndet + (long long)exc_J(x) * nstr + ib];
-        acc += (x & 1) ? -gv : gv;
-    }
-    const long long rowb = (long long)ia * nstr;
-    for (int e = 0; e < nexc; e++) {
-        const int32_t x = eb[e];
-        if (pact && !pact[exc_pair(x)]) continue;
-        const long long gv = Gp[(long long)exc_pair(x) * ndet + rowb + exc_J(x)];
-        acc += (x & 1) ? -gv : gv;
-    }
-    double *s = p.sbase + (p.sslot ? (long long)*p.sslot : 0ll) * p.stride;
-    s[I] = (double)acc * (p.Wexp[0] * p.dscale * 0x1p-45);
 }
 
 int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision) {
@@ -259,45 +214,26 @@ int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision
         SigmaProb &p = plan.probs[i];
         // the alpha-only form is a tensor-core gather; the CUDA-core paths build the full D
         p.sym = (p.sym && (tc || precision == IFCI_FP64E) && 2 * p.ndet < (1ll << 31)) ? 1 : 0;
-        long long need = sigma_elems(p.np, p.ndet);
-        if (need > budget && precision == IFCI_FP64E && p.sym) {
-            // row slabs of G: each its own wave, the scatter accumulating into S
-            if (p.npc <= 0 || !p.act) p.npc = p.np;
-            const int rpt = tcg::rows_per_tile(p.nstr);
-            const long long row_elems = (long long)p.np * p.nstr;
-            int rows = (int)std::min<long long>(p.nstr, budget / row_elems);
-            rows = rows / rpt * rpt;
-            if (rows < 1)
-                return set_error(h, IFCI_ERR_OOM, "sigma: one alpha row block needs %lld intermediate elements, "
-                                 "budget %lld", row_elems * rpt, budget);
-            close_wave((int)i);
-            const int nchunk = (((p.npc + 63) / 64) + 2) / 3;
-            for (int r0 = 0; r0 < p.nstr; r0 += rows) {
-                const int r1 = std::min(p.nstr, r0 + rows);
-                w.nprob = 1;
-                p.doff = 0;
-                p.qoff = 0;
-                w.delems = (long long)p.np * (r1 - r0) * p.nstr;
-                w.qelems = 3 * p.ndet;   // +-Q and the int64 accumulator S
-                w.k0 = (long long)r0 * p.nstr;
-                w.kn = (long long)(r1 - r0) * p.nstr;
-                w.slab_first = r0 == 0;
-                w.slab_last = r1 == p.nstr;
-                for (long long s0 = 0; s0 < p.ndet; s0 += kGatherChunk) {
-                    plan.items.push_back(WorkItem{(int)i, 0, s0});
-                    w.nitem++;
-                }
-                for (int n0 = 0; n0 < p.npc; n0 += oz_tile_n())
-                    for (int kc = 0; kc < nchunk; kc++) {
-                        size_t before = plan.tctiles.size();
-                        tcg::append_row_tiles(plan.tctiles, (int)i, n0 | (kc << 16), p.nstr, r0, r1);
-                        w.ntc += (int)(plan.tctiles.size() - before);
-                    }
-                close_wave((int)i);
+        if (precision == IFCI_FP64E) {
+            if (!p.act) p.npc = p.np;
+            // its digit planes and integer sigma (each once more for C^T without spin-flip symmetry)
+            if (!oz_supported(p.np, p.nstr, p.nexc))
+                return set_error(h, p.np > 304 ? IFCI_ERR_UNSUPPORTED : IFCI_ERR_OOM,
+                                 "FP64E: %d pairs, %d strings, %d excitations per string", p.np, p.nstr, p.nexc);
+            const long long q = (oz_plane_elems(p.nstr, p.sym) * 2 + 7) / 8, sv = (p.sym ? 1 : 2) * p.ndet;
+            if (w.nprob && w.delems + w.qelems + q + sv > budget) close_wave((int)i);
+            w.nprob++;
+            p.doff = w.delems;
+            w.delems += sv;
+            p.qoff = w.qelems * 4;   // FP16 elements
+            w.qelems += q;
+            for (long long s0 = 0; s0 < p.ndet; s0 += kGatherChunk) {
+                plan.items.push_back(WorkItem{(int)i, 0, s0});
+                w.nitem++;
             }
-            w.prob0 = (int)i + 1;
             continue;
         }
+        long long need = sigma_elems(p.np, p.ndet);
         if (need > budget)
             return set_error(h, IFCI_ERR_OOM, "sigma: one problem needs %lld intermediate elements, budget %lld",
                              need, budget);
@@ -316,18 +252,6 @@ int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision
             size_t before = plan.tctiles.size();
             tcg::append_row_tiles(plan.tctiles, (int)i, 0, p.nstr);
             w.ntc += (int)(plan.tctiles.size() - before);
-        } else if (precision == IFCI_FP64E) {
-            // one tile = up to 128 determinants x oz_tile_n() output pairs (sigma_oz.cu);
-            // the output-pair tiles of a problem run back to back so W stays resident longer
-            if (p.npc <= 0 || !p.act) p.npc = p.np;
-            // K chunks of 192 pairs keep every level sum exact (sigma_oz.cu)
-            const int nchunk = (((p.npc + 63) / 64) + 2) / 3;
-            for (int n0 = 0; n0 < p.npc; n0 += oz_tile_n())
-                for (int kc = 0; kc < nchunk; kc++) {
-                    size_t before = plan.tctiles.size();
-                    tcg::append_row_tiles(plan.tctiles, (int)i, n0 | (kc << 16), p.nstr);
-                    w.ntc += (int)(plan.tctiles.size() - before);
-                }
         } else {
             for (int m0 = 0; m0 < p.np; m0 += kGemmTM)
                 for (long long s0 = 0; s0 < p.ndet; s0 += kGemmTN) {
@@ -337,6 +261,32 @@ int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision
         }
     }
     close_wave((int)plan.probs.size());
+    if (precision == IFCI_FP64E) {
+        // one item per alpha string and pass, the problems with the longest items
+        // first (items go round robin to the CTAs), lists beyond the narrow limit last
+        for (SigmaWave &wv : plan.waves) {
+            std::vector<int> order(wv.nprob);
+            for (int k = 0; k < wv.nprob; k++) order[k] = wv.prob0 + k;
+            auto cost = [&](int i) { return (long long)plan.probs[i].nstr * plan.probs[i].npc; };
+            std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+                const bool wx = oz_wide(plan.probs[x].nexc), wy = oz_wide(plan.probs[y].nexc);
+                return wx != wy ? wy : cost(x) > cost(y);
+            });
+            wv.tc0 = (int)plan.tctiles.size();
+            wv.tile0 = (int)plan.tiles.size();
+            for (int i : order) {
+                const SigmaProb &p = plan.probs[i];
+                for (int pass = 0; pass < (p.sym ? 1 : 2); pass++)
+                    for (int ka = 0; ka < p.nstr; ka++) plan.tctiles.push_back(WorkItem{i, pass, ka});
+                (oz_wide(p.nexc) ? wv.nwide : wv.ntc) += p.nstr * (p.sym ? 1 : 2);
+                const int nt = (p.nstr + 31) / 32;
+                for (int ta = 0; ta < nt; ta++)
+                    for (int tb = ta; tb < nt; tb++) plan.tiles.push_back(WorkItem{i, tb, ta});
+            }
+            wv.nfin = (int)plan.tiles.size() - wv.tile0;
+        }
+        return IFCI_OK;
+    }
     plan.any_sym = false;
     for (const SigmaProb &p : plan.probs) plan.any_sym = plan.any_sym || p.sym;
     // dynamically scheduled tensor-core tiles: largest problems first (longest
@@ -356,7 +306,7 @@ size_t plan_device_bytes(const SigmaPlan &plan) {
 
 int upload_plan(ifci_handle_t h, SigmaPlan &plan, cudaStream_t s) {
     for (const SigmaProb &p : plan.probs)
-        if (p.sym && !p.pmap) return set_error(h, IFCI_ERR_INVALID_ARG, "sigma plan: symmetric problem without pair map");
+        if (p.sym && !p.pmap && !p.jmap) return set_error(h, IFCI_ERR_INVALID_ARG, "sigma plan: symmetric problem without pair map");
     plan.d_probs = ws_take<SigmaProb>(h, std::max<size_t>(1, plan.probs.size()));
     plan.d_items = ws_take<WorkItem>(h, std::max<size_t>(1, plan.items.size()));
     plan.d_tiles = ws_take<WorkItem>(h, std::max<size_t>(1, plan.tiles.size()));
@@ -381,7 +331,7 @@ int upload_plan(ifci_handle_t h, SigmaPlan &plan, cudaStream_t s) {
 // plan.d_probs, d_items, d_tiles, d_tctiles (each holding at least one entry).
 int upload_plan_to(ifci_handle_t h, SigmaPlan &plan, cudaStream_t s) {
     for (const SigmaProb &p : plan.probs)
-        if (p.sym && !p.pmap) return set_error(h, IFCI_ERR_INVALID_ARG, "sigma plan: symmetric problem without pair map");
+        if (p.sym && !p.pmap && !p.jmap) return set_error(h, IFCI_ERR_INVALID_ARG, "sigma plan: symmetric problem without pair map");
     if (!plan.d_probs || !plan.d_items || !plan.d_tiles || !plan.d_tctiles)
         return set_error(h, IFCI_ERR_INVALID_ARG, "sigma plan: device arrays not set");
     if (!plan.probs.empty())
@@ -397,52 +347,6 @@ int upload_plan_to(ifci_handle_t h, SigmaPlan &plan, cudaStream_t s) {
         IFCI_CUDA_TRY(h, cudaMemcpyAsync(plan.d_tctiles, plan.tctiles.data(),
                                          plan.tctiles.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, s));
     return IFCI_OK;
-}
-
-// The same for one row slab of a spin-flip-symmetric problem (SigmaWave::kn):
-// G holds alpha rows [r0, r1) only; the alpha loop takes the excitations whose
-// J row lies in the slab, the beta loop runs when I's own row does.  The sum
-// is carried in the int64 accumulator S across the slabs (exact, so the
-// result equals the unsplit scatter bit for bit) and converted on the last.
-__global__ void __launch_bounds__(kGatherChunk)
-scatter_fixed_slab_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items,
-                          const long long *__restrict__ G, long long *__restrict__ Qbuf, int r0, int r1, int first,
-                          int last) {
-    const WorkItem it = items[blockIdx.x];
-    const SigmaProb &p = probs[it.prob];
-    if (p.active && !*p.active) return;
-    const long long I = it.start + threadIdx.x;
-    if (I >= p.ndet) return;
-    const int nstr = p.nstr, nexc = p.nexc;
-    const long long kn = (long long)(r1 - r0) * nstr, k0 = (long long)r0 * nstr;
-    const int ia = (int)(I / nstr), ib = (int)(I % nstr);
-    const int32_t *__restrict__ ea = p.exc + (size_t)ia * nexc;
-    const uint8_t *__restrict__ pact = p.pact;
-    long long *S = Qbuf + p.qoff + 2 * p.ndet;
-    long long acc = first ? 0 : S[I];
-    for (int e = 0; e < nexc; e++) {
-        const int32_t x = ea[e];
-        const int J = exc_J(x);
-        if (J < r0 || J >= r1 || (pact && !pact[exc_pair(x)])) continue;
-        const long long gv = G[(long long)exc_pair(x) * kn + (long long)J * nstr + ib - k0];
-        acc += (x & 1) ? -gv : gv;
-    }
-    if (ia >= r0 && ia < r1) {
-        const int32_t *__restrict__ eb = p.exc + (size_t)ib * nexc;
-        const long long rowb = (long long)ia * nstr - k0;
-        for (int e = 0; e < nexc; e++) {
-            const int32_t x = eb[e];
-            if (pact && !pact[exc_pair(x)]) continue;
-            const long long gv = G[(long long)exc_pair(x) * kn + rowb + exc_J(x)];
-            acc += (x & 1) ? -gv : gv;
-        }
-    }
-    if (last) {
-        double *s = p.sbase + (p.sslot ? (long long)*p.sslot : 0ll) * p.stride;
-        s[I] = (double)acc * (p.Wexp[0] * p.dscale * 0x1p-45);
-    } else {
-        S[I] = acc;
-    }
 }
 
 int run_sigma(ifci_handle_t h, const SigmaPlan &plan, int precision, void *D, void *G, cudaStream_t s) {
@@ -483,31 +387,11 @@ int run_sigma(ifci_handle_t h, const SigmaPlan &plan, int precision, void *D, vo
                                                                    (const float *)G);
             IFCI_LAUNCH_CHECK(h);
         } else if (precision == IFCI_FP64E) {
-            {
-                ProfScope ps(h, s, PK_GATHER);
-                quantise_kernel<1><<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0, (char *)D);
-                IFCI_LAUNCH_CHECK(h);
-            }
-            IFCI_TRY(launch_oz_contract(h, plan, w, D, G, s));
-            ProfScope ps(h, s, PK_SCATTER);
-            if (w.kn) {
-                const int nstr = plan.probs[w.prob0].nstr;
-                scatter_fixed_slab_kernel<<<w.nitem, kGatherChunk, 0, s>>>(
-                    plan.d_probs, plan.d_items + w.item0, (const long long *)G, (long long *)D,
-                    (int)(w.k0 / nstr), (int)((w.k0 + w.kn) / nstr), w.slab_first, w.slab_last);
-            } else {
-                scatter_fixed_kernel<<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0,
-                                                                      (const long long *)G);
-            }
-            IFCI_LAUNCH_CHECK(h);
-            if (plan.any_sym && (!w.kn || w.slab_last)) {
-                sym_sum_kernel<<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0);
-                IFCI_LAUNCH_CHECK(h);
-            }
+            IFCI_TRY(run_sigma_oz(h, plan, w, D, G, s));
         } else {
             {
                 ProfScope ps(h, s, PK_GATHER);
-                quantise_kernel<0><<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0, (char *)D);
+                quantise_kernel<<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0, (float *)D);
                 IFCI_LAUNCH_CHECK(h);
             }
             IFCI_TRY(launch_tc_contract(h, plan, w, precision, D, G, s));

@@ -1,40 +1,72 @@
-// FP64-accurate contraction G = W D on the FP16 tensor cores (tcgen05).
+// FP64-accurate sigma build on the FP16 tensor cores (tcgen05), one fused
+// kernel per wave of problems.
 //
 // GB300 runs FP64 at ~1/1800 of its 16-bit tensor rate, so the sigma builds
-// that must be exact to FP64 level (Davidson restart vectors, final Rayleigh
-// quotients) are emulated with integer slices (an Ozaki-style splitting):
+// that must be exact to FP64 level are emulated with integer slices (an
+// Ozaki-style splitting):
 //
 //   W[A][B] = Wscale 2^-7 (w1 + 2^-8 w2 + ... + 2^-32 w5)    Wscale >= max|W|
-//   D[B][K] = dscale  2^-6 (d1 + 2^-8 d2 + ... + 2^-32 d5)    dscale >= max|D|
+//   c[K]    = dscale  2^-6 (d1 + 2^-8 d2 + ... + 2^-32 d5)    dscale >= 2 max|c|
 //
-// with every slice an integer in [-128, 128], exact in FP16.  D comes from the
-// fixed-point copy round(c 2^38 / dscale) of the input vector (quantise_kernel),
-// so the gather adds integers and the slices are the base-256 digits of
-// X + 128 (1 + 2^8 + ... + 2^32) minus 128, turned into FP16 by a byte permute
-// and one packed FP16 subtraction: no FP64 arithmetic in this kernel.
-// The product of two slices over K <= 204 terms stays below 2^24 even when the (up to five)
-// slice pairs of one scale level L = i + j share an accumulator, so each level
-// is summed exactly by the tensor cores in FP32; a problem with more pairs is
-// split into K chunks of 192 pairs, each its own tile, whose int64 partial
-// sums are added into G (exact, in any order).  The 15 slice pairs with
-// i + j <= 4 (0-based) are kept; the epilogue combines the five levels exactly
-// in int64, G = 2^-45 Wscale dscale sum_L 2^{8 (4 - L)} acc_L, and stores the
-// integer; the scatter sums those integers and converts once per determinant
-// (no FP64 arithmetic in the hot loop).  The dropped terms and the slice
-// truncation leave a relative error of order 2^-38 of max|W| max|D|.
+// with every slice an integer in [-128, 128], exact in FP16: c becomes the
+// fixed-point integer X = round(c 2^38 / dscale), whose slices are the
+// base-256 digits of X + 128 (1 + 2^8 + ... + 2^32) minus 128.  The 15 slice
+// products with i + j <= 4 (0-based) go to five FP32 accumulators, one per
+// scale level i + j; a level over K terms is an exact integer below
+// 5 2^14 K < 2^24 (K <= 112 here).  The levels are combined in int64,
+// T = sum_L 2^{8 (4 - L)} acc_L in units of 2^-45 Wscale dscale, every further
+// sum is an integer sum, and each determinant is converted once.  The dropped
+// terms and the slice truncation leave a relative error of order 2^-38 of
+// max|W| max|c|.
 //
-// Tile: 128 determinants (TMEM lanes) x 96 output pairs; five accumulators
-// of 96 FP32 columns (480 of the 512 TMEM columns).  K runs in 64-pair atoms:
-// the W slices of the next atom (5 x 96 x 64 FP16, pre-swizzled image) arrive
-// by bulk async copy into the second stage buffer while 512 threads (four per
-// determinant) build the five D slices of the current atom, then one thread
-// issues the 15 x 4 MMAs.  For spin-flip-symmetric vectors the gather reads
-// the alpha excitations only (see sigma.cu): one pair-map lookup and one
-// predicated load per element.
+// Spin-flip-symmetric c (C = C^T): with X_A the string matrix of E+_A and
+// T_A = sum_B W[A][B] X_B C the contraction over the alpha excitations alone,
+//   S = sum_A X_A T_A (alpha excitations of T) + T_A X_A (beta excitations),
+//   sigma = S + S^T.
+// For any other c the same S is built for C and for C^T (two passes), and
+// sigma = S(C) + S(C^T)^T.
+//
+// Row I_a of T needs only the pairs B that I_a has an alpha excitation on:
+// nexc = m (n - m + 1) of the npair = n (n + 1) / 2 pairs (48 of 171 for
+// CAS(6e,18o)), the same for every I_b of the row.  So the work item of a CTA
+// is one alpha string I_a, its contraction runs over K = nexc rows (rounded to
+// 16), and T never leaves the SM: the epilogue adds each T element
+// * to S[J_a][I_b] for the alpha excitation I_a -> J_a on its pair (one row of
+//   32 consecutive I_b per warp: coalesced 64-bit reductions in L2), and
+// * to S[I_a][J_b] for the beta excitation I_b -> J_b on its pair, in an int64
+//   accumulator row in shared memory (two 32-bit atomics per element: 64-bit
+//   ones are a compare-and-swap loop there, 23 to 43 clocks per warp against
+//   2 x 3.6), added to S once per item.
+// The earlier form contracted all pairs (dense K), wrote T (npair int64 per
+// determinant) to HBM and read it back in a scatter kernel.
+//
+// Operands arrive ready for the MMA: the digit planes of c and of -c (rows of
+// I_b for each J_a, written once per sigma) and the W image (rows of output
+// pairs for each contracted pair) are both MN-major, so a K row of either is a
+// contiguous run that cp.async places into the 128-byte-swizzled tile in
+// 16-byte chunks; no thread computes on an operand.  Output pairs run in
+// chunks of 48 columns: the five W slices of a chunk lie side by side
+// (5 x 48 = 240 columns), so digit slice j of c multiplies slices 0..4-j in
+// one MMA of N = (5 - j) 48 whose columns are the levels j..4 side by side:
+// five MMAs per 16 K rows in place of fifteen, each reading its A tile once.
+// Two accumulator sets (2 x 240 of the 512 TMEM columns) let the epilogue of a
+// chunk overlap the MMAs of the next.
+//
+// Bound: per 128 x 48 tile and 16 K rows 360 tensor clocks and 332 clocks of
+// shared-memory operand reads.  The epilogue is the longer side: ~25 issue
+// slots per T element, of which a determinant uses 28 % (its own excitations)
+// and a warp of 32 consecutive strings 90 %, and the two shared-memory
+// reductions (3.4 clocks a warp).  Sixteen warps share it, twelve for the beta
+// sums and four for the alpha sums; eight warps with both took 612 us.
+//
+// Measured, one sigma: CAS(6e,18o) 403 us (1282 us contraction + 254 us scatter
+// before), CAS(8e,20o) 29.4 ms (96.0 + 9.8 ms in three waves of 16 GB, now 0.7 GB
+// at once).
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "sigma.cuh"
-#include "tc_gather.cuh"
 #include "tcgen05.cuh"
 
 namespace ifci {
@@ -44,16 +76,25 @@ namespace {
 using namespace tc;
 
 constexpr int kS = 5;                       // slices per operand
-constexpr int kNT = 96;                     // output pairs per tile
-constexpr int kThreads = 512;               // 4 threads per determinant row
+constexpr int kNC = 48;                     // output pairs per chunk
+constexpr int kTBuf = kS * kNC;             // TMEM columns of one accumulator set
 constexpr int kOzTmemCols = 512;
-constexpr int kMaxNpExact = 204;            // exact level sums need at most 204 pairs per K chunk
-constexpr int kMaxNpTable = 304;            // 16-pair block offsets per string (kBlk16Stride) cover 304 pairs
-constexpr size_t kWStage = (size_t)kS * kNT * kAtomBytes;     // 61,440 B
-constexpr size_t kAStage = (size_t)kS * kTM * kAtomBytes;     // 81,920 B
+constexpr int kMaxK = 112;                  // contracted pairs of one string, rounded to 16
+constexpr int kMaxNp = 304;                 // pairs (norb <= 24)
+constexpr int kMaxStrings = 32767;          // 16-bit map entries (sign << 15 | J), 0xFFFF = none
+constexpr int kNarrowK = 51;                // up to here a level stays below 2^22 and a row sum of 26-bit words below 2^32
+constexpr int kMaxW = 8;                    // W chunk buffers
+constexpr int kBetaWarps = 12, kAlphaWarps = 4, kAWarps = 4, kWWarps = 2;
+constexpr int kEpiWarps = kBetaWarps + kAlphaWarps;
+constexpr int kOzThreads = 32 * (kEpiWarps + kAWarps + kWWarps + 1);
+constexpr int kSmemLimit = 232448 - 3696 - 1024;   // dynamic part: 227 KB less static (3.6 KB) and alignment
 constexpr long long kDigitBias = 128ll * 0x0101010101ll;      // 128 in each of the five digits
+constexpr uint32_t kNoMap = 0xFFFFu, kNone = 0xFFFFFFFFu;
+constexpr uint32_t kMagic = 0x4B400000u;     // FP32 1.5 2^23: kMagic + i are the bits of 1.5 2^23 + i, |i| < 2^22
+constexpr int kLowBits = 26;
 
-__host__ __device__ inline int n_tiles(int np) { return (np + kNT - 1) / kNT; }
+__host__ __device__ inline int np_pad(int np) { return round_up(np, 16); }
+__host__ __device__ inline int row_ld(int nstr) { return (nstr + 7) / 8 * 8; }   // digit plane row (halves)
 
 // slice a value in [-1, 1] into kS integers in [-128, 128]: x = 2^-7 sum_i 2^{-8i} s_i
 __device__ __forceinline__ void slice5(double x, float (&sl)[kS]) {
@@ -84,38 +125,198 @@ __device__ __forceinline__ uint32_t digit_pair_f16(uint32_t a, uint32_t b, int D
     return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// A tile's sub field: its first output pair (low 16 bits) and its K chunk (the
-// atoms [kChunkAtoms kc, kChunkAtoms (kc + 1)), so that every level sum of a
-// chunk stays an exact integer below 2^24 whatever npair is)
-constexpr int kChunkAtoms = 3;   // 192 pairs per chunk
-static_assert(kChunkAtoms * 64 <= kMaxNpExact, "a K chunk must keep its level sums exact");
-__host__ __device__ inline int tile_n0(int sub) { return sub & 0xFFFF; }
-__host__ __device__ inline int tile_kc(int sub) { return sub >> 16; }
-
-// W stage of local atom la of tile t
-__device__ __forceinline__ const uint8_t *stage_src(const SigmaProb *probs, const WorkItem *tiles, int t, int la) {
-    const WorkItem tile = tiles[t];
-    const SigmaProb &p = probs[tile.prob];
-    const int KA = k_atoms(p.act ? p.npc : p.np), nt = tile_n0(tile.sub) / kNT;
-    return (const uint8_t *)p.Woz + ((size_t)nt * KA + kChunkAtoms * tile_kc(tile.sub) + la) * kWStage;
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
 }
 
-// G[A][K] (int64, fixed point 2^-45 Wscale dscale) for one tile of 128 determinants x 96 pairs;
-// for a row slab (kn > 0) G[A][K - k0] with row stride kn.
-__global__ void __launch_bounds__(kThreads, 1)
-oz_contract_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ tiles, int ntile,
-                   const long long *__restrict__ Q, long long *__restrict__ G, int *__restrict__ err,
-                   int *__restrict__ counter, long long k0, long long kn) {
+// tcgen05 shared-memory descriptor of an MN-major operand, 128-byte swizzle:
+// atoms of 64 MN elements x 8 K rows (1024 B); `lbo` bytes between MN atoms,
+// 1024 B between groups of 8 K rows.
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t lbo) {
+    return (uint64_t)((addr & 0x3FFFF) >> 4) | (uint64_t)(lbo >> 4) << 16 | (uint64_t)(1024 >> 4) << 32 |
+           (uint64_t)1 << 46 | (uint64_t)2 << 61;
+}
+
+// kind::f16, FP16 x FP16 -> FP32, A and B MN-major
+__device__ __forceinline__ uint32_t idesc_f16_mn(int M, int N) { return idesc_f16(M, N) | (1u << 15) | (1u << 16); }
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool live) {
+    const int bytes = live ? 16 : 0;   // 0: the 16 bytes are zero-filled
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+// own copies landed and visible to the tensor core's proxy
+__device__ __forceinline__ void cp_async_done() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
+
+__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
+    uint32_t r;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
+    return r;
+}
+// (x, y) = (x sx, y sy) + (c, c)
+__device__ __forceinline__ void fma2(uint32_t &x, uint32_t &y, uint32_t sx, uint32_t sy, uint32_t c) {
+    asm("{\n\t.reg .b64 a, b, d;\n\t"
+        "mov.b64 a, {%0, %1};\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "mov.b64 d, {%4, %4};\n\t"
+        "fma.rn.f32x2 a, a, b, d;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+r"(x), "+r"(y)
+        : "r"(sx), "r"(sy), "r"(c));
+}
+__device__ __forceinline__ unsigned long long mad_wide(uint32_t a, uint32_t b, unsigned long long c) {
+    unsigned long long d;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+
+// Row sum in two 32-bit words of shared memory where the map entry m names a
+// string.  Narrow: the caller's words are T's low 26 bits and T >> 26, which
+// need no carry.  Wide: T's halves, the carry taken from the low word's old
+// value.  Predicated, so that the columns of an unrolled loop interleave.
+__device__ __forceinline__ void row_add_narrow(uint32_t m, uint32_t lo, uint32_t hi, uint32_t x, uint32_t y) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %0, 65535;\n\t"
+        "@p red.shared.add.u32 [%1], %3;\n\t"
+        "@p red.shared.add.u32 [%2], %4;\n\t}" ::"r"(m),
+        "r"(lo), "r"(hi), "r"(x), "r"(y));
+}
+__device__ __forceinline__ void row_add_wide(uint32_t m, uint32_t lo, uint32_t hi, uint32_t x, uint32_t y) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 o, c;\n\t"
+        "setp.ne.u32 p, %0, 65535;\n\t"
+        "mov.u32 o, 0;\n\t"
+        "@p atom.shared.add.u32 o, [%1], %3;\n\t"
+        "add.u32 o, o, %3;\n\t"
+        "setp.lt.u32 q, o, %3;\n\t"
+        "selp.u32 c, 1, 0, q;\n\t"
+        "add.u32 c, c, %4;\n\t"
+        "@p red.shared.add.u32 [%2], c;\n\t}" ::"r"(m),
+        "r"(lo), "r"(hi), "r"(x), "r"(y));
+}
+
+// *dst += v in L2 where `on`
+__device__ __forceinline__ void red_add_if(bool on, unsigned long long *dst, unsigned long long v) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %0, 0;\n\t"
+        "@p red.global.add.u64 [%1], %2;\n\t}" ::"r"((uint32_t)on),
+        "l"(dst), "l"(v)
+        : "memory");
+}
+
+struct OzGeom {
+    int nA, nW;      // stages of c tiles, chunk buffers of W
+    int kmax;        // K rows a buffer holds
+    int rows;        // strings the shared accumulator row holds; 0: the row is added to S in L2 directly
+    uint32_t m8, m16, m24;   // 2^8, 2^16, 2^24, in registers: one multiply-add per level instead of a shift and two adds
+};
+
+// The biased value of T from its level sums: each level as kMagic + acc, so
+// T + kBias = sum_L (kMagic + acc_L) 2^{8 (4 - L)} needs no sign handling.
+// T of levels that may reach 2^24 (levels 0 and 1 stay below 2^22 = 2 2^14 kMaxK)
+__device__ __forceinline__ unsigned long long wide_sum(float sg, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                                       uint32_t a4) {
+    const uint32_t h = __float_as_uint(fmaf(sg, __uint_as_float(a0), 12582912.0f)) - kMagic;
+    const uint32_t l = __float_as_uint(fmaf(sg, __uint_as_float(a1), 12582912.0f)) - kMagic;
+    long long T = __float2int_rn(sg * __uint_as_float(a4));
+    T += (long long)__float2int_rn(sg * __uint_as_float(a3)) * 256;
+    T += (long long)__float2int_rn(sg * __uint_as_float(a2)) * 65536;
+    T += (long long)(int)l * 16777216;
+    return (unsigned long long)T + ((unsigned long long)h << 32);
+}
+constexpr unsigned long long kBias = (unsigned long long)kMagic * 0x0101010101ull;
+__device__ __forceinline__ unsigned long long biased(const uint32_t (&b)[kS], const OzGeom &g) {
+    unsigned long long t = mad_wide(b[3], g.m8, b[4]);
+    t = mad_wide(b[2], g.m16, t);
+    t = mad_wide(b[1], g.m24, t);
+    return t + ((unsigned long long)b[0] << 32);
+}
+
+// The K rows of item (prob, ka): excitations e of string ka whose pair is
+// contracted, in list order.  out[k] = digit plane row (ROWS) or row of the W
+// image; returns their number.  NT threads with named barrier `id`.
+template <int NT, bool ROWS, typename TL>
+__device__ __forceinline__ int build_list(const SigmaProb &p, int ka, int tid, int id, TL *out, uint32_t *msk) {
+    constexpr int NWARP = NT / 32, R = (kMaxK + NT - 1) / NT;
+    const int lane = tid & 31, wi = tid >> 5, nexc = p.nexc, nstr = p.nstr;
+    const int32_t *row = p.exc + (size_t)ka * nexc;
+    const int16_t *pinv = p.pinv;
+    int val[R];
+    uint32_t bal[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        const int e = r * NT + tid;
+        int idx = -1, v = 0;
+        if (e < nexc) {
+            const int32_t x = row[e];
+            idx = pinv ? pinv[exc_pair(x)] : exc_pair(x);
+            v = ROWS ? exc_J(x) + ((x & 1) ? kS * nstr : 0) : idx;
+        }
+        val[r] = v;
+        bal[r] = __ballot_sync(0xffffffffu, idx >= 0);
+    }
+    named_sync(id, NT);   // the previous list is no longer read
+#pragma unroll
+    for (int r = 0; r < R; r++)
+        if (lane == 0) msk[r * NWARP + wi] = bal[r];
+    named_sync(id, NT);
+    int total = 0;
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        int at = 0;
+        for (int w = 0; w < R * NWARP; w++)
+            if (w < r * NWARP + wi) at += __popc(msk[w]);
+        at += __popc(bal[r] & ((1u << lane) - 1u));
+        if (bal[r] >> lane & 1u) out[at] = (TL)val[r];
+    }
+    for (int w = 0; w < R * NWARP; w++) total += __popc(msk[w]);
+    named_sync(id, NT);
+    return total;
+}
+
+// One item = alpha string tile.start of pass tile.sub (0: C, 1: C^T) of problem
+// tile.prob.  WIDE: items with more than kNarrowK excitations per string; ROW: the
+// item's row of S is summed in shared memory (always, unless WIDE).
+template <bool WIDE, bool ROW>
+__global__ void __launch_bounds__(kOzThreads, 1)
+oz_sigma_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items, int nitem,
+                const __half *__restrict__ Q, long long *__restrict__ S, int *__restrict__ err, OzGeom g) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_w[2], bar_mma;
+    __shared__ __align__(8) uint64_t b_fullA[2], b_emptyA[2], b_fullW[kMaxW], b_emptyW[kMaxW], b_tfull[2], b_tempty[2],
+        b_epi, b_drain;
     __shared__ uint32_t tmem_slot;
-    __shared__ int s_tile, s_next;
+    __shared__ int kp_of[2], okA[2], okW[2], lstA[kMaxK];
+    __shared__ uint16_t lstW[kMaxK];
+    __shared__ uint32_t mskA[4], mskW[4];
+    // the alpha excitations of the item's string, in column order, one copy per alpha warp:
+    // output pair, and J nstr | sign << 31 (element offset of row J of S)
+    __shared__ uint32_t s_aofs[kAlphaWarps][kMaxK];
+    __shared__ uint16_t s_acol[kAlphaWarps][kMaxK];
     uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *Wsm0 = base;                   // two W stages: [slice i][kNT rows][128 B]
-    uint8_t *Asm = base + 2 * kWStage;      // [slice j][128 rows][128 B]
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int row = tid & (kTM - 1), q = tid >> 7;   // determinant row of the tile, quarter
-    const uint32_t bw0 = smem_u32(&bar_w[0]), bw1 = smem_u32(&bar_w[1]), bm = smem_u32(&bar_mma);
+    const uint32_t stageA = (uint32_t)kS * g.kmax * 256, stageW = (uint32_t)g.kmax * 512;
+    uint8_t *Asm = base, *Wsm = base + g.nA * stageA;
+    uint32_t *rlo = (uint32_t *)(Wsm + g.nW * stageW), *rhi = rlo + g.rows;
+    // the warp index through a shuffle: uniform for the compiler, so that tensor
+    // addresses and descriptors stay in uniform registers (the instructions take
+    // no others; from a divergent value each operand is moved over, ~200 clocks an MMA)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
@@ -124,176 +325,320 @@ oz_contract_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restri
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        mbar_init(bw0, 1);
-        mbar_init(bw1, 1);
-        mbar_init(bm, 1);
+        for (int i = 0; i < 2; i++) {
+            mbar_init(smem_u32(&b_fullA[i]), 32 * kAWarps);
+            mbar_init(smem_u32(&b_emptyA[i]), 1);
+            mbar_init(smem_u32(&b_tfull[i]), 1);
+            mbar_init(smem_u32(&b_tempty[i]), kEpiWarps);
+        }
+        for (int i = 0; i < kMaxW; i++) {
+            mbar_init(smem_u32(&b_fullW[i]), 32 * kWWarps);
+            mbar_init(smem_u32(&b_emptyW[i]), 1);
+        }
+        mbar_init(smem_u32(&b_epi), 32 * kBetaWarps);
+        mbar_init(smem_u32(&b_drain), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    for (int i = tid; i < 2 * g.rows; i += kOzThreads) rlo[i] = 0u;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-
-    // tiles are handed out by a global counter (dynamic load balance); the tile
-    // after the current one is claimed early so that its first W stage can be
-    // prefetched during the current tile's last atom
-    uint32_t ph_m = 0;
-    uint32_t g = 0;            // W stages consumed so far: buffer g & 1, phase (g >> 1) & 1
     bool ok = true;
-    if (tid == 0) {
-        const int t = tcg::claim_tile(counter, probs, tiles, ntile);
-        s_tile = t;
-        if (t < ntile) bulk_load(smem_u32(Wsm0), stage_src(probs, tiles, t, 0), (uint32_t)kWStage, bw0);
-    }
-    __syncthreads();
-    for (int t = s_tile; t < ntile && ok;) {
-        if (tid == 0) s_next = tcg::claim_tile(counter, probs, tiles, ntile);
-        const WorkItem tile = tiles[t];
-        // descriptor fields in registers (the asm memory clobbers below would
-        // otherwise make the compiler reload them from global memory)
-        const SigmaProb &pg = probs[tile.prob];
-        // np: the pairs contracted (a sectored space: its active pairs, in compact order)
-        const int np = pg.act ? pg.npc : pg.np, nstr = pg.nstr, sym = pg.sym;
-        // G row stride: the problem's determinants, or those of its row slab [k0, k0 + kn)
-        const long long gld = kn ? kn : pg.ndet, doff = pg.doff;
-        const int32_t *pmap = pg.act ? pg.pmapc : pg.pmap;
-        const int32_t *act = pg.act;
-        const long long *C = Q + pg.qoff;   // round(c 2^38 / dscale) (and its negation when sym)
-        const int KA = k_atoms(np), n0 = tile_n0(tile.sub);
-        const int a0 = kChunkAtoms * tile_kc(tile.sub), a1 = min(KA, a0 + kChunkAtoms);
-        const bool chunked = KA > kChunkAtoms;   // partial sums: added to G (zeroed before the launch)
-        const int Nt = round_up(min(kNT, np - n0), 16);
-        const tcg::TileGeom geo = tcg::tile_geom(tile.start, nstr);
-        const bool live = row < geo.R * geo.Cw;
-        const int r = live ? row / geo.Cw : 0;
-        const int ka = geo.ka0 + r, kb = geo.kb0 + (live ? row % geo.Cw : 0);
-        const long long K = (long long)ka * nstr + kb;
-        int4 pmn[4];               // pair-map row of this thread's next block
-        if (sym && live) tcg::pmap_load16(pmap, np, ka, 4 * a0 + q, pmn);
-        for (int a = a0; a < a1; a++, g++) {
-            // ---- loads of this atom's block (pairs 64a + 16q .. + 16): they overlap
-            // the MMAs of the previous atom, which are still running
-            const int b = 4 * a + q;
-            long long x[16];
-#pragma unroll
-            for (int k = 0; k < 16; k++) x[k] = 0;
-            if (live) {
-                if (sym) {
-                    int4 pmc[4];
-#pragma unroll
-                    for (int u = 0; u < 4; u++) pmc[u] = pmn[u];
-                    if (a + 1 < a1) tcg::pmap_load16(pmap, np, ka, b + 4, pmn);
-                    tcg::gather_pm16<long long>(C, kb, pmc, x);
-                } else {
-                    tcg::gather_block16<long long>(probs[tile.prob], C, ka, kb, b, x);
-                }
-            }
-            // MMAs of the previous atom done: A and W buffer (g + 1) & 1 are free
-            // (thread 0 polls, the others wait at the barrier)
-            if (a > a0) {
-                if (!__syncthreads_and(tid == 0 ? (ok && mbar_wait(bm, ph_m)) : 1)) { ok = false; break; }
-                ph_m ^= 1;
-            }
-            // prefetch the next W stage (thread 0 wrote s_next itself: no barrier needed to read it)
-            if (tid == 0) {
-                const int nt2 = a + 1 < a1 ? t : s_next, na = a + 1 < a1 ? a + 1 - a0 : 0;
-                if (nt2 < ntile)
-                    bulk_load(smem_u32(Wsm0 + ((g + 1) & 1) * kWStage), stage_src(probs, tiles, nt2, na),
-                              (uint32_t)kWStage, ((g + 1) & 1) ? bw1 : bw0);
-            }
-            // ---- five digit slices of the block, two 16-byte chunks per slice
-#pragma unroll
-            for (int half = 0; half < 2; half++) {
-                uint32_t lo[8], hi[8];
-#pragma unroll
-                for (int e = 0; e < 8; e++) {
-                    const unsigned long long Xb = (unsigned long long)(x[8 * half + e] + kDigitBias);
-                    lo[e] = (uint32_t)Xb;
-                    hi[e] = (uint32_t)(Xb >> 32);
-                }
-                const int ch = 2 * q + half;
-                uint8_t *dst = Asm + row * kAtomBytes + ((ch ^ (row & 7)) << 4);
-#pragma unroll
-                for (int j = 0; j < kS; j++) {
-                    const int d = kS - 1 - j;          // slice j = digit d (j = 0 most significant)
-                    uint32_t w4[4];
-#pragma unroll
-                    for (int e = 0; e < 8; e += 2)
-                        w4[e / 2] = d == 4 ? digit_pair_f16(hi[e], hi[e + 1], 0) : digit_pair_f16(lo[e], lo[e + 1], d);
-                    *(uint4 *)(dst + (size_t)j * kTM * kAtomBytes) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-                }
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncthreads();
-            // ---- one thread: wait for this stage's W, issue the 15 x (up to 4) MMAs
-            if (tid == 0) {
-                ok = ok && mbar_wait((g & 1) ? bw1 : bw0, (g >> 1) & 1);
-                if (ok) {
+
+    if (warp < kBetaWarps) {
+        // ---- beta excitations: every T element to the item's row of S
+        const int q = warp & 3, part = warp >> 2;   // TMEM lane quarter, share of the columns
+        const uint32_t lane_base = (uint32_t)(q * 32) << 16, row_lo = smem_u32(rlo), row_hi = row_lo + 4u * (uint32_t)g.rows;
+        uint32_t tn = 0, ep = 0;
+        auto epi_sync = [&]() {   // bounded: a role that gave up must not hang the others
+            mbar_arrive(smem_u32(&b_epi));
+            const bool r = mbar_wait(smem_u32(&b_epi), ep & 1);
+            ep++;
+            return __all_sync(0xffffffffu, r) != 0;
+        };
+        for (int it = blockIdx.x; it < nitem && ok; it += gridDim.x) {
+            const WorkItem item = items[it];
+            const SigmaProb &p = probs[item.prob];
+            if (p.active && !*p.active) continue;
+            const int nstr = p.nstr, npad = np_pad(p.act ? p.npc : p.np), ldj = p.ldj, ka = (int)item.start;
+            long long *Srow = S + p.doff + (item.sub ? p.ndet : 0) + (long long)ka * nstr;
+            const uint2 *jmap = reinterpret_cast<const uint2 *>(p.jmap);
+            for (int mt = 0; mt * kTM < nstr && ok; mt++) {
+                const int ib0 = mt * kTM + q * 32;
+                const bool wlive = ib0 < nstr;
+                // map entries of four output pairs of this determinant's string
+                const uint2 *jcol = jmap + ib0 + lane;
+                for (int c0 = 0; c0 < npad; c0 += kNC, tn++) {
+                    const int w = min(kNC, npad - c0);
+                    const uint32_t buf = tn & 1;
+                    constexpr int kStep = kBetaWarps;   // columns between two groups of a warp
+                    auto map_of = [&](int cc) {
+                        return wlive && cc < w ? jcol[(size_t)((c0 + cc) >> 2) * ldj] : make_uint2(kNone, kNone);
+                    };
+                    uint2 jn[2] = {map_of(4 * part), map_of(4 * part + kStep)};
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&b_tfull[buf]), (tn >> 1) & 1))) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t idesc = idesc_f16(kTM, Nt);
-                    // descriptors of the stage bases; an offset below 256 KB adds (offset >> 4)
-                    const uint64_t ad0 = smem_desc(smem_u32(Asm));
-                    const uint64_t wd0 = smem_desc(smem_u32(Wsm0 + (g & 1) * kWStage));
-                    const int kst = min(4, (round_up(np, 16) - a * 64) / 16);
+                    for (int cc = 4 * part; cc < w && wlive; cc += 2 * kStep) {
+                        // two groups of four columns, all levels
+                        uint32_t v[2][kS][4];
 #pragma unroll
-                    for (int j = 0; j < kS; j++)
+                        for (int h = 0; h < 2; h++)
 #pragma unroll
-                        for (int i = 0; i + j < kS; i++)
+                            for (int L = 0; L < kS; L++)
+                                tmem_ld4(tmem + lane_base + buf * kTBuf + (uint32_t)(L * w + min(cc + kStep * h, w - 4)), v[h][L]);
+                        const uint2 jm[2] = {jn[0], jn[1]};
+                        jn[0] = map_of(cc + 2 * kStep);
+                        jn[1] = map_of(cc + 3 * kStep);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                            for (int ks = 0; ks < 4; ks++)
-                                if (ks < kst)
-                                    mma_f16(tmem + (uint32_t)((i + j) * kNT),
-                                            ad0 + (uint64_t)((j * kTM * kAtomBytes + ks * 32) >> 4),
-                                            wd0 + (uint64_t)((i * kNT * kAtomBytes + ks * 32) >> 4), idesc,
-                                            (a > a0 || j > 0 || ks > 0) ? 1u : 0u);
-                    mma_commit(bm);
+                        for (int h = 0; h < 2; h++)
+#pragma unroll
+                            for (int k = 0; k < 2; k++) {
+                                const uint32_t mw = k ? jm[h].y : jm[h].x;   // kNone past the last column
+                                const uint32_t s0 = 0x3F800000u | (mw << 16 & 0x80000000u), s1 = 0x3F800000u | (mw & 0x80000000u);
+                                if (!WIDE) {
+                                    // |acc| < 2^22: 1.5 2^23 +- acc is exact and holds it in its low bits
+#pragma unroll
+                                    for (int L = 0; L < kS; L++) fma2(v[h][L][2 * k], v[h][L][2 * k + 1], s0, s1, kMagic);
+                                }
+#pragma unroll
+                                for (int e = 2 * k; e < 2 * k + 2; e++) {
+                                    const uint32_t m = e & 1 ? mw >> 16 : mw & 0xFFFFu, j4 = (m & 0x7FFFu) * 4u;
+                                    if (WIDE) {
+                                        const unsigned long long T = wide_sum(__uint_as_float(e & 1 ? s1 : s0), v[h][0][e], v[h][1][e],
+                                                                              v[h][2][e], v[h][3][e], v[h][4][e]);
+                                        if (ROW) row_add_wide(m, row_lo + j4, row_hi + j4, (uint32_t)T, (uint32_t)(T >> 32));
+                                        else red_add_if(m != kNoMap, reinterpret_cast<unsigned long long *>(Srow) + (m & 0x7FFFu), T);
+                                    } else {
+                                        const uint32_t b[kS] = {v[h][0][e], v[h][1][e], v[h][2][e], v[h][3][e], v[h][4][e]};
+                                        const unsigned long long T = biased(b, g);
+                                        row_add_narrow(m, row_lo + j4, row_hi + j4, (uint32_t)T & ((1u << kLowBits) - 1u),
+                                                       __funnelshift_r((uint32_t)T, (uint32_t)(T >> 32), kLowBits));
+                                    }
+                                }
+                            }
+                    }
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&b_tempty[buf]));
                 }
+            }
+            if (!ok) break;
+            if (ROW) {
+                ok = epi_sync();   // every beta excitation of the row is in
+                for (int i = tid; i < nstr && ok; i += 32 * kBetaWarps) {
+                    const uint32_t lo = rlo[i], hi = rhi[i];
+                    rlo[i] = 0u;
+                    rhi[i] = 0u;
+                    unsigned long long v;
+                    if (WIDE) {
+                        v = (unsigned long long)hi << 32 | lo;
+                    } else {
+                        // less the bias of every term; |row sum| < 2^57, so its low 58 bits are enough
+                        v = ((unsigned long long)hi << kLowBits) + lo;
+                        v -= (unsigned long long)(p.kcnt ? p.kcnt[i] : p.nexc) * kBias;
+                        v = (unsigned long long)((long long)(v << (32 - kLowBits)) >> (32 - kLowBits));
+                    }
+                    red_add_if(v != 0, reinterpret_cast<unsigned long long *>(Srow) + i, v);
+                }
+                ok = epi_sync() && ok;   // the row is clear again
+            }
+        }
+    } else if (warp < kEpiWarps) {
+        // ---- alpha excitations of the item's string: some columns, the same for every lane
+        const int q = warp & 3;
+        const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        uint32_t *aofs = s_aofs[q];
+        uint16_t *acol = s_acol[q];
+        uint32_t tn = 0;
+        for (int it = blockIdx.x; it < nitem && ok; it += gridDim.x) {
+            const WorkItem item = items[it];
+            const SigmaProb &p = probs[item.prob];
+            if (p.active && !*p.active) continue;
+            const int nstr = p.nstr, npad = np_pad(p.act ? p.npc : p.np), ldj = p.ldj, ka = (int)item.start;
+            unsigned long long *Sp = reinterpret_cast<unsigned long long *>(S) + p.doff + (item.sub ? p.ndet : 0);
+            int na = 0;
+            for (int A0 = 0; A0 < npad; A0 += 32) {
+                const int A = A0 + lane;
+                const uint32_t m = A < npad ? p.jmap[((size_t)(A >> 2) * ldj + ka) * 4 + (A & 3)] : kNoMap;
+                const uint32_t bal = __ballot_sync(0xffffffffu, m != kNoMap);
+                if (m != kNoMap) {
+                    const int at = na + __popc(bal & ((1u << lane) - 1u));
+                    acol[at] = (uint16_t)A;
+                    aofs[at] = (m & 0x7FFFu) * (uint32_t)nstr | (m >> 15) << 31;
+                }
+                na += __popc(bal);
             }
             __syncwarp();
-        }
-        // the MMAs of the tile's last atom (every thread reaches this barrier: a
-        // failed vote above made all of them leave the atom loop together, and
-        // thread 0 alone may hold ok = false from its W wait)
-        if (!__syncthreads_and(tid == 0 ? (ok && mbar_wait(bm, ph_m)) : ok)) ok = false;
-        ph_m ^= 1;
-        if (!ok) break;
-        // read before the closing barrier: thread 0 overwrites s_next after it
-        const int t_next = s_next;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // ---- epilogue: the levels are exact integers below 2^24; combine them
-        // in int64, G = sum_L acc_L 2^{8 (4 - L)}  (no FP64 arithmetic)
-        long long *Gp = G + doff;
-        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        for (int c0 = 16 * (warp >> 2); c0 < Nt; c0 += 64) {
-            long long gi[16];
+            for (int mt = 0; mt * kTM < nstr && ok; mt++) {
+                const int ib0 = mt * kTM + q * 32, ib = ib0 + lane;
+                int i = 0;
+                for (int c0 = 0; c0 < npad; c0 += kNC, tn++) {
+                    const int w = min(kNC, npad - c0);
+                    const uint32_t buf = tn & 1, tcol = tmem + lane_base + buf * kTBuf - (uint32_t)c0;
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&b_tfull[buf]), (tn >> 1) & 1))) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    // four columns of the list at a time
+                    while (i < na && acol[i] < c0 + w) {
+                        uint32_t v[4][kS], of[4];
+                        int n = 0;
 #pragma unroll
-            for (int j = 0; j < 16; j++) gi[j] = 0;
+                        for (int u = 0; u < 4; u++) {
+                            const int k = min(i + u, na - 1);
+                            const uint32_t col = min((uint32_t)acol[k], (uint32_t)(c0 + w - 1));
+                            n += i + u < na && acol[k] < c0 + w;
+                            of[u] = aofs[k];
 #pragma unroll
-            for (int L = 0; L < kS; L++) {
-                float v[16];
-                tmem_ld16(tmem + lane_base + (uint32_t)(L * kNT + c0), v);
+                            for (int L = 0; L < kS; L++) v[u][L] = tmem_ld1(tcol + (uint32_t)(L * w) + col);
+                        }
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int j = 0; j < 16; j++) gi[j] += (long long)__float2int_rn(v[j]) << (8 * (kS - 1 - L));
-            }
-            if (live) {
+                        for (int u = 0; u < 4; u++) {
+                            const float sg = __uint_as_float(0x3F800000u | (of[u] & 0x80000000u));
+                            unsigned long long T;
+                            if (WIDE) {
+                                T = wide_sum(sg, v[u][0], v[u][1], v[u][2], v[u][3], v[u][4]);
+                            } else {
 #pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const int A = n0 + c0 + j;
-                    if (c0 + j < Nt && A < np) {
-                        long long *dst = Gp + (long long)(act ? act[A] : A) * gld + (K - k0);
-                        if (chunked) atomicAdd(reinterpret_cast<unsigned long long *>(dst), (unsigned long long)gi[j]);
-                        else *dst = gi[j];
+                                for (int L = 0; L < kS; L++)
+                                    v[u][L] = __float_as_uint(fmaf(sg, __uint_as_float(v[u][L]), 12582912.0f));
+                                T = biased(v[u], g) - kBias;
+                            }
+                            red_add_if(u < n && ib < nstr, Sp + (of[u] & 0x7FFFFFFFu) + ib, T);
+                        }
+                        i += n;
                     }
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&b_tempty[buf]));
                 }
             }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        t = t_next;
+    } else if (warp < kEpiWarps + kAWarps) {
+        // ---- digit tiles of c: K rows J_a, 128 determinants of each
+        const int t = tid - 32 * kEpiWarps;
+        uint32_t an = 0;
+        for (int it = blockIdx.x; it < nitem && ok; it += gridDim.x) {
+            const WorkItem item = items[it];
+            const SigmaProb &p = probs[item.prob];
+            if (p.active && !*p.active) continue;
+            const int nstr = p.nstr, ldq = row_ld(nstr);
+            const __half *src = Q + p.qoff + (item.sub ? (size_t)2 * kS * nstr * ldq : 0);
+            const int kc = build_list<32 * kAWarps, true>(p, (int)item.start, t, 1, lstA, mskA), Kp = round_up(kc, 16);
+            const int ch = t & 15;
+            for (int mt = 0; mt * kTM < nstr; mt++, an++) {
+                const uint32_t slot = an % g.nA;
+                if (t == 0) okA[an & 1] = mbar_wait(smem_u32(&b_emptyA[slot]), ((an / g.nA) & 1) ^ 1);
+                named_sync(1, 32 * kAWarps);
+                if (!okA[an & 1]) { ok = false; break; }
+                const uint32_t dst = smem_u32(Asm) + slot * stageA + (ch >> 3) * (uint32_t)Kp * 128;
+                const int col = mt * kTM + ch * 8;
+                for (int j = 0; j < kS; j++)
+                    for (int k = t >> 4; k < Kp; k += 2 * kAWarps) {
+                        const bool lv = k < kc && col < nstr;
+                        const __half *s = lv ? src + ((size_t)lstA[k] + (size_t)j * nstr) * ldq + col : Q;
+                        cp_async16(dst + (uint32_t)(j * Kp * 256 + k * 128 + (((ch & 7) ^ (k & 7)) << 4)), s, lv);
+                    }
+                if (t == 0) kp_of[slot] = Kp;
+                cp_async_done();
+                mbar_arrive(smem_u32(&b_fullA[slot]));
+            }
+        }
+        cp_async_done();
+    } else if (warp < kEpiWarps + kAWarps + kWWarps) {
+        // ---- W chunks: K rows = contracted pairs, 5 slices x w output pairs of each
+        const int t = tid - 32 * (kEpiWarps + kAWarps), wi = t >> 5;
+        uint32_t wn = 0;
+        for (int it = blockIdx.x; it < nitem && ok; it += gridDim.x) {
+            const WorkItem item = items[it];
+            const SigmaProb &p = probs[item.prob];
+            if (p.active && !*p.active) continue;
+            const int nstr = p.nstr, npc = p.act ? p.npc : p.np, npad = np_pad(npc), nch = (npad + kNC - 1) / kNC;
+            const uint8_t *img = (const uint8_t *)p.Woz;
+            const int kc = build_list<32 * kWWarps, false>(p, (int)item.start, t, 2, lstW, mskW), Kp = round_up(kc, 16);
+            const int reps = nch <= g.nW ? 1 : (nstr + kTM - 1) / kTM;   // resident chunks are loaded once per item
+            for (int r = 0; r < reps && ok; r++)
+                for (int c0 = 0; c0 < npad; c0 += kNC, wn++) {
+                    const int w = min(kNC, npad - c0);
+                    const uint32_t slot = wn % g.nW;
+                    if (t == 0) okW[wn & 1] = mbar_wait(smem_u32(&b_emptyW[slot]), ((wn / g.nW) & 1) ^ 1);
+                    named_sync(2, 32 * kWWarps);
+                    if (!okW[wn & 1]) { ok = false; break; }
+                    const uint8_t *cimg = img + (size_t)npc * 10 * c0;
+                    const int n8 = lane;                       // 16-byte chunk of a row (5 w / 8 <= 30 of them)
+                    const uint32_t dst = smem_u32(Wsm) + slot * stageW + (uint32_t)(n8 >> 3) * Kp * 128;
+                    if (n8 < kS * w / 8)
+                        for (int k = wi; k < Kp; k += kWWarps) {
+                            const bool lv = k < kc;
+                            const uint8_t *s = lv ? cimg + (size_t)lstW[k] * 10 * w + n8 * 16 : img;
+                            cp_async16(dst + (uint32_t)(k * 128 + (((n8 & 7) ^ (k & 7)) << 4)), s, lv);
+                        }
+                    cp_async_done();
+                    mbar_arrive(smem_u32(&b_fullW[slot]));
+                }
+        }
+        cp_async_done();
+    } else {
+        // ---- the MMAs: the warp runs the loop together, one elected lane issues
+        const bool lead = elect_one();
+        const uint32_t idesc0 = idesc_f16_mn(kTM, 0);
+        uint32_t an = 0, wn = 0, tn = 0;
+        for (int it = blockIdx.x; it < nitem && ok; it += gridDim.x) {
+            const WorkItem item = items[it];
+            const SigmaProb &p = probs[item.prob];
+            if (p.active && !*p.active) continue;
+            const int nstr = p.nstr, npad = np_pad(p.act ? p.npc : p.np), nch = (npad + kNC - 1) / kNC;
+            const int nmt = (nstr + kTM - 1) / kTM;
+            const bool res = nch <= g.nW;
+            const uint32_t w0 = wn;
+            for (int mt = 0; mt < nmt && ok; mt++, an++) {
+                const uint32_t sa = an % g.nA;
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&b_fullA[sa]), (an / g.nA) & 1));
+                if (!ok) break;
+                const int Kp = __shfl_sync(0xffffffffu, kp_of[sa], 0), ns = Kp / 16;
+                const uint32_t lbo = (uint32_t)Kp * 128;
+                const uint64_t ad0 = smem_desc_mn(smem_u32(Asm) + sa * stageA, lbo);
+                for (int c = 0; c < nch; c++, tn++) {
+                    const int w = min(kNC, npad - c * kNC);
+                    uint32_t sw = (w0 + c) % g.nW;
+                    if (!res || mt == 0) {
+                        sw = wn % g.nW;
+                        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&b_fullW[sw]), (wn / g.nW) & 1));
+                        if (!ok) break;
+                        wn++;
+                    }
+                    const uint32_t tb = tn & 1;
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&b_tempty[tb]), ((tn >> 1) & 1) ^ 1));
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    if (lead) {
+                        const uint64_t wd = smem_desc_mn(smem_u32(Wsm) + sw * stageW, lbo);
+#pragma unroll
+                        for (int j = 0; j < kS; j++) {
+                            const uint32_t idesc = idesc0 | (uint32_t)((kS - j) * w >> 3) << 17;
+                            const uint32_t td = tmem + tb * kTBuf + (uint32_t)(j * w);
+                            const uint64_t aj = ad0 + (uint64_t)(j * Kp * 16);
+                            mma_f16(td, aj, wd, idesc, j > 0 ? 1u : 0u);
+                            for (int s = 1; s < ns; s++)
+                                mma_f16(td, aj + (uint64_t)(s * 128), wd + (uint64_t)(s * 128), idesc, 1u);
+                        }
+                        mma_commit(smem_u32(&b_tfull[tb]));
+                        if (!res || mt + 1 == nmt) mma_commit(smem_u32(&b_emptyW[sw]));
+                        if (c + 1 == nch) mma_commit(smem_u32(&b_emptyA[sa]));
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        if (!ok) {   // MMAs may still be in flight: wait for them (bounded) before the buffers go
+            if (lead) mma_commit(smem_u32(&b_drain));
+            __syncwarp();
+            mbar_wait(smem_u32(&b_drain), 0);
+        }
     }
-    if (!ok && tid == 0) atomicExch(err, 1);
-    // a prefetch may still be in flight after a timeout: wait for it (bounded)
-    if (!ok) __syncthreads_and(mbar_wait((g & 1) ? bw1 : bw0, (g >> 1) & 1));
+    __syncwarp();
+    if (!ok && lane == 0) atomicExch(err, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
@@ -301,53 +646,176 @@ oz_contract_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restri
                      : "memory");
 }
 
-// Sliced image of W: [tile nt][atom a][slice i][kNT rows][128 B], W scaled by
-// 2^-e with one exponent per problem (max |W| <= 2^e, stored in Wexp[0]), the
-// 16-byte chunk c of a row at c ^ (row % 8), zeros beyond npair.
-__global__ void oz_pack_w_kernel(const SigmaProb *__restrict__ probs) {
+// Digit planes of a problem's input vector: plane (sign s, digit j) of pass t
+// at [(t 2 + s) kS + j][nstr][row_ld] holds digit j (0 = most significant) of
+// +-round(c 2^38 / dscale); pass 1 (only without spin-flip symmetry) is C^T.
+// Clears the problem's S as well.
+__global__ void __launch_bounds__(kGatherChunk)
+oz_quantise_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items, __half *__restrict__ Q,
+                   long long *__restrict__ S) {
+    const WorkItem it = items[blockIdx.x];
+    const SigmaProb &p = probs[it.prob];
+    if (p.active && !*p.active) return;
+    const long long I = it.start + threadIdx.x;
+    if (I >= p.ndet) return;
+    const int nstr = p.nstr, ldq = row_ld(nstr);
+    const int ka = (int)(I / nstr), kb = (int)(I % nstr);
+    const double *c = p.cbase + (p.cslot ? (long long)*p.cslot : 0ll) * p.stride;
+    const double sc = 274877906944.0 / p.dscale;   // 2^38 / dscale
+    const size_t plane = (size_t)nstr * ldq;
+    unsigned short *out = reinterpret_cast<unsigned short *>(Q) + p.qoff + (size_t)ka * ldq + kb;
+    for (int t = 0; t < (p.sym ? 1 : 2); t++) {
+        const long long x = __double2ll_rn((t ? c[(long long)kb * nstr + ka] : c[I]) * sc);
+        const unsigned long long u = (unsigned long long)(x + kDigitBias), v = (unsigned long long)(-x + kDigitBias);
+#pragma unroll
+        for (int j = 0; j < kS; j++) {
+            const uint32_t h = j == 0 ? digit_pair_f16((uint32_t)(u >> 32), (uint32_t)(v >> 32), 0)
+                                      : digit_pair_f16((uint32_t)u, (uint32_t)v, kS - 1 - j);
+            out[(size_t)j * plane] = (unsigned short)(h & 0xFFFF);
+            out[(size_t)(kS + j) * plane] = (unsigned short)(h >> 16);
+        }
+        out += 2 * kS * plane;
+        S[p.doff + (t ? p.ndet : 0) + I] = 0;
+    }
+}
+
+// sigma = S + S^T (spin-flip-symmetric) or S(C) + S(C^T)^T, converted from the
+// integer units; one 32 x 32 tile of strings and its transpose per block.
+__global__ void __launch_bounds__(256)
+oz_finish_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items, const long long *__restrict__ S) {
+    const WorkItem it = items[blockIdx.x];
+    const SigmaProb &p = probs[it.prob];
+    if (p.active && !*p.active) return;
+    __shared__ double sh[2][32][33];
+    const int n = p.nstr, r0 = (int)it.start * 32, c0 = it.sub * 32, x = threadIdx.x & 31, y0 = threadIdx.x >> 5;
+    const double f = p.Wexp[0] * p.dscale * 0x1p-45;
+    const long long *S1 = S + p.doff, *S2 = p.sym ? S1 : S1 + p.ndet;
+    double *s = p.sbase + (p.sslot ? (long long)*p.sslot : 0ll) * p.stride;
+    for (int y = y0; y < 32; y += 8) {
+        const int r = r0 + y, c = c0 + y;   // rows of the tile and of its transpose
+        sh[0][y][x] = c < n && r0 + x < n ? (double)S2[(long long)c * n + r0 + x] * f : 0.0;
+        sh[1][y][x] = !p.sym && r < n && c0 + x < n ? (double)S2[(long long)r * n + c0 + x] * f : 0.0;
+    }
+    __syncthreads();
+    double v[4], u[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int y = y0 + 8 * k, r = r0 + y, c = c0 + y;
+        v[k] = r < n && c0 + x < n ? (double)S1[(long long)r * n + c0 + x] * f + sh[0][x][y] : 0.0;
+        u[k] = !p.sym && c < n && r0 + x < n ? (double)S1[(long long)c * n + r0 + x] * f + sh[1][x][y] : 0.0;
+    }
+    __syncthreads();
+    if (p.sym)
+#pragma unroll
+        for (int k = 0; k < 4; k++) sh[0][y0 + 8 * k][x] = v[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int y = y0 + 8 * k, r = r0 + y, c = c0 + y;
+        if (r < n && c0 + x < n) s[(long long)r * n + c0 + x] = v[k];
+        if (c < n && r0 + x < n) s[(long long)c * n + r0 + x] = p.sym ? sh[0][x][y] : u[k];
+    }
+}
+
+// one exponent per problem: max |W| over the contracted pairs <= 2^e (Wexp[0])
+__global__ void __launch_bounds__(512) oz_wmax_kernel(const SigmaProb *__restrict__ probs) {
     const SigmaProb &p = probs[blockIdx.x];
-    // a sectored space packs only its active pairs, in compact order
-    const int np = p.act ? p.npc : p.np, KA = k_atoms(np), NTl = n_tiles(np);
+    const int np = p.act ? p.npc : p.np, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t *act = p.act;
+    __shared__ double red[16];
+    double mx = 0.0;
+    for (int r = warp; r < np; r += 16)
+        for (int c = lane; c < np; c += 32)
+            mx = fmax(mx, fabs(p.W[(act ? act[r] : r) * (long long)p.ld + (act ? act[c] : c)]));
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red[warp] = mx;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 16; w++) mx = fmax(mx, red[w]);
+        int e = 0;
+        if (mx > 0.0) frexp(mx, &e);          // max = f 2^e, f in [0.5, 1)
+        p.Wexp[0] = ldexp(1.0, e);
+    }
+}
+
+// Sliced image of W, MN-major: for each chunk of w = 48 output pairs (the last
+// one narrower, a multiple of 16) [contracted pair b][slice i][output pair of
+// the chunk] FP16, zeros beyond npair.  A sectored space packs its active
+// pairs only, in compact order.  Blocks (problem, part).
+__global__ void __launch_bounds__(256) oz_pack_w_kernel(const SigmaProb *__restrict__ probs) {
+    const SigmaProb &p = probs[blockIdx.x];
+    const int np = p.act ? p.npc : p.np, npad = np_pad(np), n8 = npad / 8;
     const int32_t *act = p.act;
     uint8_t *img = (uint8_t *)const_cast<void *>(p.Woz);
-    __shared__ double red[256];
-    double mx = 0.0;
-    for (long long i = threadIdx.x; i < (long long)np * np; i += blockDim.x) {
-        const long long r = i / np, c = i % np;
-        mx = fmax(mx, fabs(p.W[(act ? act[r] : r) * (long long)p.ld + (act ? act[c] : c)]));
-    }
-    red[threadIdx.x] = mx;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + o]);
-        __syncthreads();
-    }
-    int e = 0;
-    if (red[0] > 0.0) frexp(red[0], &e);          // max = f 2^e, f in [0.5, 1)
-    const double scale = ldexp(1.0, e);
-    if (threadIdx.x == 0) p.Wexp[0] = scale;
-    const int rows = NTl * kNT;
-    for (int t = threadIdx.x; t < rows * KA * 8; t += blockDim.x) {
-        const int n = t / (KA * 8), rest = t % (KA * 8), a = rest / 8, ch = rest % 8;
-        const int nt = n / kNT, r = n % kNT;
+    const double scale = p.Wexp[0];
+    for (int t = blockIdx.y * 256 + threadIdx.x; t < np * n8; t += gridDim.y * 256) {
+        const int b = t / n8, a0 = t % n8 * 8, c0 = a0 / kNC * kNC, w = min(kNC, npad - c0);
+        const int kb = act ? act[b] : b;
         float sl[8][kS];
-        for (int e2 = 0; e2 < 8; e2++) {
-            const int k = a * 64 + ch * 8 + e2;
-            double x = (n < np && k < np) ? p.W[(long long)(act ? act[n] : n) * p.ld + (act ? act[k] : k)] / scale
-                                          : 0.0;
-            slice5(x, sl[e2]);
+        for (int e = 0; e < 8; e++) {
+            const int a = a0 + e;
+            slice5(a < np ? p.W[(long long)(act ? act[a] : a) * p.ld + kb] / scale : 0.0, sl[e]);
         }
-        for (int i = 0; i < kS; i++) {
-            uint4 qv = make_uint4(pack2(sl[0][i], sl[1][i]), pack2(sl[2][i], sl[3][i]), pack2(sl[4][i], sl[5][i]),
-                                  pack2(sl[6][i], sl[7][i]));
-            size_t off = (((size_t)nt * KA + a) * kS + i) * (kNT * kAtomBytes) + (size_t)r * kAtomBytes +
-                         ((ch ^ (r & 7)) << 4);
-            *(uint4 *)(img + off) = qv;
+        for (int i = 0; i < kS; i++)
+            *(uint4 *)(img + (size_t)np * 10 * c0 + ((size_t)b * kS * w + i * w + (a0 - c0)) * 2) =
+                make_uint4(pack2(sl[0][i], sl[1][i]), pack2(sl[2][i], sl[3][i]), pack2(sl[4][i], sl[5][i]),
+                           pack2(sl[6][i], sl[7][i]));
+    }
+}
+
+// Excitation map of a string class: entry of output pair A and string I at
+// [A / 4][I][A % 4] (one 8-byte load per thread and four columns), sign << 15 | J
+// of E+_A |I> = +-|J>, kNoMap where there is none, beyond np and beyond nstr
+// (ldj strings, np_pad(np) pairs).
+__global__ void __launch_bounds__(128) oz_map_kernel(int nstr, int nexc, int np, int ldj, const int32_t *__restrict__ exc,
+                                                     uint16_t *__restrict__ jmap) {
+    // one thread per string: its list is sorted by pair
+    const int I = blockIdx.x * 128 + threadIdx.x;
+    if (I >= ldj) return;
+    const int32_t *row = exc + (size_t)I * nexc;
+    int e = 0;
+    int32_t x = I < nstr ? row[0] : -1;
+    for (int A0 = 0; A0 < np_pad(np); A0 += 4) {
+        uint32_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            v[u] = kNoMap;
+            if (I < nstr && e < nexc && exc_pair(x) == A0 + u) {
+                v[u] = (uint32_t)exc_J(x) | (uint32_t)(x & 1) << 15;
+                if (++e < nexc) x = row[e];
+            }
+        }
+        reinterpret_cast<uint2 *>(jmap)[(size_t)(A0 >> 2) * ldj + I] = make_uint2(v[0] | v[1] << 16, v[2] | v[3] << 16);
+    }
+}
+
+// maps of the sectored units: their class's map restricted to the active pairs
+__global__ void __launch_bounds__(256) oz_compact_maps_kernel(const OzMapDesc *__restrict__ desc, int n) {
+    for (int u = blockIdx.x; u < n; u += gridDim.x) {
+        const OzMapDesc d = desc[u];
+        for (int t = threadIdx.x; t < np_pad(d.npc) / 4 * d.ldj; t += 256) {
+            const int g = t / d.ldj, I = t % d.ldj;
+            uint32_t v[4];
+            for (int k = 0; k < 4; k++) {
+                const int A = 4 * g + k < d.npc ? d.act[4 * g + k] : -1;
+                v[k] = A >= 0 ? d.map[((size_t)(A >> 2) * d.ldj + I) * 4 + (A & 3)] : kNoMap;
+            }
+            reinterpret_cast<uint2 *>(d.out)[t] = make_uint2(v[0] | v[1] << 16, v[2] | v[3] << 16);
+        }
+        // contracted pairs of each string
+        for (int I = threadIdx.x; I < d.nstr; I += 256) {
+            int k = 0;
+            for (int c = 0; c < d.npc; c++)
+                k += d.map[((size_t)(d.act[c] >> 2) * d.ldj + I) * 4 + (d.act[c] & 3)] != kNoMap;
+            d.kcnt[I] = (uint8_t)k;
         }
     }
 }
 
-// dscale = smallest power of two >= 2 max|c| (|D| <= 2 max|c|)
+// dscale of a caller's vector: the smallest power of two >= 2 max|c| with
+// spin-flip symmetry, >= max|c| without (two passes, each with its own
+// rounding: half the scale keeps their sum below the error of one pass over
+// alpha and beta sums; the top digit stays below 65)
 __global__ void oz_absmax_kernel(const double *__restrict__ c, long long n, unsigned long long *__restrict__ out) {
     double m = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -359,21 +827,64 @@ __global__ void oz_absmax_kernel(const double *__restrict__ c, long long n, unsi
 __global__ void oz_set_dscale_kernel(SigmaProb *__restrict__ p, const unsigned long long *__restrict__ mx) {
     double m = __longlong_as_double((long long)*mx);
     int e = 0;
-    if (m > 0.0) frexp(2.0 * m, &e);
+    if (m > 0.0) frexp((p->sym ? 2.0 : 1.0) * m, &e);
     p->dscale = m > 0.0 ? ldexp(1.0, e) : 1.0;
+}
+
+int contracted_pairs(const SigmaProb &p) { return p.act ? p.npc : p.np; }
+
+// Buffers for items of at most k contracted pairs per string, nch chunks and
+// nstr strings: the accumulator row in shared memory if anything can be had
+// with it (its atomics are ~5 times cheaper there than in L2), then two c
+// stages before more than two W buffers, then as many W buffers as there are
+// chunks (resident for the whole item).
+bool choose_geom(int k, int nch, int nstr, OzGeom &g) {
+    g.kmax = round_up(k, 16);
+    if (g.kmax > kMaxK) return false;
+    const int sa = kS * g.kmax * 256, sw = g.kmax * 512;
+    for (int row = 1; row >= 0; row--)
+        for (int nA = 2; nA >= 1; nA--)
+            for (int nW = std::min(kMaxW, std::max(nch, 2)); nW >= (row || nA > 1 ? 2 : 1); nW--)
+                if (nA * sa + nW * sw + row * 8 * nstr <= kSmemLimit) {
+                    g.nA = nA;
+                    g.nW = nW;
+                    g.rows = row * nstr;
+                    return true;
+                }
+    return false;
 }
 
 }  // namespace
 
-int oz_tile_n() { return kNT; }
+int oz_operand_bytes(int np) { return np * np_pad(np) * 2 * kS + 256; }
+int oz_map_ld(int nstr) { return round_up(nstr, kTM); }
+size_t oz_map_elems(int np, int nstr) { return (size_t)np_pad(np) * oz_map_ld(nstr); }
+long long oz_plane_elems(int nstr, bool sym) { return (sym ? 2ll : 4ll) * kS * nstr * row_ld(nstr); }
+bool oz_supported(int np, int nstr, int nexc) { return np <= kMaxNp && nstr <= kMaxStrings && nexc <= kMaxK; }
+bool oz_wide(int nexc) { return nexc > kNarrowK; }
 
-int oz_operand_bytes(int np) {
-    return (int)((size_t)n_tiles(np) * k_atoms(np) * kWStage + (size_t)np * 8 + 256);
+int launch_oz_map(ifci_handle_t h, int nstr, int nexc, int np, const int32_t *exc, uint16_t *jmap, cudaStream_t s) {
+    const int ldj = oz_map_ld(nstr);
+    oz_map_kernel<<<ldj / 128, 128, 0, s>>>(nstr, nexc, np, ldj, exc, jmap);
+    IFCI_LAUNCH_CHECK(h);
+    return IFCI_OK;
 }
 
-int launch_oz_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, cudaStream_t s) {
+int launch_oz_compact_maps(ifci_handle_t h, int n, const OzMapDesc *d_desc, cudaStream_t s) {
+    if (n <= 0) return IFCI_OK;
+    oz_compact_maps_kernel<<<stride_grid(h->device, n, 8), 256, 0, s>>>(d_desc, n);
+    IFCI_LAUNCH_CHECK(h);
+    return IFCI_OK;
+}
+
+int launch_oz_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, int max_np, cudaStream_t s) {
     if (nprob <= 0) return IFCI_OK;
-    oz_pack_w_kernel<<<nprob, 256, 0, s>>>(d_probs);
+    oz_wmax_kernel<<<nprob, 512, 0, s>>>(d_probs);
+    IFCI_LAUNCH_CHECK(h);
+    // one 8-pair group per thread while there are few problems
+    const int parts = (max_np * np_pad(max_np) / 8 + 255) / 256;
+    const int room = std::max(1, 16 * device_sm_count(h->device) / nprob);
+    oz_pack_w_kernel<<<dim3(nprob, std::max(1, std::min(parts, room))), 256, 0, s>>>(d_probs);
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;
 }
@@ -390,29 +901,47 @@ int launch_oz_dscale(ifci_handle_t h, SigmaProb *d_prob, const double *c, long l
     return IFCI_OK;
 }
 
-int launch_oz_contract(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, const void *Q, void *G,
-                       cudaStream_t s) {
-    if (w.ntc == 0) return IFCI_OK;
-    for (const SigmaProb &p : plan.probs)
-        if (p.np > kMaxNpTable)
-            return set_error(h, IFCI_ERR_UNSUPPORTED, "FP64E: npair %d > %d", p.np, kMaxNpTable);
-    // K chunks add their partial sums: zero those problems' G first
-    for (int i = w.prob0; i < w.prob0 + w.nprob; i++) {
-        const SigmaProb &p = plan.probs[i];
-        if (k_atoms(p.act ? p.npc : p.np) > kChunkAtoms)
-            IFCI_CUDA_TRY(h, cudaMemsetAsync(static_cast<long long *>(G) + p.doff, 0,
-                                             (size_t)p.np * (w.kn ? w.kn : p.ndet) * 8, s));
+int run_sigma_oz(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, void *D, void *G, cudaStream_t s) {
+    if (!h->d_err) return set_error(h, IFCI_ERR_INVALID_ARG, "FP64E: no error flag");
+    auto *Q = static_cast<__half *>(D);
+    auto *S = static_cast<long long *>(G);
+    {
+        ProfScope ps(h, s, PK_GATHER);
+        oz_quantise_kernel<<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0, Q, S);
+        IFCI_LAUNCH_CHECK(h);
     }
-    if (!h->d_err || !h->d_counter) return set_error(h, IFCI_ERR_INVALID_ARG, "FP64E: no error flag / counter");
-    const size_t smem = 1024 + 2 * kWStage + kAStage;   // 205,824 B
-    static SmemOptIn opt;
-    IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, oz_contract_kernel, (int)smem));
-    const int grid = std::min(w.ntc, device_sm_count(h->device));
-    IFCI_CUDA_TRY(h, cudaMemsetAsync(h->d_counter, 0, sizeof(int), s));
-    ProfScope ps(h, s, PK_CONTRACT_HI);
-    oz_contract_kernel<<<grid, kThreads, smem, s>>>(plan.d_probs, plan.d_tctiles + w.tc0, w.ntc,
-                                                    (const long long *)Q, (long long *)G, h->d_err, h->d_counter,
-                                                    w.k0, w.kn);
+    static SmemOptIn opt_n, opt_w, opt_g;
+    for (int wide = 0; wide < 2; wide++) {
+        const int i0 = wide ? w.tc0 + w.ntc : w.tc0, ni = wide ? w.nwide : w.ntc;
+        if (ni == 0) continue;
+        int k = 0, nch = 0, nstr = 0;
+        for (int i = w.prob0; i < w.prob0 + w.nprob; i++) {
+            const SigmaProb &p = plan.probs[i];
+            if (oz_wide(p.nexc) != (wide != 0)) continue;
+            k = std::max(k, std::min(p.nexc, contracted_pairs(p)));
+            nch = std::max(nch, (np_pad(contracted_pairs(p)) + kNC - 1) / kNC);
+            nstr = std::max(nstr, p.nstr);
+        }
+        OzGeom g{};
+        g.m8 = 1u << 8;
+        g.m16 = 1u << 16;
+        g.m24 = 1u << 24;
+        if (!choose_geom(k, nch, nstr, g) || (!wide && !g.rows)) return set_error(h, IFCI_ERR_UNSUPPORTED, "FP64E: %d excitations per string", k);
+        const size_t smem = 1024 + (size_t)g.nA * kS * g.kmax * 256 + (size_t)g.nW * g.kmax * 512 + (size_t)g.rows * 8;
+        const int grid = std::min(ni, device_sm_count(h->device));
+        ProfScope ps(h, s, PK_CONTRACT_HI);
+        auto launch = [&](auto kernel, SmemOptIn &opt) {
+            const cudaError_t e = ensure_smem(opt, h->device, kernel, (int)smem);
+            if (e == cudaSuccess)
+                kernel<<<grid, kOzThreads, smem, s>>>(plan.d_probs, plan.d_tctiles + i0, ni, Q, S, h->d_err, g);
+            return e;
+        };
+        IFCI_CUDA_TRY(h, !wide ? launch(oz_sigma_kernel<false, true>, opt_n)
+                         : g.rows ? launch(oz_sigma_kernel<true, true>, opt_w) : launch(oz_sigma_kernel<true, false>, opt_g));
+        IFCI_LAUNCH_CHECK(h);
+    }
+    ProfScope ps(h, s, PK_SCATTER);
+    oz_finish_kernel<<<w.nfin, 256, 0, s>>>(plan.d_probs, plan.d_tiles + w.tile0, S);
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;
 }

@@ -51,17 +51,19 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 
-// Bounded wait on an mbarrier phase; false on timeout.
+// Bounded wait on an mbarrier phase; false on timeout.  The hint lets the
+// hardware suspend the thread for up to 2 us per attempt instead of having it
+// spin in the issue slots of the warps that work.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     long long t0 = clock64();
     while (true) {
         uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(done)
-            : "r"(bar), "r"(parity)
+            : "r"(bar), "r"(parity), "r"(2000u)
             : "memory");
         if (done) return true;
         if (clock64() - t0 > kWaitCycles) return false;
