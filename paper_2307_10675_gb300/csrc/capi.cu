@@ -35,6 +35,20 @@ int ifci_sigma(ifci_handle_t h, const ifci_strings_t *str, const double *h1, con
     const int n = str->norb, np = n * (n + 1) / 2, ld = np;
     const long long ndet = (long long)nstr * nstr;
 
+    if (precision == IFCI_FP64) {
+        // string Hamiltonian, then one fused kernel; descriptors by value
+        const int nnz = string_h_nnz(n, str->nelec_spin);
+        IFCI_TRY(ws_reserve(h, ws_round((size_t)nnz * nstr * 8) + ws_round((size_t)nnz * nstr * 4)));
+        double *hval = ws_take<double>(h, (size_t)nnz * nstr);
+        int *hidx = ws_take<int>(h, (size_t)nnz * nstr);
+        SigmaProb q{};
+        q.n = n; q.nstr = nstr; q.nexc = nexc; q.np = np;
+        q.ndet = ndet; q.stride = ndet; q.exc = str->exc; q.eri = eri;
+        q.hval = hval; q.hidx = hidx; q.nnz = nnz;
+        q.cbase = c; q.sbase = sigma;
+        IFCI_TRY(launch_string_h(h, StringHDesc{n, str->nelec_spin, nstr, nnz, h1, eri, hval, hidx}, s));
+        return run_sigma64_one(h, q, s);
+    }
     SigmaPlan plan;
     SigmaProb p{};
     p.n = n; p.nstr = nstr; p.nexc = nexc; p.np = np; p.ld = ld;

@@ -159,6 +159,33 @@ inline cudaError_t ensure_smem(SmemOptIn &opt, int device, K kernel, int bytes) 
     if (e == cudaSuccess) opt.bytes[device] = bytes;
     return e;
 }
+// string <-> rank (combinatorial number system: rank(I) = sum_k C(p_k, k + 1)
+// over the occupied orbitals p_0 < p_1 < ...)
+struct StringBinom {
+    int c[32][32];
+};
+StringBinom string_binom();
+__device__ __forceinline__ int string_rank_of(uint32_t mask, const StringBinom &B) {
+    int r = 0, k = 1;
+    while (mask) {
+        int p = __ffs(mask) - 1;
+        r += B.c[p][k];
+        k++;
+        mask &= mask - 1;
+    }
+    return r;
+}
+__device__ __forceinline__ uint32_t string_of_rank(int rank, int n, int m, const StringBinom &B) {
+    uint32_t mask = 0;
+    int rem = rank;
+    for (int k = m; k >= 1; k--) {
+        int p = k - 1;
+        while (p + 1 < n && B.c[p + 1][k] <= rem) p++;
+        rem -= B.c[p][k];
+        mask |= 1u << p;
+    }
+    return mask;
+}
 int launch_exc_blocks(ifci_handle_t h, int nstr, int nexc, const int32_t *exc, uint8_t *blk, cudaStream_t s);
 // row stride (int32 entries) of the dense pair map
 __host__ __device__ inline int pmap_ld(int np) { return (np + 15) / 16 * 16; }

@@ -124,7 +124,7 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         sp.n = p.n; sp.nstr = nstr; sp.nexc = nexc; sp.np = np; sp.ld = np;
         sp.ndet = ndet; sp.stride = ndet;
         sp.sym = ((tc || oz) && 2ll * nstr * nstr < (1ll << 31)) ? 1 : 0;   // plan_sigma keeps it for tensor cores
-        if (lo || !oz) max_pd = std::max(max_pd, sigma_elems(np, ndet));   // D and G of a problem stay whole there
+        if (lo) max_pd = std::max(max_pd, sigma_elems(np, ndet));   // D and G of a problem stay whole there
         sum_pd += sigma_elems(np, ndet);
         sp.dscale = 2.0;   // basis vectors are normalised: |D| <= 2
         hi.probs.push_back(sp);
@@ -159,6 +159,13 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
     IFCI_TRY(plan_sigma(h, hi, budget, hi_prec));
     if (lo) IFCI_TRY(plan_sigma(h, lop, budget * 8 / (long long)sigma_elem_bytes(o.precision), o.precision));
 
+    // plain FP64: string Hamiltonians, their lists built in chunks of strings
+    const bool f64 = hi_prec == IFCI_FP64;
+    std::vector<WorkItem> hitems;
+    if (f64)
+        for (int u = 0; u < nu; u++)
+            for (int i0 = 0; i0 < hi.probs[u].nstr; i0 += kStringHChunk) hitems.push_back(WorkItem{u, 0, i0});
+
     // ---- device memory, counted then taken in the same order
     struct Mem {
         std::vector<uint64_t *> st;
@@ -171,6 +178,10 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         std::vector<char *> Woz;
         std::vector<double *> hd, B, S, cblk;
         std::vector<uint16_t *> jm, jmc;
+        std::vector<double *> hval;
+        std::vector<int *> hidx;
+        StringHDesc *hdesc = nullptr;
+        WorkItem *hitems = nullptr;
         OzMapDesc *mdesc = nullptr;
         std::vector<uint8_t *> kcnt;
         int32_t *act_all = nullptr;
@@ -197,6 +208,7 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
     auto carve = [&](Carver &c, Mem &m) {
         const int nc = (int)cls_keys.size();
         m.st.resize(nc); m.ex.resize(nc); m.bl.assign(nc, nullptr); m.pm.assign(nc, nullptr); m.jm.assign(nc, nullptr);
+        m.hidx.assign(nc, nullptr);
         for (int k = 0; k < nc; k++) {
             const int nn = cls_keys[k].first, mm = cls_keys[k].second;
             const int nstr = (int)binom(nn, mm), nexc = mm * (nn - mm + 1), np = nn * (nn + 1) / 2;
@@ -207,6 +219,7 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
             if (tc) m.bl[k] = c.take<uint8_t>((size_t)nstr * kBlk16Stride);
             if (tc && 2ll * nstr * nstr < (1ll << 31)) m.pm[k] = c.take<int32_t>((size_t)nstr * pmap_ld(np));
             if (oz) m.jm[k] = c.take<uint16_t>(oz_map_elems(np, nstr));
+            if (f64) m.hidx[k] = c.take<int>((size_t)string_h_nnz(nn, mm) * nstr);
         }
         // active pairs of every sectored unit in one array each (one copy for all units)
         m.act_all = c.take<int32_t>(act_off.back());
@@ -219,13 +232,18 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         m.kcnt.assign(nu, nullptr);
         for (int u = 0; u < nu; u++)
             if (!act[u].empty()) m.kcnt[u] = c.take<uint8_t>((size_t)binom(units[u].spec.n, units[u].spec.m));
+        m.hval.assign(nu, nullptr);
+        for (int u = 0; u < nu && f64; u++)
+            m.hval[u] = c.take<double>((size_t)string_h_nnz(units[u].spec.n, units[u].spec.m) * binom(units[u].spec.n, units[u].spec.m));
+        m.hdesc = c.take<StringHDesc>(f64 ? nu : 1);
+        m.hitems = c.take<WorkItem>(hitems.size());
         m.W.resize(nu); m.Wf.assign(nu, nullptr); m.Wtc.assign(nu, nullptr); m.Woz.assign(nu, nullptr);
         m.gc.assign(nu, nullptr); m.gs.assign(nu, nullptr);
         for (int u = 0; u < nu; u++) {
             const ProbSpec &p = units[u].spec;
             const int np = p.n * (p.n + 1) / 2;
             const long long ndet = binom(p.n, p.m) * binom(p.n, p.m);
-            m.W[u] = c.take<double>((size_t)np * np);
+            m.W[u] = c.take<double>(lo || oz ? (size_t)np * np : 1);
             if (lo) m.Wf[u] = c.take<float>((size_t)np * np);
             if (tc) m.Wtc[u] = c.take<char>(tc_operand_bytes(np, o.precision));
             if (oz) m.Woz[u] = c.take<char>(oz_operand_bytes(np));
@@ -266,7 +284,7 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         // D holds the gathered intermediate on the CUDA-core paths and the quantised
         // copies of c on the tensor-core ones, G the other intermediate or, on the
         // FP64-emulating path, the integer sigma
-        const long long whole = (oz && !lo) ? 1 : budget;
+        const long long whole = lo ? budget : 1;
         m.D = c.take<char>((size_t)std::max(whole, oz ? hi.max_qelems : 0ll) * 8);
         m.G = c.take<char>((size_t)std::max(whole, oz ? hi.max_delems : 0ll) * 8);
         m.hi_p = c.take<SigmaProb>(hi.probs.size());
@@ -320,6 +338,10 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         for (SigmaPlan *pl : {&hi, &lop}) {
             SigmaProb &sp = pl->probs[u];
             sp.exc = mem.ex[k];
+            sp.eri = U.eri;
+            sp.hval = mem.hval[u];
+            sp.hidx = mem.hidx[k];
+            sp.nnz = string_h_nnz(p.n, p.m);
             sp.blk = mem.bl[k];
             sp.pmap = mem.pm[k];
             sp.jmap = mem.jm[k];
@@ -412,6 +434,20 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
                                      cudaMemcpyHostToDevice, s));
     IFCI_CUDA_TRY(h, cudaMemsetAsync(b.d_gs, 0, (size_t)n * kMaxSpace * kMaxSpace * 8, s));
     IFCI_CUDA_TRY(h, cudaMemsetAsync(b.d_y, 0, (size_t)n * kYStride * 8, s));
+    if (f64) {
+        // one unit of each class writes the class's column list
+        std::vector<StringHDesc> hd(nu);
+        std::vector<char> done(cls_keys.size(), 0);
+        for (int u = 0; u < nu; u++) {
+            const ProbSpec &p = units[u].spec;
+            const int k = cls[{p.n, p.m}];
+            hd[u] = StringHDesc{p.n, p.m, hi.probs[u].nstr, hi.probs[u].nnz, units[u].h1, units[u].eri, mem.hval[u],
+                                done[k] ? nullptr : mem.hidx[k]};
+            done[k] = 1;
+        }
+        IFCI_CUDA_TRY(h, cudaMemcpyAsync(mem.hdesc, hd.data(), nu * sizeof(StringHDesc), cudaMemcpyHostToDevice, s));
+        IFCI_CUDA_TRY(h, cudaMemcpyAsync(mem.hitems, hitems.data(), hitems.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, s));
+    }
     if (act_off.back() > 0) {
         std::vector<int32_t> act_h;
         std::vector<int16_t> pinv_h;
@@ -433,7 +469,8 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         ProfScope ps(h, s, PK_SETUP);
         int maxnp = 0;
         for (const Unit &U : units) maxnp = std::max(maxnp, U.spec.n * (U.spec.n + 1) / 2);
-        IFCI_TRY(launch_fold(h, nu, mem.fold, maxnp, s));
+        if (lo || oz) IFCI_TRY(launch_fold(h, nu, mem.fold, maxnp, s));
+        if (f64) IFCI_TRY(launch_string_h_batch(h, mem.hdesc, mem.hitems, (int)hitems.size(), s));
         if (lo) IFCI_TRY(launch_convert_w(h, nu, lop.d_probs, s));
         if (tc) IFCI_TRY(launch_tc_pack_w(h, nu, lop.d_probs, o.precision, s));
         if (oz) IFCI_TRY(launch_oz_pack_w(h, nu, hi.d_probs, maxnp, s));

@@ -1,5 +1,7 @@
-// Sigma build sigma = H c for a batch of CI problems (Knowles–Handy-style
-// resolution of the identity over singly excited determinants):
+// Sigma build sigma = H c for a batch of CI problems: plans, and the FP32, BF16
+// and TF32 paths (Knowles–Handy-style resolution of the identity over singly
+// excited determinants; the FP64 gather, contraction and scatter serve the
+// allocation-free entry point only, see sigma64.cu for the FP64 path):
 //
 //   D[A][K] = <K| E+_A |c>          gather over K's own alpha and beta excitations
 //   G[A][K] = sum_B W[A][B] D[B][K]  dense contraction (W folds h1 into the ERIs)
@@ -233,6 +235,11 @@ int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision
             }
             continue;
         }
+        if (precision == IFCI_FP64) {   // no intermediates: one item per alpha string, one wave
+            w.nprob++;
+            w.nitem += p.nstr;
+            continue;
+        }
         long long need = sigma_elems(p.np, p.ndet);
         if (need > budget)
             return set_error(h, IFCI_ERR_OOM, "sigma: one problem needs %lld intermediate elements, budget %lld",
@@ -259,6 +266,15 @@ int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision
                     w.ntile++;
                 }
         }
+    }
+    if (precision == IFCI_FP64) {
+        // the problems with the longest items first (their blocks start first)
+        std::vector<int> order(plan.probs.size());
+        for (size_t i = 0; i < order.size(); i++) order[i] = (int)i;
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int x, int y) { return plan.probs[x].nstr > plan.probs[y].nstr; });
+        for (int i : order)
+            for (int ka = 0; ka < plan.probs[i].nstr; ka++) plan.items.push_back(WorkItem{i, 0, ka});
     }
     close_wave((int)plan.probs.size());
     if (precision == IFCI_FP64E) {
@@ -353,22 +369,7 @@ int run_sigma(ifci_handle_t h, const SigmaPlan &plan, int precision, void *D, vo
     for (const SigmaWave &w : plan.waves) {
         if (w.nitem == 0) continue;
         if (precision == IFCI_FP64) {
-            {
-                ProfScope ps(h, s, PK_GATHER);
-                gather_kernel<double><<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0,
-                                                                       (double *)D);
-                IFCI_LAUNCH_CHECK(h);
-            }
-            {
-                ProfScope ps(h, s, PK_CONTRACT);
-                contract_simt_kernel<double><<<w.ntile, 256, 0, s>>>(plan.d_probs, plan.d_tiles + w.tile0,
-                                                                     (const double *)D, (double *)G);
-                IFCI_LAUNCH_CHECK(h);
-            }
-            ProfScope ps(h, s, PK_SCATTER);
-            scatter_kernel<double><<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0,
-                                                                    (const double *)G);
-            IFCI_LAUNCH_CHECK(h);
+            IFCI_TRY(run_sigma64(h, plan, w, s));
         } else if (precision == IFCI_FP32) {
             {
                 ProfScope ps(h, s, PK_GATHER);

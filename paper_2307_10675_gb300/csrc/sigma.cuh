@@ -26,6 +26,11 @@ struct SigmaProb {
     const uint16_t *jmap;    // excitation map over the contracted pairs (FP64-emulating path) or nullptr
     int ldj;
     long long qoff;          // element offset of the quantised copies of c in their wave buffer
+    // plain FP64 path: the integrals, and the string Hamiltonian (nnz elements per string)
+    const double *eri;
+    const double *hval;      // [nnz][nstr]
+    const int *hidx;         // [nnz][nstr]
+    int nnz;
     const double *cbase;
     double *sbase;
     const int *cslot;        // device slot index or nullptr (= 0)
@@ -92,6 +97,20 @@ int upload_plan_to(ifci_handle_t h, SigmaPlan &plan, cudaStream_t s);
 // FP64E: max_qelems and max_delems elements of 8 B.
 int run_sigma(ifci_handle_t h, const SigmaPlan &plan, int precision, void *D, void *G, cudaStream_t s);
 size_t sigma_elem_bytes(int precision);
+
+// plain FP64 sigma (sigma64.cu)
+constexpr int kStringHChunk = 32;              // strings per block of the list build
+struct StringHDesc {
+    int n, m, nstr, nnz;
+    const double *h1, *eri;
+    double *val;             // [nnz][nstr] or nullptr
+    int *idx;                // [nnz][nstr] or nullptr
+};
+int string_h_nnz(int n, int m);
+int launch_string_h(ifci_handle_t h, const StringHDesc &one, cudaStream_t s);
+int launch_string_h_batch(ifci_handle_t h, const StringHDesc *d_desc, const WorkItem *d_items, int nitem, cudaStream_t s);
+int run_sigma64_one(ifci_handle_t h, const SigmaProb &p, cudaStream_t s);
+int run_sigma64(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, cudaStream_t s);
 
 // FP64-accurate sigma on FP16 tensor cores (sigma_oz.cu)
 int oz_operand_bytes(int np);                  // bytes of one problem's sliced W image (+ scale)

@@ -9,40 +9,13 @@
 
 namespace ifci {
 
-struct Binom {
-    int c[32][32];
-};
-
-__device__ __forceinline__ int string_rank(uint32_t mask, const Binom &B) {
-    int r = 0, k = 1;
-    while (mask) {
-        int p = __ffs(mask) - 1;
-        r += B.c[p][k];
-        k++;
-        mask &= mask - 1;
-    }
-    return r;
-}
-
-__device__ __forceinline__ uint32_t string_unrank(int rank, int n, int m, const Binom &B) {
-    uint32_t mask = 0;
-    int rem = rank;
-    for (int k = m; k >= 1; k--) {
-        int p = k - 1;
-        while (p + 1 < n && B.c[p + 1][k] <= rem) p++;
-        rem -= B.c[p][k];
-        mask |= 1u << p;
-    }
-    return mask;
-}
-
 // One thread per string I: its mask and its nexc excitation entries in
 // ascending pair order.
-__global__ void build_strings_kernel(int n, int m, int nstr, int nexc, Binom B,
+__global__ void build_strings_kernel(int n, int m, int nstr, int nexc, StringBinom B,
                                      uint64_t *__restrict__ strings, int32_t *__restrict__ exc) {
     int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nstr) return;
-    uint32_t mask = string_unrank(I, n, m, B);
+    uint32_t mask = string_of_rank(I, n, m, B);
     strings[I] = mask;
     int32_t *row = exc + (size_t)I * nexc;
     int k = 0;
@@ -59,7 +32,7 @@ __global__ void build_strings_kernel(int n, int m, int nstr, int nexc, Binom B,
                 uint32_t J = mask ^ (1u << P) ^ (1u << Q);
                 uint32_t between = ((1u << P) - 1u) & ~((2u << Q) - 1u);
                 int neg = __popc(mask & between) & 1;
-                if (k < nexc) row[k++] = (string_rank(J, B) << 10) | (A << 1) | neg;
+                if (k < nexc) row[k++] = (string_rank_of(J, B) << 10) | (A << 1) | neg;
             }
         }
     }
@@ -134,9 +107,7 @@ int ifci_build_strings(ifci_handle_t h, int norb, int nelec_spin, uint64_t *stri
         return ifci::set_error(h, IFCI_ERR_INVALID_ARG, "build_strings: norb=%d nelec_spin=%d out of range",
                                norb, nelec_spin);
     if (!strings || !exc) return ifci::set_error(h, IFCI_ERR_INVALID_ARG, "build_strings: null output");
-    ifci::Binom B;
-    for (int i = 0; i < 32; i++)
-        for (int j = 0; j < 32; j++) B.c[i][j] = (int)ifci::binom(i, j);
+    const ifci::StringBinom B = ifci::string_binom();
     IFCI_CUDA_TRY(h, cudaSetDevice(h->device));
     int threads = 128, blocks = (nstr + threads - 1) / threads;
     ifci::build_strings_kernel<<<blocks, threads, 0, ifci::as_cuda(stream)>>>(norb, nelec_spin, nstr, nexc, B,
