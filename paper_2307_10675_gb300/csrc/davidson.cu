@@ -211,7 +211,15 @@ __global__ void select_kernel(const DavState *__restrict__ st, int nprob, int mi
 
 // ------------------------------------------------------------------ subspace
 
+// The vector kernels below hold one register value (or several) per basis
+// slot, so they come in two sizes: KM = 12 slots for the default subspace and
+// KM = kMaxSpace = 24 for larger ones.  They are bound by the FP64 pipe, which
+// only fills with enough warps in flight: at 24 slots the residual kernel takes
+// RES24_REGS registers a thread, at 12 slots RES12_REGS, and an expansion of 298 sets
+// spends VEC12_MS ms in them instead of VEC24_MS ms.  The arithmetic is the same.
+
 // partial[item][j] = <b_j | sigma_new> over the item's determinants, j <= newest.
+template <int KM>
 __device__ __forceinline__ void dots_kernel_body(const DavProb *__restrict__ probs, const DavState *__restrict__ st,
                                                    const WorkItem *__restrict__ items, double *__restrict__ part, int w_) {
     const WorkItem it = items[w_];
@@ -219,24 +227,25 @@ __device__ __forceinline__ void dots_kernel_body(const DavProb *__restrict__ pro
     if (!s.active) return;
     const DavProb &p = probs[it.prob];
     const int k = s.newest + 1;
-    double acc[kMaxSpace];
+    double acc[KM];
 #pragma unroll
-    for (int j = 0; j < kMaxSpace; j++) acc[j] = 0.0;
+    for (int j = 0; j < KM; j++) acc[j] = 0.0;
     const double *Sn = p.S + (long long)s.newest * p.ndet;
     long long end = min(it.start + (long long)kVecChunk, p.ndet);
     for (long long I = it.start + threadIdx.x; I < end; I += blockDim.x) {
         const double sv = Sn[I];
 #pragma unroll
-        for (int j = 0; j < kMaxSpace; j++)
+        for (int j = 0; j < KM; j++)
             if (j < k) acc[j] += p.B[(long long)j * p.ndet + I] * sv;
     }
-    block_sum_store<kMaxSpace>(acc, k, part + (long long)w_ * kNP);
+    block_sum_store<KM>(acc, k, part + (long long)w_ * kNP);
 }
 
+template <int KM>
 __global__ void __launch_bounds__(256) dots_kernel(const DavProb *__restrict__ probs, const DavState *__restrict__ st,
                                                    const WorkItem *__restrict__ items, double *__restrict__ part, int nitem_) {
     for (int w = blockIdx.x; w < nitem_; w += gridDim.x) {
-        dots_kernel_body(probs, st, items, part, w);
+        dots_kernel_body<KM>(probs, st, items, part, w);
         __syncthreads();   // shared memory is reused by the next body
     }
 }
@@ -363,6 +372,7 @@ __global__ void __launch_bounds__(32 * kSolveWarps) solve_kernel(const DavProb *
 
 // For the targeted Ritz pair (theta, y): t = sum_j y_j (S_j - theta B_j);
 // ||t||^2; t /= (theta - H_II); dots <b_j|t>.
+template <int KM>
 __device__ __forceinline__ void residual_kernel_body(const DavProb *__restrict__ probs,
                                                        const DavState *__restrict__ st,
                                                        const WorkItem *__restrict__ items,
@@ -377,59 +387,60 @@ __device__ __forceinline__ void residual_kernel_body(const DavProb *__restrict__
     const int tgt = s.tgt < min(k, kKeep) ? s.tgt : 0;
     const double *yt = ys + (long long)it.prob * kYStride + tgt * kNP;
     const double theta = yt[kMaxSpace];
-    double y[kMaxSpace];
+    double y[KM];
 #pragma unroll
-    for (int j = 0; j < kMaxSpace; j++) y[j] = yt[j];
-    double acc[kMaxSpace + 2];
+    for (int j = 0; j < KM; j++) y[j] = yt[j];
+    double acc[KM + 2];
 #pragma unroll
-    for (int j = 0; j < kMaxSpace + 2; j++) acc[j] = 0.0;
+    for (int j = 0; j < KM + 2; j++) acc[j] = 0.0;
     double *T = p.B + (long long)max_space * p.ndet;   // scratch slot for the correction
     long long end = min(it.start + (long long)kVecChunk, p.ndet);
     for (long long I = it.start + threadIdx.x; I < end; I += blockDim.x) {
         double r = 0.0;
-        double bv[kMaxSpace];
+        double bv[KM];
 #pragma unroll
-        for (int j = 0; j < kMaxSpace; j++) {
+        for (int j = 0; j < KM; j++) {
             if (j < k) {
                 bv[j] = p.B[(long long)j * p.ndet + I];
                 r += y[j] * (p.S[(long long)j * p.ndet + I] - theta * bv[j]);
             }
         }
-        acc[kMaxSpace + 1] += r * r;
+        acc[KM + 1] += r * r;
         double den = theta - p.hd[I];
         if (fabs(den) < 1e-4) den = den < 0 ? -1e-4 : 1e-4;
         double t = r / den;
         T[I] = t;
 #pragma unroll
-        for (int j = 0; j < kMaxSpace; j++)
+        for (int j = 0; j < KM; j++)
             if (j < k) acc[j] += bv[j] * t;
-        acc[kMaxSpace] += t * t;
+        acc[KM] += t * t;
     }
     // layout of part: [0..k) dots, kMaxSpace: |t|^2, kMaxSpace+1: |r|^2
-    __shared__ double red[8][kMaxSpace + 2];
+    __shared__ double red[8][KM + 2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int j = 0; j < kMaxSpace + 2; j++) {
-        if (j < k || j >= kMaxSpace) {
+    for (int j = 0; j < KM + 2; j++) {
+        if (j < k || j >= KM) {
             double v = warp_sum(acc[j]);
             if (lane == 0) red[warp][j] = v;
         }
     }
     __syncthreads();
-    if (threadIdx.x < kMaxSpace + 2 && (threadIdx.x < k || threadIdx.x >= kMaxSpace)) {
+    if (threadIdx.x < KM + 2 && (threadIdx.x < k || threadIdx.x >= KM)) {
         double v = 0.0;
         for (int w = 0; w < 8; w++) v += red[w][threadIdx.x];
-        part[(long long)w_ * kNP + threadIdx.x] = v;
+        part[(long long)w_ * kNP + (threadIdx.x < KM ? threadIdx.x : threadIdx.x - KM + kMaxSpace)] = v;
     }
 }
 
+template <int KM>
 __global__ void __launch_bounds__(256) residual_kernel(const DavProb *__restrict__ probs,
                                                        const DavState *__restrict__ st,
                                                        const WorkItem *__restrict__ items,
                                                        const double *__restrict__ ys, int max_space,
                                                        double *__restrict__ part, int nitem_) {
     for (int w = blockIdx.x; w < nitem_; w += gridDim.x) {
-        residual_kernel_body(probs, st, items, ys, max_space, part, w);
+        residual_kernel_body<KM>(probs, st, items, ys, max_space, part, w);
         __syncthreads();   // shared memory is reused by the next body
     }
 }
@@ -573,6 +584,7 @@ __global__ void check_kernel(const DavProb *__restrict__ probs, DavState *__rest
 // correction from the scratch slot to slot nform, a phase switch of the mixed
 // mode (tslot < 0) drops it and rebuilds the S_r exactly.  Every old slot of
 // an element is read before any is written.
+template <int KM>
 __device__ __forceinline__ void restart_kernel_body(const DavProb *__restrict__ probs,
                                                       const DavState *__restrict__ st,
                                                       const WorkItem *__restrict__ items, const double *__restrict__ ys,
@@ -588,9 +600,9 @@ __device__ __forceinline__ void restart_kernel_body(const DavProb *__restrict__ 
     const double *T = p.B + (long long)max_space * p.ndet;
     const int kk = s.kold;   // only the slots of the old subspace are read
     for (long long I = it.start + threadIdx.x; I < end; I += blockDim.x) {
-        double bv[kMaxSpace], sv[kMaxSpace];
+        double bv[KM], sv[KM];
 #pragma unroll
-        for (int j = 0; j < kMaxSpace; j++) {
+        for (int j = 0; j < KM; j++) {
             bv[j] = j < kk ? p.B[(long long)j * p.ndet + I] : 0.0;
             sv[j] = j < kk ? p.S[(long long)j * p.ndet + I] : 0.0;
         }
@@ -599,7 +611,7 @@ __device__ __forceinline__ void restart_kernel_body(const DavProb *__restrict__ 
             if (r < keep) {
                 double x = 0.0, sx = 0.0;
 #pragma unroll
-                for (int j = 0; j < kMaxSpace; j++) {
+                for (int j = 0; j < KM; j++) {
                     x += yr[r * kNP + j] * bv[j];
                     sx += yr[r * kNP + j] * sv[j];
                 }
@@ -611,14 +623,16 @@ __device__ __forceinline__ void restart_kernel_body(const DavProb *__restrict__ 
     }
 }
 
+template <int KM>
 __global__ void __launch_bounds__(256) restart_kernel(const DavProb *__restrict__ probs,
                                                       const DavState *__restrict__ st,
                                                       const WorkItem *__restrict__ items, const double *__restrict__ ys,
                                                       int max_space, int mixed, int nitem_) {
-    for (int w = blockIdx.x; w < nitem_; w += gridDim.x) restart_kernel_body(probs, st, items, ys, max_space, mixed, w);
+    for (int w = blockIdx.x; w < nitem_; w += gridDim.x) restart_kernel_body<KM>(probs, st, items, ys, max_space, mixed, w);
 }
 
 // t -= sum_{j<k} coef_j b_j ; then dots <b_j|t> and |t|^2 for the next pass.
+template <int KM>
 __device__ __forceinline__ void ortho_kernel_body(const DavProb *__restrict__ probs, const DavState *__restrict__ st,
                                                     const WorkItem *__restrict__ items,
                                                     const double *__restrict__ coef, int max_space,
@@ -629,53 +643,54 @@ __device__ __forceinline__ void ortho_kernel_body(const DavProb *__restrict__ pr
     if (pass == 1 && s.skip2) return;
     const DavProb &p = probs[it.prob];
     const int k = s.k;
-    double c[kMaxSpace];
+    double c[KM];
 #pragma unroll
-    for (int j = 0; j < kMaxSpace; j++) c[j] = coef[(long long)it.prob * kNP + j];
+    for (int j = 0; j < KM; j++) c[j] = coef[(long long)it.prob * kNP + j];
     double *T = p.B + (long long)s.tslot * p.ndet;
     if (!s.restart && s.tslot == k) T = p.B + (long long)max_space * p.ndet;
-    double acc[kMaxSpace + 1];
+    double acc[KM + 1];
 #pragma unroll
-    for (int j = 0; j <= kMaxSpace; j++) acc[j] = 0.0;
+    for (int j = 0; j <= KM; j++) acc[j] = 0.0;
     long long end = min(it.start + (long long)kVecChunk, p.ndet);
     for (long long I = it.start + threadIdx.x; I < end; I += blockDim.x) {
         double t = T[I];
-        double bv[kMaxSpace];
+        double bv[KM];
 #pragma unroll
-        for (int j = 0; j < kMaxSpace; j++)
+        for (int j = 0; j < KM; j++)
             if (j < k) {
                 bv[j] = p.B[(long long)j * p.ndet + I];
                 t -= c[j] * bv[j];
             }
         T[I] = t;
 #pragma unroll
-        for (int j = 0; j < kMaxSpace; j++)
+        for (int j = 0; j < KM; j++)
             if (j < k) acc[j] += bv[j] * t;
-        acc[kMaxSpace] += t * t;
+        acc[KM] += t * t;
     }
-    __shared__ double red[8][kMaxSpace + 1];
+    __shared__ double red[8][KM + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int j = 0; j <= kMaxSpace; j++) {
-        if (j < k || j == kMaxSpace) {
+    for (int j = 0; j <= KM; j++) {
+        if (j < k || j == KM) {
             double v = warp_sum(acc[j]);
             if (lane == 0) red[warp][j] = v;
         }
     }
     __syncthreads();
-    if (threadIdx.x <= kMaxSpace && (threadIdx.x < k || threadIdx.x == kMaxSpace)) {
+    if (threadIdx.x <= KM && (threadIdx.x < k || threadIdx.x == KM)) {
         double v = 0.0;
         for (int w = 0; w < 8; w++) v += red[w][threadIdx.x];
-        part[(long long)w_ * kNP + threadIdx.x] = v;
+        part[(long long)w_ * kNP + (threadIdx.x < KM ? (int)threadIdx.x : kMaxSpace)] = v;
     }
 }
 
+template <int KM>
 __global__ void __launch_bounds__(256) ortho_kernel(const DavProb *__restrict__ probs, const DavState *__restrict__ st,
                                                     const WorkItem *__restrict__ items,
                                                     const double *__restrict__ coef, int max_space,
                                                     double *__restrict__ part, int pass, int nitem_) {
     for (int w = blockIdx.x; w < nitem_; w += gridDim.x) {
-        ortho_kernel_body(probs, st, items, coef, max_space, part, pass, w);
+        ortho_kernel_body<KM>(probs, st, items, coef, max_space, part, pass, w);
         __syncthreads();   // shared memory is reused by the next body
     }
 }
@@ -896,12 +911,14 @@ static int dav_step(ifci_handle_t h, DavBatch &b, SigmaPlan &hi_plan, SigmaPlan 
         IFCI_LAUNCH_CHECK(h);
     }
     ProfScope vec_scope(h, s, PK_VECTOR);
-    dots_kernel<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_part, nitem);
+    const bool small = b.max_space <= kSmallSpace;
+    (small ? dots_kernel<kSmallSpace> : dots_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_part, nitem);
     IFCI_LAUNCH_CHECK(h);
     solve_kernel<<<stride_grid(h->device, (b.nprob + kSolveWarps - 1) / kSolveWarps, 8), 32 * kSolveWarps, 0, s>>>(
         b.d_probs, b.d_state, b.d_part, b.d_gs, b.d_y, b.nprob);
     IFCI_LAUNCH_CHECK(h);
-    residual_kernel<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_y, b.max_space, b.d_part, nitem);
+    (small ? residual_kernel<kSmallSpace> : residual_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(
+        b.d_probs, b.d_state, b.d_vitems, b.d_y, b.max_space, b.d_part, nitem);
     IFCI_LAUNCH_CHECK(h);
     IFCI_CUDA_TRY(h, cudaMemsetAsync(b.d_nactive, 0, sizeof(int), s));
     // check_kernel records the subspace size before a restart (kold) for restart_kernel
@@ -909,10 +926,12 @@ static int dav_step(ifci_handle_t h, DavBatch &b, SigmaPlan &hi_plan, SigmaPlan 
                                         restart_at, b.keep, mixed ? 1 : 0, b.max_iter, b.e_tol, b.r_tol,
                                         b.d_nactive, b.nprob);
     IFCI_LAUNCH_CHECK(h);
-    restart_kernel<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_y, b.max_space, mixed ? 1 : 0, nitem);
+    (small ? restart_kernel<kSmallSpace> : restart_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_y,
+                                                                                    b.max_space, mixed ? 1 : 0, nitem);
     IFCI_LAUNCH_CHECK(h);
     for (int pass = 0; pass < 2; pass++) {
-        ortho_kernel<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_coef, b.max_space, b.d_part, pass, nitem);
+        (small ? ortho_kernel<kSmallSpace> : ortho_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_coef,
+                                                                                b.max_space, b.d_part, pass, nitem);
         IFCI_LAUNCH_CHECK(h);
         reduce_coef_kernel<<<gp, 32, 0, s>>>(b.d_probs, b.d_state, b.d_part, b.d_coef, pass, b.nprob);
         IFCI_LAUNCH_CHECK(h);

@@ -60,6 +60,7 @@ struct DavState {
 
 constexpr int kVecChunk = 4096;   // determinants per vector work item
 constexpr int kMaxSpace = 24;
+constexpr int kSmallSpace = 12;   // subspaces up to here take the smaller instances of the vector kernels
 constexpr int kNP = kMaxSpace + 2;
 // thick restart keeps the lowest kKeep Ritz vectors (a near-degenerate pair
 // of lowest states is resolved by Rayleigh-Ritz instead of being re-found
