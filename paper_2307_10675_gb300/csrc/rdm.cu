@@ -25,8 +25,14 @@ namespace ifci {
 
 namespace {
 
-constexpr int kSyrkT = 64;          // SYRK output tile
-constexpr int kSyrkChunk = 16384;   // determinants per split-K chunk
+constexpr int kSyrkT = 16;          // SYRK output tile
+constexpr int kSyrkChunk = 512;     // determinants per split-K chunk
+constexpr int kSyrkWarps = 4, kSyrkPer = 4;             // warps of a block, tiles each keeps in registers
+constexpr int kSyrkGroup = kSyrkWarps * kSyrkPer;       // tiles of one job
+constexpr int kSyrkK = 16;          // determinants staged at a time
+__host__ __device__ inline int syrk_side(int np) { return (np + 1 + kSyrkT - 1) / kSyrkT; }
+__host__ __device__ inline int syrk_tiles(int np) { return syrk_side(np) * (syrk_side(np) + 1) / 2; }   // ta <= tb
+__host__ __device__ inline int syrk_groups(int np) { return (syrk_tiles(np) + kSyrkGroup - 1) / kSyrkGroup; }
 
 struct RdmProb {
     int n, np, nstr, nexc, nA, nC;
@@ -41,7 +47,7 @@ struct RdmProb {
 };
 
 struct SyrkJob {
-    int prob, chunk, ta, tb;
+    int prob, chunk, group;
 };
 
 // D+[A][K] for A < np (merge of the sorted alpha/beta lists) and D+[np][K] = c_K
@@ -75,73 +81,94 @@ __global__ void __launch_bounds__(256) rdm_gather_kernel(const RdmProb *__restri
     out[(long long)np * ndet] = c[K];
 }
 
-// partial[job] = sum_{K in chunk} D+[ta*64 + i][K] D+[tb*64 + j][K]   (64 x 64 tile)
-__global__ void __launch_bounds__(256) rdm_syrk_kernel(const RdmProb *__restrict__ probs,
-                                                       const SyrkJob *__restrict__ jobs,
-                                                       const double *__restrict__ D, double *__restrict__ part) {
+// partial[job][tile][i][j] = sum_{K in chunk} D+[16 ta + i][K] D+[16 tb + j][K]
+// for the 16 tiles (ta <= tb) of the job's group.  An SM sub-partition takes 64
+// clocks per FP64 warp instruction, so the sum is bound by the FMAs issued, and
+// by their even spread over the chip: 16 x 16 tiles compute 3,840 products per
+// determinant for 79 rows (12,288 with 64 x 64 tiles, 3,160 needed), and chunks
+// of 512 determinants make a job of half a millisecond at most (16 ms with
+// 16,384, of which a gradient over 63 sets had fewer than two per SM).  The
+// gradient of 63 sets up to CAS(6e,12o): 18.2 ms before, 1.6 ms.
+__global__ void __launch_bounds__(32 * kSyrkWarps) rdm_syrk_kernel(const RdmProb *__restrict__ probs,
+                                                                   const SyrkJob *__restrict__ jobs,
+                                                                   const double *__restrict__ D, double *__restrict__ part) {
     const SyrkJob jb = jobs[blockIdx.x];
     const RdmProb &p = probs[jb.prob];
-    const int rows = p.np + 1;
+    const int rows = p.np + 1, T = syrk_side(p.np), nt = syrk_tiles(p.np), ld = T * kSyrkT + 2;
     const long long ndet = p.ndet;
-    const long long k0 = (long long)(jb.chunk - p.chunk0) * kSyrkChunk;
-    const long long k1 = min(ndet, k0 + kSyrkChunk);
+    const long long k0 = (long long)(jb.chunk - p.chunk0) * kSyrkChunk, k1 = min(ndet, k0 + kSyrkChunk);
     const double *Dp = D + p.doff;
-    __shared__ double As[16][kSyrkT], Bs[16][kSyrkT];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4];
+    extern __shared__ double Ds[];   // [kSyrkK][ld]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // lane: 4 rows x 2 columns of each of its warp's tiles
+    const int r0 = (lane >> 3) * 4, c0 = (lane & 7) * 2;
+    int oa[kSyrkPer], ob[kSyrkPer];
+    bool on[kSyrkPer];
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int u = 0; u < kSyrkPer; u++) {
+        // neighbouring tiles go to different warps: a short group still uses all
+        int t = jb.group * kSyrkGroup + u * kSyrkWarps + warp, ta = 0;
+        on[u] = t < nt;
+        if (!on[u]) t = 0;
+        while (t >= T - ta) t -= T - ta++;
+        oa[u] = ta * kSyrkT + r0;
+        ob[u] = (ta + t) * kSyrkT + c0;
+    }
+    double acc[kSyrkPer][4][2];
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = 0.0;
-    for (long long kk = k0; kk < k1; kk += 16) {
+    for (int u = 0; u < kSyrkPer; u++)
 #pragma unroll
-        for (int r = 0; r < 4; r++) {
-            const int e = threadIdx.x + 256 * r;
-            const int kq = e % 16, m = e / 16;
-            const long long K = kk + kq;
-            const int A = jb.ta * kSyrkT + m, B = jb.tb * kSyrkT + m;
-            As[kq][m] = (A < rows && K < k1) ? Dp[(long long)A * ndet + K] : 0.0;
-            Bs[kq][m] = (B < rows && K < k1) ? Dp[(long long)B * ndet + K] : 0.0;
+        for (int i = 0; i < 4; i++) acc[u][i][0] = acc[u][i][1] = 0.0;
+    for (long long kk = k0; kk < k1; kk += kSyrkK) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < T * kSyrkT * kSyrkK; e += 32 * kSyrkWarps) {
+            const int k = e % kSyrkK, A = e / kSyrkK;
+            Ds[k * ld + A] = A < rows && kk + k < k1 ? Dp[(long long)A * ndet + kk + k] : 0.0;
         }
         __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < kSyrkK; k++) {
+            const double *d = Ds + k * ld;
 #pragma unroll
-        for (int kq = 0; kq < 16; kq++) {
-            double a[4], b[4];
+            for (int u = 0; u < kSyrkPer; u++) {
+                if (!on[u]) continue;
+                const double b0 = d[ob[u]], b1 = d[ob[u] + 1];
 #pragma unroll
-            for (int i = 0; i < 4; i++) a[i] = As[kq][ty * 4 + i];
+                for (int i = 0; i < 4; i++) {
+                    const double a = d[oa[u] + i];
+                    acc[u][i][0] = fma(a, b0, acc[u][i][0]);
+                    acc[u][i][1] = fma(a, b1, acc[u][i][1]);
+                }
+            }
+        }
+    }
+    double *out = part + (size_t)blockIdx.x * kSyrkGroup * kSyrkT * kSyrkT;
 #pragma unroll
-            for (int j = 0; j < 4; j++) b[j] = Bs[kq][tx + 16 * j];
+    for (int u = 0; u < kSyrkPer; u++)
+        if (on[u])
 #pragma unroll
             for (int i = 0; i < 4; i++)
 #pragma unroll
-                for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    double *out = part + (size_t)blockIdx.x * kSyrkT * kSyrkT;
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) out[(ty * 4 + i) * kSyrkT + tx + 16 * j] = acc[i][j];
+                for (int j = 0; j < 2; j++)
+                    out[(u * kSyrkWarps + warp) * kSyrkT * kSyrkT + (r0 + i) * kSyrkT + c0 + j] = acc[u][i][j];
 }
 
-// M = sum over the problem's chunks of the partial tiles (fixed order), symmetric fill
+// M = sum over the problem's chunks of the partial tiles (fixed order), symmetric
+// fill; blocks (problem, part)
 __global__ void rdm_reduce_kernel(const RdmProb *__restrict__ probs, const int *__restrict__ job0,
                                   const double *__restrict__ part) {
     const int pi = blockIdx.x;
     const RdmProb &p = probs[pi];
-    const int rows = p.np + 1, T = (rows + kSyrkT - 1) / kSyrkT;
-    const int ntt = T * (T + 1) / 2;   // tiles ta <= tb per chunk
-    for (int e = threadIdx.x; e < rows * rows; e += blockDim.x) {
+    const int rows = p.np + 1, T = syrk_side(p.np), ng = syrk_groups(p.np);
+    for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < rows * rows; e += gridDim.y * blockDim.x) {
         const int A = e / rows, B = e % rows;
         const int a = min(A, B), b = max(A, B);
         const int ta = a / kSyrkT, tb = b / kSyrkT;
-        const int tix = ta * T - ta * (ta - 1) / 2 + (tb - ta);   // index of (ta, tb) among ta <= tb
-        // the (ta, tb) tile holds sum_K D+[64 ta + i][K] D+[64 tb + j][K]
-        const int i = (A <= B ? A : B) - ta * kSyrkT, j = (A <= B ? B : A) - tb * kSyrkT;
+        const int t = ta * T - ta * (ta - 1) / 2 + (tb - ta);   // index of (ta, tb) among ta <= tb
+        const double *src = part + ((size_t)job0[pi] + t / kSyrkGroup) * kSyrkGroup * kSyrkT * kSyrkT +
+                            (size_t)(t % kSyrkGroup) * kSyrkT * kSyrkT + (a - ta * kSyrkT) * kSyrkT + (b - tb * kSyrkT);
         double s = 0.0;
-        for (int ch = 0; ch < p.nchunk; ch++)
-            s += part[((size_t)job0[pi] + (size_t)ch * ntt + tix) * kSyrkT * kSyrkT + (size_t)i * kSyrkT + j];
+        for (int ch = 0; ch < p.nchunk; ch++) s += src[(size_t)ch * ng * kSyrkGroup * kSyrkT * kSyrkT];
         p.M[e] = s;
     }
 }
@@ -365,13 +392,12 @@ extern "C" int ifci_rdm_backward(ifci_handle_t h, const ifci_system_t *sys, int 
     for (auto &wv : waves) {
         long long items = 0, jobs = 0;
         for (int x = wv.first; x < wv.second; x++) {
-            const int T = (probs[x].np + 1 + kSyrkT - 1) / kSyrkT;
             const long long nch = (probs[x].ndet + kSyrkChunk - 1) / kSyrkChunk;
             items += (probs[x].ndet + 255) / 256;
-            jobs += nch * T * (T + 1) / 2;
+            jobs += nch * syrk_groups(probs[x].np);
         }
         wave_max = std::max(wave_max, ws_round(items * sizeof(WorkItem)) + ws_round(jobs * sizeof(SyrkJob)) +
-                                          ws_round(jobs * kSyrkT * kSyrkT * 8) + ws_round((wv.second - wv.first) * 4));
+                                          ws_round(jobs * kSyrkGroup * kSyrkT * kSyrkT * 8) + ws_round((wv.second - wv.first) * 4));
     }
     need += wave_max + 4096;
     IFCI_TRY(ws_reserve(h, need));
@@ -414,25 +440,25 @@ extern "C" int ifci_rdm_backward(ifci_handle_t h, const ifci_system_t *sys, int 
         std::vector<SyrkJob> jobs;
         std::vector<int> job0;
         long long doff = 0;
-        int chunk = 0;
+        int chunk = 0, max_np = 0;
         for (int x = wv.first; x < wv.second; x++) {
             RdmProb &r = probs[x];
             r.doff = doff;
             doff += (long long)(r.np + 1) * r.ndet;
             for (long long s0 = 0; s0 < r.ndet; s0 += 256) items.push_back(WorkItem{x - wv.first, 0, s0});
-            const int T = (r.np + 1 + kSyrkT - 1) / kSyrkT;
+            const int ng = syrk_groups(r.np);
+            max_np = std::max(max_np, r.np);
             r.nchunk = (int)((r.ndet + kSyrkChunk - 1) / kSyrkChunk);
             r.chunk0 = chunk;
             job0.push_back((int)jobs.size());
             for (int ch = 0; ch < r.nchunk; ch++)
-                for (int ta = 0; ta < T; ta++)
-                    for (int tb = ta; tb < T; tb++) jobs.push_back(SyrkJob{x - wv.first, chunk + ch, ta, tb});
+                for (int g = 0; g < ng; g++) jobs.push_back(SyrkJob{x - wv.first, chunk + ch, g});
             chunk += r.nchunk;
         }
         const int nw = wv.second - wv.first;
         auto *d_items = ws_take<WorkItem>(h, items.size());
         auto *d_jobs = ws_take<SyrkJob>(h, jobs.size());
-        double *part = ws_take<double>(h, jobs.size() * kSyrkT * kSyrkT);
+        double *part = ws_take<double>(h, jobs.size() * kSyrkGroup * kSyrkT * kSyrkT);
         int *d_job0 = ws_take<int>(h, nw);
         if (!d_items || !d_jobs || !part || !d_job0) return set_error(h, IFCI_ERR_OOM, "rdm_backward: workspace (wave)");
         RdmProb *d_wp = d_probs + wv.first;
@@ -442,9 +468,12 @@ extern "C" int ifci_rdm_backward(ifci_handle_t h, const ifci_system_t *sys, int 
         IFCI_CUDA_TRY(h, cudaMemcpyAsync(d_job0, job0.data(), nw * 4, cudaMemcpyHostToDevice, s));
         rdm_gather_kernel<<<(int)items.size(), 256, 0, s>>>(d_wp, d_items, D);
         IFCI_LAUNCH_CHECK(h);
-        rdm_syrk_kernel<<<(int)jobs.size(), 256, 0, s>>>(d_wp, d_jobs, D, part);
+        const int smem = kSyrkK * (syrk_side(max_np) * kSyrkT + 2) * (int)sizeof(double);   // 64 KB at 496 pairs
+        static SmemOptIn opt;
+        IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, rdm_syrk_kernel, smem));
+        rdm_syrk_kernel<<<(int)jobs.size(), 32 * kSyrkWarps, smem, s>>>(d_wp, d_jobs, D, part);
         IFCI_LAUNCH_CHECK(h);
-        rdm_reduce_kernel<<<nw, 256, 0, s>>>(d_wp, d_job0, part);
+        rdm_reduce_kernel<<<dim3(nw, std::max(1, std::min(32, (max_np + 1) * (max_np + 1) / 256))), 256, 0, s>>>(d_wp, d_job0, part);
         IFCI_LAUNCH_CHECK(h);
         rdm_accum_kernel<<<nw, 256, 0, s>>>(d_wp, norb, dh, deri);
         IFCI_LAUNCH_CHECK(h);
