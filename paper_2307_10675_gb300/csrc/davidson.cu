@@ -214,9 +214,10 @@ __global__ void select_kernel(const DavState *__restrict__ st, int nprob, int mi
 // The vector kernels below hold one register value (or several) per basis
 // slot, so they come in two sizes: KM = 12 slots for the default subspace and
 // KM = kMaxSpace = 24 for larger ones.  They are bound by the FP64 pipe, which
-// only fills with enough warps in flight: at 24 slots the residual kernel takes
-// RES24_REGS registers a thread, at 12 slots RES12_REGS, and an expansion of 298 sets
-// spends VEC12_MS ms in them instead of VEC24_MS ms.  The arithmetic is the same.
+// only fills with enough warps in flight: the residual kernel takes 255
+// registers a thread for 24 slots and 198 for 12, the Gram-Schmidt kernel 255
+// and 155.  An expansion of 298 sets (subspace 12) spends 90.5 ms in the vector
+// kernels, 122.6 ms with the 24-slot ones.  The arithmetic is the same.
 
 // partial[item][j] = <b_j | sigma_new> over the item's determinants, j <= newest.
 template <int KM>
@@ -250,124 +251,147 @@ __global__ void __launch_bounds__(256) dots_kernel(const DavProb *__restrict__ p
     }
 }
 
-// Cyclic Jacobi on the symmetric k x k matrix A (shared memory, row stride
-// kSolveLd) by one warp: every lane derives the same rotation from the
-// settled entries, then lane r rotates row r / column r (columns, rows and V
-// in turn, as the serial sweep does, so the arithmetic per element is the
-// same).  A sweep ends the iteration once the off-diagonal part is below
-// 1e-26 of |A|_F^2 (eigenvalue errors ~1e-26 |A| / gap); a rotation whose
-// A_pq is below 1e-18 (|A_pp| + |A_qq|) only sets A_pq = A_qp = 0.
-constexpr int kSolveLd = kMaxSpace + 1;
+// Cyclic Jacobi on symmetric k x k matrices A (shared memory, row stride LD),
+// one per group of G lanes (32 / G problems share a warp): every lane of a group
+// derives the same rotation from the settled entries, then lane r rotates row
+// r / column r (columns, rows and V in turn, as the serial sweep does, so the
+// arithmetic per element is the same).  A sweep ends the iteration once the
+// off-diagonal part is below 1e-26 of |A|_F^2 (eigenvalue errors ~1e-26 |A| /
+// gap); a rotation whose A_pq is below 1e-18 (|A_pp| + |A_qq|) only sets
+// A_pq = A_qp = 0.  The groups walk the index pairs together, one that has
+// nothing to rotate writes nothing: an FP64 warp instruction takes 64 clocks
+// for one lane as for 32, so two subspaces of up to 16 vectors cost one.
 constexpr int kSolveWarps = 4;
 
+template <int G, int LD>
 __device__ void jacobi_warp(double *A, double *V, int k, int lane) {
+    int kmax = k;
+#pragma unroll
+    for (int o = 16; o >= G; o >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
     if (lane < k)
-        for (int j = 0; j < k; j++) V[lane * kSolveLd + j] = lane == j ? 1.0 : 0.0;
+        for (int j = 0; j < k; j++) V[lane * LD + j] = lane == j ? 1.0 : 0.0;
     __syncwarp();
+    bool done = k < 2;
     for (int sweep = 0; sweep < 60; sweep++) {
         double off = 0.0, tot = 0.0;
         if (lane < k)
             for (int j = 0; j < k; j++) {
-                const double a = A[lane * kSolveLd + j];
+                const double a = A[lane * LD + j];
                 tot += a * a;
                 if (j != lane) off += a * a;
             }
-        off = warp_sum(off);
-        tot = warp_sum(tot);
-        if (off <= 1e-26 * tot || off == 0.0) break;
-        for (int pp = 0; pp < k - 1; pp++)
-            for (int q = pp + 1; q < k; q++) {
-                const double apq = A[pp * kSolveLd + q];
-                if (apq == 0.0) continue;
-                const double app = A[pp * kSolveLd + pp], aqq = A[q * kSolveLd + q];
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        }
+        done = done || off <= 1e-26 * tot || off == 0.0;
+        if (__all_sync(0xffffffffu, done)) break;
+        for (int pp = 0; pp < kmax - 1; pp++)
+            for (int q = pp + 1; q < kmax; q++) {
+                const bool in = !done && q < k;
+                const double apq = in ? A[pp * LD + q] : 0.0;
+                const bool go = (dbits(apq) << 1) != 0;   // not +-0
+                const double app = in ? A[pp * LD + pp] : 0.0, aqq = in ? A[q * LD + q] : 0.0;
+                const bool tiny = go && jacobi_negligible(app, aqq, apq);
+                const bool rot = go && !tiny;
                 __syncwarp();   // every lane has read the rotation's entries
-                if (fabs(apq) <= 1e-18 * (fabs(app) + fabs(aqq))) {
-                    if (lane == 0) A[pp * kSolveLd + q] = A[q * kSolveLd + pp] = 0.0;
-                    __syncwarp();
-                    continue;
-                }
-                double c, sn;
-                jacobi_rotation(app, aqq, apq, c, sn);
-                if (lane < k) {
-                    const double arp = A[lane * kSolveLd + pp], arq = A[lane * kSolveLd + q];
-                    A[lane * kSolveLd + pp] = c * arp - sn * arq;
-                    A[lane * kSolveLd + q] = sn * arp + c * arq;
+                if (tiny && lane == 0) A[pp * LD + q] = A[q * LD + pp] = 0.0;
+                if (!__any_sync(0xffffffffu, rot)) continue;   // the vote orders the zeros written above
+                double c = 1.0, sn = 0.0;
+                if (rot) jacobi_rotation(app, aqq, apq, c, sn);
+                __syncwarp();
+                const bool mine = rot && lane < k;
+                if (mine) {
+                    const double arp = A[lane * LD + pp], arq = A[lane * LD + q];
+                    A[lane * LD + pp] = c * arp - sn * arq;
+                    A[lane * LD + q] = sn * arp + c * arq;
                 }
                 __syncwarp();
-                if (lane < k) {
-                    const double apr = A[pp * kSolveLd + lane], aqr = A[q * kSolveLd + lane];
-                    A[pp * kSolveLd + lane] = c * apr - sn * aqr;
-                    A[q * kSolveLd + lane] = sn * apr + c * aqr;
-                    const double vrp = V[lane * kSolveLd + pp], vrq = V[lane * kSolveLd + q];
-                    V[lane * kSolveLd + pp] = c * vrp - sn * vrq;
-                    V[lane * kSolveLd + q] = sn * vrp + c * vrq;
+                if (mine) {
+                    const double apr = A[pp * LD + lane], aqr = A[q * LD + lane];
+                    A[pp * LD + lane] = c * apr - sn * aqr;
+                    A[q * LD + lane] = sn * apr + c * aqr;
+                    const double vrp = V[lane * LD + pp], vrq = V[lane * LD + q];
+                    V[lane * LD + pp] = c * vrp - sn * vrq;
+                    V[lane * LD + q] = sn * vrp + c * vrq;
                 }
                 __syncwarp();
             }
     }
 }
 
-// One warp per problem: finish the subspace column and solve the projected
-// problem (its kKeep lowest Ritz pairs).
-__device__ __forceinline__ void solve_warp_body(const DavProb *__restrict__ probs, DavState *__restrict__ st,
-                                                const double *__restrict__ part, double *__restrict__ gs,
-                                                double *__restrict__ ys, int i, double *A, double *V) {
-    const int lane = threadIdx.x & 31;
-    DavState s = st[i];
-    if (!s.active) return;
-    const DavProb &p = probs[i];
-    const int k = s.newest + 1;
-    double *Gm = gs + (long long)i * kMaxSpace * kMaxSpace;
+// G lanes per problem: finish the subspace column and solve the projected
+// problem (its kKeep lowest Ritz pairs).  `i` = the group's problem, -1: none.
+template <int G, int LD>
+__device__ __forceinline__ void solve_body(const DavProb *__restrict__ probs, DavState *__restrict__ st,
+                                           const double *__restrict__ part, double *__restrict__ gs,
+                                           double *__restrict__ ys, int i, double *A, double *V) {
+    const int lane = threadIdx.x & (G - 1);
+    DavState s{};
+    if (i >= 0) s = st[i];
+    const bool on = i >= 0 && s.active;
+    const int k = on ? s.newest + 1 : 0;
     if (lane < k) {
+        const DavProb &p = probs[i];
+        double *Gm = gs + (long long)i * kMaxSpace * kMaxSpace;
         double v = 0.0;
         for (int w = 0; w < p.nitem; w++) v += part[(long long)(p.item0 + w) * kNP + lane];
         Gm[lane * kMaxSpace + s.newest] = v;
         Gm[s.newest * kMaxSpace + lane] = v;
     }
     __syncwarp();
-    if (lane < k)
-        for (int b = 0; b < k; b++) A[lane * kSolveLd + b] = 0.5 * (Gm[lane * kMaxSpace + b] + Gm[b * kMaxSpace + lane]);
+    if (lane < k) {
+        const double *Gm = gs + (long long)i * kMaxSpace * kMaxSpace;
+        for (int b = 0; b < k; b++) A[lane * LD + b] = 0.5 * (Gm[lane * kMaxSpace + b] + Gm[b * kMaxSpace + lane]);
+    }
     __syncwarp();
-    jacobi_warp(A, V, k, lane);
-    if (lane == 0) {
-        // the nk lowest eigenpairs in ascending order; each vector's largest
-        // component made positive (deterministic sign)
-        const int nk = k < kKeep ? k : kKeep;
+    jacobi_warp<G, LD>(A, V, k, lane);
+    // the lowest eigenpairs in ascending order (ties by index), lane j ranking
+    // eigenvalue j and writing its vector; each vector's largest component made
+    // positive (deterministic sign)
+    if (on) {
         double *yo = ys + (long long)i * kYStride;
-        bool used[kMaxSpace];
-        for (int j = 0; j < k; j++) used[j] = false;
-        for (int r = 0; r < kKeep; r++) {
-            if (r >= nk) {
-                for (int j = 0; j < kNP; j++) yo[r * kNP + j] = 0.0;
-                continue;
+        for (int r = k; r < kKeep; r++)
+            for (int j = lane; j < kNP; j += G) yo[r * kNP + j] = 0.0;
+        if (lane < k) {
+            const double e = A[lane * LD + lane];
+            const long long key = dkey(e);
+            int rank = 0, big = 0;
+            long long bm = dmag(V[lane]);
+            for (int j = 0; j < k; j++) {
+                const long long o = dkey(A[j * LD + j]), m = dmag(V[j * LD + lane]);
+                rank += o < key || (o == key && j < lane);
+                if (m > bm) {
+                    bm = m;
+                    big = j;
+                }
             }
-            int best = -1;
-            for (int j = 0; j < k; j++)
-                if (!used[j] && (best < 0 || A[j * kSolveLd + j] < A[best * kSolveLd + best])) best = j;
-            used[best] = true;
-            int big = 0;
-            for (int j = 1; j < k; j++)
-                if (fabs(V[j * kSolveLd + best]) > fabs(V[big * kSolveLd + best])) big = j;
-            const double sg = V[big * kSolveLd + best] < 0 ? -1.0 : 1.0;
-            for (int j = 0; j < kNP; j++) yo[r * kNP + j] = j < k ? sg * V[j * kSolveLd + best] : 0.0;
-            yo[r * kNP + kMaxSpace] = A[best * kSolveLd + best];
-            if (r == 0) s.theta = A[best * kSolveLd + best];
+            if (rank < kKeep) {
+                const uint32_t neg = (uint32_t)__double2hiint(V[big * LD + lane]) & 0x80000000u;
+                for (int j = 0; j < kNP; j++) yo[rank * kNP + j] = j < k ? dflip(V[j * LD + lane], neg) : 0.0;
+                yo[rank * kNP + kMaxSpace] = e;
+                if (rank == 0) {
+                    st[i].theta = e;
+                    st[i].iters = s.iters + 1;
+                }
+            }
         }
-        s.iters += 1;
-        st[i] = s;
     }
     __syncwarp();   // A and V are reused by the warp's next problem
 }
 
+template <int G, int LD>
 __global__ void __launch_bounds__(32 * kSolveWarps) solve_kernel(const DavProb *__restrict__ probs,
                                                                  DavState *__restrict__ st,
                                                                  const double *__restrict__ part,
                                                                  double *__restrict__ gs, double *__restrict__ ys,
                                                                  int nprob_) {
-    __shared__ double sm[kSolveWarps][2][kMaxSpace * kSolveLd];
-    const int warp = threadIdx.x >> 5;
-    for (int w = blockIdx.x * kSolveWarps + warp; w < nprob_; w += gridDim.x * kSolveWarps)
-        solve_warp_body(probs, st, part, gs, ys, w, sm[warp][0], sm[warp][1]);
+    constexpr int kGroups = 32 * kSolveWarps / G;   // problems a block takes at a time
+    __shared__ double sm[kGroups][2][(LD - 1) * LD];
+    const int g = threadIdx.x / G;
+    for (int w0 = blockIdx.x * kGroups; w0 < nprob_; w0 += gridDim.x * kGroups)
+        solve_body<G, LD>(probs, st, part, gs, ys, w0 + g < nprob_ ? w0 + g : -1, sm[g][0], sm[g][1]);
 }
 
 // For the targeted Ritz pair (theta, y): t = sum_j y_j (S_j - theta B_j);
@@ -914,8 +938,12 @@ static int dav_step(ifci_handle_t h, DavBatch &b, SigmaPlan &hi_plan, SigmaPlan 
     const bool small = b.max_space <= kSmallSpace;
     (small ? dots_kernel<kSmallSpace> : dots_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_part, nitem);
     IFCI_LAUNCH_CHECK(h);
-    solve_kernel<<<stride_grid(h->device, (b.nprob + kSolveWarps - 1) / kSolveWarps, 8), 32 * kSolveWarps, 0, s>>>(
-        b.d_probs, b.d_state, b.d_part, b.d_gs, b.d_y, b.nprob);
+    if (b.max_space <= 16)
+        solve_kernel<16, 17><<<stride_grid(h->device, (b.nprob + 2 * kSolveWarps - 1) / (2 * kSolveWarps), 8), 32 * kSolveWarps, 0, s>>>(
+            b.d_probs, b.d_state, b.d_part, b.d_gs, b.d_y, b.nprob);
+    else
+        solve_kernel<32, kMaxSpace + 1><<<stride_grid(h->device, (b.nprob + kSolveWarps - 1) / kSolveWarps, 8), 32 * kSolveWarps, 0, s>>>(
+            b.d_probs, b.d_state, b.d_part, b.d_gs, b.d_y, b.nprob);
     IFCI_LAUNCH_CHECK(h);
     (small ? residual_kernel<kSmallSpace> : residual_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(
         b.d_probs, b.d_state, b.d_vitems, b.d_y, b.max_space, b.d_part, nitem);

@@ -145,10 +145,10 @@ __device__ __forceinline__ void psp_jacobi_cyclic(double *A, double *V, int P, d
         for (int pp = 0; pp < P - 1; pp++)
             for (int q = pp + 1; q < P; q++) {
                 const double apq = A[pp * LD + q];
-                if (fabs(apq) < 1e-300) continue;
+                if (dmag(apq) < dbits(1e-300)) continue;
                 const double app = A[pp * LD + pp], aqq = A[q * LD + q];
                 __syncwarp();   // every lane has read the rotation's entries
-                if (fabs(apq) <= 1e-18 * (fabs(app) + fabs(aqq))) {
+                if (jacobi_negligible(app, aqq, apq)) {
                     if (lane == 0) A[pp * LD + q] = A[q * LD + pp] = 0.0;
                     __syncwarp();
                     continue;
@@ -232,9 +232,9 @@ __device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, do
                 const int pp = min(a, b), q = max(a, b);
                 const double apq = A[pp * LD + q];
                 int rot = 0;
-                if (!(fabs(apq) < 1e-300)) {
+                if (dmag(apq) >= dbits(1e-300)) {
                     const double app = A[pp * LD + pp], aqq = A[q * LD + q];
-                    if (fabs(apq) <= 1e-18 * (fabs(app) + fabs(aqq))) {
+                    if (jacobi_negligible(app, aqq, apq)) {
                         A[pp * LD + q] = A[q * LD + pp] = 0.0;
                     } else {
                         double c, sn;

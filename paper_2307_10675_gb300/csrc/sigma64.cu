@@ -53,10 +53,6 @@ __host__ __device__ inline int fit64(int nstr, int np, int nexc, long long cap) 
     return (int)kb;
 }
 
-__device__ __forceinline__ double flip(double x, uint32_t neg) {   // neg: 0 or 0x80000000
-    return __hiloint2double(__double2hiint(x) ^ (int)neg, __double2loint(x));
-}
-
 __device__ __forceinline__ void sigma64_body(const SigmaProb &p, int ka, int cap) {
     extern __shared__ double sm[];
     __shared__ double lv[kList];
@@ -116,7 +112,7 @@ __device__ __forceinline__ void sigma64_body(const SigmaProb &p, int ka, int cap
             const int32_t x = exc[(size_t)ka * nexc + k0 + k];
             const uint32_t neg = (uint32_t)(x & 1) << 31;
             const double *src = c + (long long)exc_J(x) * nstr, *v = p.eri + (long long)exc_pair(x) * np;
-            for (int i = t; i < nstr; i += nt) Cs[(size_t)k * nstr + i] = flip(src[i], neg);
+            for (int i = t; i < nstr; i += nt) Cs[(size_t)k * nstr + i] = dflip(src[i], neg);
             for (int A = t; A < np; A += nt) Vs[A * ldv + k] = v[A];
         }
         __syncthreads();
@@ -127,8 +123,8 @@ __device__ __forceinline__ void sigma64_body(const SigmaProb &p, int ka, int cap
             for (int e = 0; e < nexc; e++) {
                 const int32_t x = eb[e];
                 const uint32_t neg = (uint32_t)(x & 1) << 31;
-                a0 = flip(a0, cur ^ neg);
-                a1 = flip(a1, cur ^ neg);
+                a0 = dflip(a0, cur ^ neg);
+                a1 = dflip(a1, cur ^ neg);
                 cur = neg;
                 const double *v = Vs + exc_pair(x) * ldv, *cs = Cs + exc_J(x);
                 int k = 0;
@@ -139,7 +135,7 @@ __device__ __forceinline__ void sigma64_body(const SigmaProb &p, int ka, int cap
                 }
                 if (k < kn) a0 = fma(v[k], cs[(size_t)k * nstr], a0);
             }
-            acc[ib] += flip(a0, cur) + flip(a1, cur);
+            acc[ib] += dflip(a0, cur) + dflip(a1, cur);
         }
     }
     if (rows)
