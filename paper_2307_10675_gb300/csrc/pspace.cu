@@ -107,15 +107,18 @@ __global__ void __launch_bounds__(kSelThreads) psp_select_kernel(const DavProb *
 }
 
 // Row-cyclic Jacobi on the symmetric P x P matrix A (shared memory, row
-// stride LD) by one warp: every lane derives the same rotation from the
-// settled entries, then rotates the columns of its rows, and after a warp
-// barrier its columns' rows and V.  Sweeps end once the off-diagonal part is
-// below 1e-26 of |A|_F^2 (a start guess needs no more); a rotation whose A_pq
-// is below 1e-18 (|A_pp| + |A_qq|) only sets A_pq = A_qp = 0.  Zero couplings
+// stride LD), in two forms.  Sweeps end once the off-diagonal part is below
+// 1e-26 of |A|_F^2 (a start guess needs no more); a rotation whose A_pq is
+// below 1e-18 (|A_pp| + |A_qq|) only sets A_pq = A_qp = 0.  Zero couplings
 // (other sectors, pair functions beyond a double excitation apart) are skipped.
-// The chain of dependent FP64 operations of one rotation bounds it; one warp
-// pays that chain once where a block of two warps paid it twice and three
-// block barriers with it.
+// The order of rotations and every rounding are those of one rotation at a
+// time: columns p, q <- fma(c, a_p, -(s a_q)), fma(s, a_p, c a_q), then rows,
+// then V, whoever computes them.
+//
+// One warp: every lane derives the same rotation from the settled entries, then
+// rotates the columns of its rows, and after a warp barrier its columns' rows
+// and V.  The chain of dependent FP64 operations of one rotation bounds it.
+// Serves the small blocks of sectored spaces, sixteen to an SM.
 template <int MAXP>
 __device__ __forceinline__ void psp_jacobi_cyclic(double *A, double *V, int P, double *red, double *red2) {
     constexpr int LD = MAXP + 1, R = (MAXP + 31) / 32;
@@ -177,6 +180,170 @@ __device__ __forceinline__ void psp_jacobi_cyclic(double *A, double *V, int P, d
                 }
                 __syncwarp();
             }
+    }
+}
+
+// bar.sync and bar.arrive on a numbered barrier of all kPairThreads threads
+constexpr int kPairThreads = 160;
+__device__ __forceinline__ void pair_sync(int id) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kPairThreads) : "memory");
+}
+__device__ __forceinline__ void pair_arrive(int id) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kPairThreads) : "memory");
+}
+
+// Five warps: one derives the rotations, four apply them.  An SM sub-partition's
+// FP64 pipe takes 64 clk for a warp instruction however few lanes are in it, so
+// what bounds a rotation is the chain from its 2 x 2 block to the next one.
+// The deriving warp therefore runs ahead: from the rows p and q as they stand
+// before rotation (p, q) it computes row p and A_pp after it, which with the
+// untouched diagonal is all that (p, q + 1) needs, while the four warps rotate
+// A and V.  Where that does not find the next rotation (the end of a row, or an
+// entry to be set to zero) it scans A.
+// The others: lane l the p and lane l + 16 the q element of one row, then of
+// one column, then of one row of V, a multiply and an FMA each.  Only the 2 x 2
+// block needs both mixes of A; its rows and columns belong to one warp, so no
+// barrier is needed between.
+// Barrier 1: a rotation is applied to A (the four arrive, the deriving warp
+// waits); barrier 2: the next one is in shared memory (it arrives, they wait).
+template <int MAXP>
+__device__ __forceinline__ void psp_jacobi_ahead(double *A, double *V, int P, double *red, double *red2) {
+    static_assert(MAXP == 64, "sixteen rows to each of four warps");
+    constexpr int LD = MAXP + 1;
+    __shared__ double rot_c, rot_s;
+    __shared__ int rot_p, rot_q;                   // rot_q < 0: the sweep is over
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, half = lane >> 4;
+    for (int sweep = 0; sweep < 40; sweep++) {
+        if (t < P) {
+            double off = 0.0, all = 0.0;
+            for (int c = 0; c < P; c++) {
+                const double a2 = A[t * LD + c] * A[t * LD + c];
+                all += a2;
+                if (c != t) off += a2;
+            }
+            red[t] = off;
+            red2[t] = all;
+        }
+        __syncthreads();
+        const double *part = lane & 1 ? red2 : red;   // even lanes add up the off-diagonal part, odd lanes all
+        double sum = 0.0;
+        for (int i = 0; i < P; i++) sum += part[i];
+        const double tot = __shfl_sync(0xffffffffu, sum, 0), fro = __shfl_sync(0xffffffffu, sum, 1);
+        __syncthreads();
+        if (tot <= 1e-26 * fro || tot == 0.0) break;
+        if (warp == 4) {
+            int p = 0, q = 0, nq = -1;             // the last rotation; nq >= 0: the next one is (p, nq)
+            bool applied = true;                   // A has had the last one
+            double app = 0.0, aqq = 0.0, apq = 0.0;
+            while (true) {
+                if (nq < 0) {
+                    if (!applied) pair_sync(1);
+                    applied = true;
+                    int sp = p, sq = q + 1;
+                    while (sp < P - 1) {
+                        // first coupling of row sp from column sq on that is not zero
+                        int f = P;
+                        for (int c0 = sq; c0 < P; c0 += 32) {
+                            const bool nz = c0 + lane < P && dmag(A[sp * LD + c0 + lane]) >= dbits(1e-300);
+                            const unsigned m = __ballot_sync(0xffffffffu, nz);
+                            if (m) {
+                                f = c0 + __ffs(m) - 1;
+                                break;
+                            }
+                        }
+                        if (f >= P) {
+                            sp++;
+                            sq = sp + 1;
+                            continue;
+                        }
+                        apq = A[sp * LD + f];
+                        app = A[sp * LD + sp];
+                        aqq = A[f * LD + f];
+                        if (!jacobi_negligible(app, aqq, apq)) {
+                            p = sp;
+                            nq = f;
+                            break;
+                        }
+                        __syncwarp();
+                        if (lane == 0) A[sp * LD + f] = A[f * LD + sp] = 0.0;
+                        __syncwarp();
+                        sq = f + 1;
+                    }
+                    if (nq < 0) {
+                        if (lane == 0) rot_q = -1;
+                        __syncwarp();
+                        pair_arrive(2);
+                        break;
+                    }
+                }
+                double c, s;
+                jacobi_rotation(app, aqq, apq, c, s);
+                if (jacobi_negligible(app, aqq, apq)) {   // found ahead, but to be set to zero
+                    nq = -1;
+                    continue;
+                }
+                q = nq;
+                if (!applied) pair_sync(1);
+                if (lane == 0) {
+                    rot_p = p;
+                    rot_q = q;
+                    rot_c = c;
+                    rot_s = s;
+                }
+                const int col = q + 1 + lane;
+                const bool in = col < P;
+                const double rp = in ? A[p * LD + col] : 0.0, rq = in ? A[q * LD + col] : 0.0;
+                const double dg = in ? A[col * LD + col] : 0.0, aqp = A[q * LD + p];
+                const double ms = dflip(s, 0x80000000u);
+                // columns p of rows p and q, then row p; row p at the columns ahead
+                const double xp = __fma_rn(c, app, __dmul_rn(ms, apq)), yp = __fma_rn(c, aqp, __dmul_rn(ms, aqq));
+                const double row = __fma_rn(c, rp, __dmul_rn(ms, rq));
+                app = __fma_rn(c, xp, __dmul_rn(ms, yp));
+                const unsigned m = __ballot_sync(0xffffffffu, in && dmag(row) >= dbits(1e-300));
+                nq = m ? q + __ffs(m) : -1;
+                apq = __shfl_sync(0xffffffffu, row, __ffs(m) - 1);
+                aqq = __shfl_sync(0xffffffffu, dg, __ffs(m) - 1);
+                pair_arrive(2);
+                applied = false;
+            }
+        } else {
+            while (true) {
+                pair_sync(2);
+                const int q = rot_q, p = rot_p;
+                if (q < 0) break;
+                const double c = rot_c, s = rot_s;
+                const double x = half ? s : c, y = half ? c : dflip(s, 0x80000000u);
+                // slots 0 and 1 hold rows (columns) p and q, whose own slots get 0 and 1
+                const int slot = 16 * warp + (lane & 15);
+                int r = slot == 1 ? q : slot == q ? 1 : slot;
+                r = r == 0 ? p : r == p ? 0 : r;
+                const bool on = r < P;
+                double ap = 0.0, aq = 0.0;
+                if (on) {
+                    ap = A[r * LD + p];
+                    aq = A[r * LD + q];
+                }
+                __syncwarp();
+                if (on) A[r * LD + (half ? q : p)] = __fma_rn(x, ap, __dmul_rn(y, aq));
+                __syncwarp();
+                if (on) {
+                    ap = A[p * LD + r];
+                    aq = A[q * LD + r];
+                }
+                __syncwarp();
+                if (on) A[(half ? q : p) * LD + r] = __fma_rn(x, ap, __dmul_rn(y, aq));
+                __syncwarp();
+                pair_arrive(1);
+                if (slot < P) {
+                    ap = V[slot * LD + p];
+                    aq = V[slot * LD + q];
+                }
+                __syncwarp();
+                if (slot < P) V[slot * LD + (half ? q : p)] = __fma_rn(x, ap, __dmul_rn(y, aq));
+                __syncwarp();
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -291,15 +458,17 @@ __device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, do
 // eigenvectors, written to the start slots 0..nv-1; the random start vector is
 // cleared on the P-space determinants.
 //
-// NT = 256 runs the round-robin sweeps, NT = 32 the cyclic ones.  The round-robin
-// order is the faster one for a 64-function problem (21.8 ms with one rotation at
-// a time on 64 threads, 3.5 ms) and serves the whole spaces of an FP64 solve,
-// where a last-bit change of the start vector stays one.  With a quantised
-// contraction (FP64E and the mixed modes that end on it) such a change turns up
-// at the contraction's own level, ~5e-11 Eh, so those solves keep the order of
-// rotations, and with it every bit of their start vectors (an expansion of 298
-// sets: 68.6 ms of P-space solves before, 64.0 ms on one warp each).  So do the blocks of sectored spaces (MAXP = 24), which come by the
-// hundred thousand and share an SM sixteen at a time.
+// NT = 256 runs the round-robin sweeps, the others the cyclic ones.  The
+// round-robin order is the faster one for a 64-function problem (2.2 ms, against
+// 20.1 ms with one rotation at a time) and serves the whole spaces of an FP64
+// solve, where a last-bit change of the start vector stays one.  With a
+// quantised contraction (FP64E and the mixed modes that end on it) such a change
+// turns up at the contraction's own level, ~5e-11 Eh, so those solves keep the
+// order of rotations, and with it every bit of their start vectors, on five
+// warps a problem: 64 functions 20.1 ms on one warp, 13.8 ms; 298 such problems
+// at once 21.9 ms, 15.7 ms; the P-space solves of an expansion of 298 sets
+// 58.9 ms, 42.9 ms.  So do the blocks of sectored spaces (MAXP = 24), which come
+// by the hundred thousand and share an SM sixteen at a time, a warp each.
 template <int MAXP, int NT>
 __device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict__ probs, const HdiagDesc *__restrict__ hdd, const long long *__restrict__ pidx,
                  const int *__restrict__ pcount, int max_space, double *__restrict__ blk_energy, int w_) {
@@ -371,6 +540,7 @@ __device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict_
     }
     __syncthreads();
     if constexpr (NT == 32) psp_jacobi_cyclic<MAXP>(A, V, P, red, red2);
+    else if constexpr (NT == kPairThreads) psp_jacobi_ahead<MAXP>(A, V, P, red, red2);
     else psp_jacobi_pairs<MAXP, NT>(A, V, P, red, red2);
     __syncthreads();
     int nv, ns;
@@ -556,9 +726,9 @@ int launch_pspace_start(ifci_handle_t h, const DavBatch &b, const HdiagDesc *d_h
         IFCI_LAUNCH_CHECK(h);
     } else if (whole) {
         static SmemOptIn opt;
-        IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel<kPsp, 32>, smem));
+        IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel<kPsp, kPairThreads>, smem));
         ProfScope ps(h, s, PK_PSPACE);
-        psp_solve_kernel<kPsp, 32><<<stride_grid(h->device, b.nprob, 3), 32, smem, s>>>(
+        psp_solve_kernel<kPsp, kPairThreads><<<stride_grid(h->device, b.nprob, 3), kPairThreads, smem, s>>>(
             b.d_probs, d_hd, pidx, pcount, b.max_space, b.d_blk_energy, b.nprob);
         IFCI_LAUNCH_CHECK(h);
     }
