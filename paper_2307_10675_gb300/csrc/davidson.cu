@@ -321,24 +321,129 @@ __device__ void jacobi_warp(double *A, double *V, int k, int lane) {
     }
 }
 
-// G lanes per problem: finish the subspace column and solve the projected
-// problem (its kKeep lowest Ritz pairs).  `i` = the group's problem, -1: none.
+// The same by four warps in round-robin order: a step rotates up to k / 2
+// disjoint index pairs at once, each derived by its own lane of warp 0, and a
+// sweep is k - 1 (k even) such steps instead of k (k - 1) / 2 dependent
+// rotations.  Within a step every (pair, row) and then every (pair, column) of A
+// is one lane's two multiplies and two FMAs; the (pair, row)s of V follow while
+// the next step's rotations are derived (those of step `step` in buffer step & 1).
+// The chain of a step (~1200 clk to derive, 2 x 256 to mix) bounds it: 32 problems
+// of up to 12 vectors take 62 us on average, 194 us one rotation at a time.  Only
+// FP64 solves take it: with a quantised sigma another rounding here turns up at
+// the contraction's own level (energies of selected spaces moved by 7e-10 of
+// themselves), so those keep the serial order and every bit.
+constexpr int kPairSolveThreads = 128;
+
+template <int LD>
+__device__ void jacobi_pairs(double *A, double *V, int k) {
+    constexpr int NT = kPairSolveThreads, NP = LD / 2;
+    __shared__ double rc[2][NP], rs[2][NP], red[2][NT / 32];
+    __shared__ int rp[2][NP], rq[2][NP];   // the step's index pairs; rq < 0: no rotation
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int e = t; e < k * k; e += NT) V[e / k * LD + e % k] = e / k == e % k ? 1.0 : 0.0;
+    __syncthreads();
+    const int n = k + (k & 1), npr = n / 2;
+    const int i0 = k ? t / k : 0, r0 = t - i0 * k, di = k ? NT / k : 0, dr = NT - di * k;   // items t, t + NT, ... = (i, r)
+    const int j0 = k ? (t - 32) / k : 0, s0 = t - 32 - j0 * k, dj = k ? (NT - 32) / k : 0, ds = NT - 32 - dj * k;
+    for (int sweep = 0; sweep < 60 && k > 1; sweep++) {
+        double off = 0.0, tot = 0.0;
+        for (int e = t; e < k * k; e += NT) {
+            const double a = A[e / k * LD + e % k];
+            tot += a * a;
+            if (e / k != e % k) off += a * a;
+        }
+        off = warp_sum(off);
+        tot = warp_sum(tot);
+        if (lane == 0) {
+            red[0][warp] = off;
+            red[1][warp] = tot;
+        }
+        __syncthreads();
+        off = (red[0][0] + red[0][1]) + (red[0][2] + red[0][3]);
+        tot = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
+        if (off <= 1e-26 * tot || off == 0.0) break;
+        for (int step = 0; step < n; step++) {   // the last one only finishes V
+            const int cur = step & 1;
+            if (warp == 0) {
+                if (lane < npr && step < n - 1) {
+                    // index n - 1 stays, the others turn
+                    const int a = lane == 0 ? n - 1 : (step + lane) % (n - 1);
+                    const int b = lane == 0 ? step : (step + n - 1 - lane) % (n - 1);
+                    const int p = min(a, b), q = max(a, b);
+                    bool rot = false;
+                    if (q < k) {
+                        const double apq = A[p * LD + q], app = A[p * LD + p], aqq = A[q * LD + q];
+                        if ((dbits(apq) << 1) != 0) {   // not +-0
+                            rot = !jacobi_negligible(app, aqq, apq);
+                            if (rot) {
+                                double c, sn;
+                                jacobi_rotation(app, aqq, apq, c, sn);
+                                rc[cur][lane] = c;
+                                rs[cur][lane] = sn;
+                            } else {
+                                A[p * LD + q] = A[q * LD + p] = 0.0;
+                            }
+                        }
+                    }
+                    rp[cur][lane] = p;
+                    rq[cur][lane] = rot ? q : -1;
+                }
+            } else if (step > 0) {
+                for (int i = j0, r = s0; i < npr; i += dj, r += ds) {
+                    if (r >= k) {
+                        r -= k;
+                        if (++i >= npr) break;
+                    }
+                    const int p = rp[cur ^ 1][i], q = rq[cur ^ 1][i];
+                    if (q < 0) continue;
+                    const double c = rc[cur ^ 1][i], sn = rs[cur ^ 1][i], vp = V[r * LD + p], vq = V[r * LD + q];
+                    V[r * LD + p] = c * vp - sn * vq;
+                    V[r * LD + q] = sn * vp + c * vq;
+                }
+            }
+            __syncthreads();
+            if (step == n - 1) break;
+            for (int i = i0, r = r0; i < npr; i += di, r += dr) {
+                if (r >= k) {
+                    r -= k;
+                    if (++i >= npr) break;
+                }
+                const int p = rp[cur][i], q = rq[cur][i];
+                if (q < 0) continue;
+                const double c = rc[cur][i], sn = rs[cur][i], ap = A[r * LD + p], aq = A[r * LD + q];
+                A[r * LD + p] = c * ap - sn * aq;
+                A[r * LD + q] = sn * ap + c * aq;
+            }
+            __syncthreads();
+            for (int i = i0, r = r0; i < npr; i += di, r += dr) {
+                if (r >= k) {
+                    r -= k;
+                    if (++i >= npr) break;
+                }
+                const int p = rp[cur][i], q = rq[cur][i];
+                if (q < 0) continue;
+                const double c = rc[cur][i], sn = rs[cur][i], ap = A[p * LD + r], aq = A[q * LD + r];
+                A[p * LD + r] = c * ap - sn * aq;
+                A[q * LD + r] = sn * ap + c * aq;
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// G lanes per problem: finish the subspace column of k = newest + 1 vectors
+// and fill A with the projected matrix.
 template <int G, int LD>
-__device__ __forceinline__ void solve_body(const DavProb *__restrict__ probs, DavState *__restrict__ st,
-                                           const double *__restrict__ part, double *__restrict__ gs,
-                                           double *__restrict__ ys, int i, double *A, double *V) {
+__device__ __forceinline__ void solve_load(const DavProb *__restrict__ probs, const double *__restrict__ part,
+                                           double *__restrict__ gs, int i, int k, double *A) {
     const int lane = threadIdx.x & (G - 1);
-    DavState s{};
-    if (i >= 0) s = st[i];
-    const bool on = i >= 0 && s.active;
-    const int k = on ? s.newest + 1 : 0;
     if (lane < k) {
         const DavProb &p = probs[i];
         double *Gm = gs + (long long)i * kMaxSpace * kMaxSpace;
         double v = 0.0;
         for (int w = 0; w < p.nitem; w++) v += part[(long long)(p.item0 + w) * kNP + lane];
-        Gm[lane * kMaxSpace + s.newest] = v;
-        Gm[s.newest * kMaxSpace + lane] = v;
+        Gm[lane * kMaxSpace + k - 1] = v;
+        Gm[(k - 1) * kMaxSpace + lane] = v;
     }
     __syncwarp();
     if (lane < k) {
@@ -346,7 +451,14 @@ __device__ __forceinline__ void solve_body(const DavProb *__restrict__ probs, Da
         for (int b = 0; b < k; b++) A[lane * LD + b] = 0.5 * (Gm[lane * kMaxSpace + b] + Gm[b * kMaxSpace + lane]);
     }
     __syncwarp();
-    jacobi_warp<G, LD>(A, V, k, lane);
+}
+
+// G lanes per problem: the kKeep lowest Ritz pairs from the diagonal of A and
+// the columns of V.
+template <int G, int LD>
+__device__ __forceinline__ void solve_store(DavState *__restrict__ st, double *__restrict__ ys, int i, bool on, int k,
+                                            const double *A, const double *V) {
+    const int lane = threadIdx.x & (G - 1);
     // the lowest eigenpairs in ascending order (ties by index), lane j ranking
     // eigenvalue j and writing its vector; each vector's largest component made
     // positive (deterministic sign)
@@ -373,12 +485,43 @@ __device__ __forceinline__ void solve_body(const DavProb *__restrict__ probs, Da
                 yo[rank * kNP + kMaxSpace] = e;
                 if (rank == 0) {
                     st[i].theta = e;
-                    st[i].iters = s.iters + 1;
+                    st[i].iters++;
                 }
             }
         }
     }
+}
+
+// G lanes per problem.  `i` = the group's problem, -1: none.
+template <int G, int LD>
+__device__ __forceinline__ void solve_body(const DavProb *__restrict__ probs, DavState *__restrict__ st,
+                                           const double *__restrict__ part, double *__restrict__ gs,
+                                           double *__restrict__ ys, int i, double *A, double *V) {
+    const bool on = i >= 0 && st[i].active;
+    const int k = on ? st[i].newest + 1 : 0;
+    solve_load<G, LD>(probs, part, gs, i, k, A);
+    jacobi_warp<G, LD>(A, V, k, threadIdx.x & (G - 1));
+    solve_store<G, LD>(st, ys, i, on, k, A, V);
     __syncwarp();   // A and V are reused by the warp's next problem
+}
+
+// One problem per block, rotations in round-robin order.
+__global__ void __launch_bounds__(kPairSolveThreads) solve_pairs_kernel(const DavProb *__restrict__ probs,
+                                                                        DavState *__restrict__ st,
+                                                                        const double *__restrict__ part,
+                                                                        double *__restrict__ gs,
+                                                                        double *__restrict__ ys, int nprob_) {
+    constexpr int LD = kMaxSpace + 1;
+    __shared__ double A[kMaxSpace * LD], V[kMaxSpace * LD];
+    for (int i = blockIdx.x; i < nprob_; i += gridDim.x) {
+        if (!st[i].active) continue;
+        const int k = st[i].newest + 1;
+        if (threadIdx.x < 32) solve_load<32, LD>(probs, part, gs, i, k, A);
+        __syncthreads();
+        jacobi_pairs<LD>(A, V, k);
+        if (threadIdx.x < 32) solve_store<32, LD>(st, ys, i, true, k, A, V);
+        __syncthreads();   // A and V are reused by the next problem
+    }
 }
 
 template <int G, int LD>
@@ -938,7 +1081,10 @@ static int dav_step(ifci_handle_t h, DavBatch &b, SigmaPlan &hi_plan, SigmaPlan 
     const bool small = b.max_space <= kSmallSpace;
     (small ? dots_kernel<kSmallSpace> : dots_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_part, nitem);
     IFCI_LAUNCH_CHECK(h);
-    if (b.max_space <= 16)
+    if (b.precision == IFCI_FP64)
+        solve_pairs_kernel<<<stride_grid(h->device, b.nprob, 16), kPairSolveThreads, 0, s>>>(b.d_probs, b.d_state, b.d_part,
+                                                                                     b.d_gs, b.d_y, b.nprob);
+    else if (b.max_space <= 16)
         solve_kernel<16, 17><<<stride_grid(h->device, (b.nprob + 2 * kSolveWarps - 1) / (2 * kSolveWarps), 8), 32 * kSolveWarps, 0, s>>>(
             b.d_probs, b.d_state, b.d_part, b.d_gs, b.d_y, b.nprob);
     else
