@@ -87,20 +87,24 @@ int ifci_sigma(ifci_handle_t h, const ifci_strings_t *str, const double *h1, con
     int32_t *pmap = sym && tc ? ws_take<int32_t>(h, (size_t)nstr * pmap_ld(np)) : nullptr;
     plan.probs[0].pmap = pmap;
     FoldDesc f{n, 2 * str->nelec_spin, ld, h1, eri, W};
+    void *D, *G;
+    if (oz) {
+        unsigned long long *mx = ws_take<unsigned long long>(h, 2);
+        IFCI_TRY(upload_plan(h, plan, s));
+        D = ws_take<char>(h, (size_t)delems_D * eb);
+        G = ws_take<char>(h, (size_t)plan.max_delems * eb);
+        if (!D || !G || !mx) return set_error(h, IFCI_ERR_OOM, "ifci_sigma: workspace");
+        return run_sigma_oz_one(h, plan, f, c, jmap, mx, D, G, s);
+    }
     IFCI_CUDA_TRY(h, cudaMemcpyAsync(fd, &f, sizeof(f), cudaMemcpyHostToDevice, s));
     IFCI_TRY(launch_fold(h, 1, fd, np, s));
     if (blk) IFCI_TRY(launch_exc_blocks(h, nstr, nexc, str->exc, blk, s));
     if (pmap) IFCI_TRY(launch_pair_map(h, nstr, nexc, np, str->exc, pmap, s));
-    if (jmap) IFCI_TRY(launch_oz_map(h, nstr, nexc, np, str->exc, jmap, s));
     IFCI_TRY(upload_plan(h, plan, s));
     if (precision == IFCI_FP32) IFCI_TRY(launch_convert_w(h, 1, plan.d_probs, s));
     if (tc) IFCI_TRY(launch_tc_pack_w(h, 1, plan.d_probs, precision, s));
-    if (oz) {
-        IFCI_TRY(launch_oz_pack_w(h, 1, plan.d_probs, np, s));
-        IFCI_TRY(launch_oz_dscale(h, plan.d_probs, c, ndet, s));
-    }
-    void *D = ws_take<char>(h, (size_t)delems_D * eb);
-    void *G = ws_take<char>(h, (size_t)plan.max_delems * eb);
+    D = ws_take<char>(h, (size_t)delems_D * eb);
+    G = ws_take<char>(h, (size_t)plan.max_delems * eb);
     if (!D || !G) return set_error(h, IFCI_ERR_OOM, "ifci_sigma: workspace");
     return run_sigma(h, plan, precision, D, G, s);
 }

@@ -2,7 +2,7 @@
 // diagonal <I|H|I> and the reference energy.
 #include <algorithm>
 
-#include "hamiltonian.cuh"
+#include "fold.cuh"
 
 namespace ifci {
 
@@ -66,30 +66,12 @@ __global__ void fold_kernel(const FoldDesc *__restrict__ desc) {
     const FoldDesc d = desc[blockIdx.x];
     const int n = d.n, np = n * (n + 1) / 2, ld = d.ld;
     extern __shared__ double kpair[];  // [np]
-    for (int A = threadIdx.x; A < np; A += blockDim.x) {
-        int P = 0;
-        while ((P + 1) * (P + 2) / 2 <= A) P++;
-        int Q = A - P * (P + 1) / 2;
-        double k = d.h1[P * n + Q];
-        for (int r = 0; r < n; r++) k -= 0.5 * d.eri[(long long)pair_of(P, r) * np + pair_of(r, Q)];
-        kpair[A] = k;
-    }
+    for (int A = threadIdx.x; A < np; A += blockDim.x) kpair[A] = fold_pair(d, A);
     __syncthreads();
     const double invN = d.nelec > 0 ? 1.0 / (double)d.nelec : 0.0;
     for (long long t = blockIdx.y * blockDim.x + threadIdx.x; t < (long long)ld * ld; t += (long long)gridDim.y * blockDim.x) {
-        int A = (int)(t / ld), B = (int)(t % ld);
-        double w = 0.0;
-        if (A < np && B < np) {
-            int P = 0;
-            while ((P + 1) * (P + 2) / 2 <= A) P++;
-            int R = 0;
-            while ((R + 1) * (R + 2) / 2 <= B) R++;
-            bool dA = (A - P * (P + 1) / 2) == P, dB = (B - R * (R + 1) / 2) == R;
-            w = d.eri[(long long)A * np + B];
-            if (dB) w += invN * kpair[A];
-            if (dA) w += invN * kpair[B];
-            w *= 0.5;
-        }
+        const int A = (int)(t / ld), B = (int)(t % ld);
+        const double w = A < np && B < np ? fold_element(d, kpair, invN, A, B) : 0.0;
         d.W[t] = w;
     }
 }

@@ -130,8 +130,12 @@ bool oz_supported(int np, int nstr, int nexc);
 bool oz_wide(int nexc);
 int launch_oz_map(ifci_handle_t h, int nstr, int nexc, int np, const int32_t *exc, uint16_t *jmap, cudaStream_t s);
 int launch_oz_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, int max_np, cudaStream_t s);
-int launch_oz_dscale(ifci_handle_t h, SigmaProb *d_prob, const double *c, long long n, cudaStream_t s);
 int run_sigma_oz(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, void *D, void *G, cudaStream_t s);
+// The one problem of a plan, from its integrals and the caller's vector: builds
+// W, its image, the excitation map and the scales (mx: two words of scratch) too.
+struct FoldDesc;
+int run_sigma_oz_one(ifci_handle_t h, const SigmaPlan &plan, const FoldDesc &f, const double *c, uint16_t *jmap,
+                     unsigned long long *mx, void *D, void *G, cudaStream_t s);
 
 // tensor-core contraction (sigma_tc.cu)
 int tc_supported(int precision);

@@ -66,6 +66,8 @@
 
 #include <algorithm>
 
+#include "fold.cuh"
+#include "fp64int.cuh"
 #include "sigma.cuh"
 #include "tcgen05.cuh"
 
@@ -104,6 +106,24 @@ __device__ __forceinline__ void slice5(double x, float (&sl)[kS]) {
         double q = rint(r);
         sl[i] = (float)q;
         r = (r - q) * 256.0;
+    }
+}
+
+// The same for w / 2^e, |w| < 2^e, on the integer pipe (an FP64 instruction
+// takes a sub-partition 64 to 104 clk, a division 564): w 2^(59 - e) with a
+// sticky lowest bit, its digits rounded to nearest even one by one as rint does.
+__device__ __forceinline__ void slice5_pow2(double w, int e, float (&sl)[kS]) {
+    const int f = dexp_field(w);
+    const long long mant = (dbits(w) & 0xFFFFFFFFFFFFFll) | (f ? 1ll << 52 : 0ll);
+    const int sh = (f ? f : 1) - 1075 - e + 59;   // <= 6
+    long long x = sh >= 0 ? mant << sh : sh > -63 ? (mant >> -sh) | ((mant & ((1ll << -sh) - 1)) != 0) : mant != 0;
+    if (dbits(w) < 0) x = -x;
+#pragma unroll
+    for (int i = 0; i < kS; i++) {
+        const int b = 52 - 8 * i;
+        const long long half = 1ll << (b - 1), q = (x + half - 1 + (x >> b & 1)) >> b;
+        sl[i] = (float)(int)q;
+        x -= q << b;
     }
 }
 
@@ -650,18 +670,14 @@ oz_sigma_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict_
 // at [(t 2 + s) kS + j][nstr][row_ld] holds digit j (0 = most significant) of
 // +-round(c 2^38 / dscale); pass 1 (only without spin-flip symmetry) is C^T.
 // Clears the problem's S as well.
-__global__ void __launch_bounds__(kGatherChunk)
-oz_quantise_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items, __half *__restrict__ Q,
-                   long long *__restrict__ S) {
-    const WorkItem it = items[blockIdx.x];
-    const SigmaProb &p = probs[it.prob];
-    if (p.active && !*p.active) return;
-    const long long I = it.start + threadIdx.x;
-    if (I >= p.ndet) return;
+__device__ __forceinline__ void quantise_one(const SigmaProb &p, long long I, double dscale, __half *__restrict__ Q,
+                                             long long *__restrict__ S) {
     const int nstr = p.nstr, ldq = row_ld(nstr);
     const int ka = (int)(I / nstr), kb = (int)(I % nstr);
     const double *c = p.cbase + (p.cslot ? (long long)*p.cslot : 0ll) * p.stride;
-    const double sc = 274877906944.0 / p.dscale;   // 2^38 / dscale
+    // 2^38 / dscale: exact on the integer pipe while both are normal powers of two
+    const int f = dexp_field(dscale);
+    const double sc = f > 38 && f < 2047 ? __hiloint2double((2046 + 38 - f) << 20, 0) : 274877906944.0 / dscale;
     const size_t plane = (size_t)nstr * ldq;
     unsigned short *out = reinterpret_cast<unsigned short *>(Q) + p.qoff + (size_t)ka * ldq + kb;
     for (int t = 0; t < (p.sym ? 1 : 2); t++) {
@@ -677,6 +693,16 @@ oz_quantise_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restri
         out += 2 * kS * plane;
         S[p.doff + (t ? p.ndet : 0) + I] = 0;
     }
+}
+
+__global__ void __launch_bounds__(kGatherChunk)
+oz_quantise_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ items, __half *__restrict__ Q,
+                   long long *__restrict__ S) {
+    const WorkItem it = items[blockIdx.x];
+    const SigmaProb &p = probs[it.prob];
+    if (p.active && !*p.active) return;
+    const long long I = it.start + threadIdx.x;
+    if (I < p.ndet) quantise_one(p, I, p.dscale, Q, S);
 }
 
 // sigma = S + S^T (spin-flip-symmetric) or S(C) + S(C^T)^T, converted from the
@@ -741,52 +767,63 @@ __global__ void __launch_bounds__(512) oz_wmax_kernel(const SigmaProb *__restric
 // Sliced image of W, MN-major: for each chunk of w = 48 output pairs (the last
 // one narrower, a multiple of 16) [contracted pair b][slice i][output pair of
 // the chunk] FP16, zeros beyond npair.  A sectored space packs its active
-// pairs only, in compact order.  Blocks (problem, part).
-__global__ void __launch_bounds__(256) oz_pack_w_kernel(const SigmaProb *__restrict__ probs) {
-    const SigmaProb &p = probs[blockIdx.x];
+// pairs only, in compact order.  Group t of 8 output pairs; scale = 2^e > max |W|.
+__device__ __forceinline__ void pack_group(const SigmaProb &p, int t, double scale) {
     const int np = p.act ? p.npc : p.np, npad = np_pad(np), n8 = npad / 8;
     const int32_t *act = p.act;
     uint8_t *img = (uint8_t *)const_cast<void *>(p.Woz);
-    const double scale = p.Wexp[0];
-    for (int t = blockIdx.y * 256 + threadIdx.x; t < np * n8; t += gridDim.y * 256) {
-        const int b = t / n8, a0 = t % n8 * 8, c0 = a0 / kNC * kNC, w = min(kNC, npad - c0);
-        const int kb = act ? act[b] : b;
-        float sl[8][kS];
-        for (int e = 0; e < 8; e++) {
-            const int a = a0 + e;
-            slice5(a < np ? p.W[(long long)(act ? act[a] : a) * p.ld + kb] / scale : 0.0, sl[e]);
-        }
-        for (int i = 0; i < kS; i++)
-            *(uint4 *)(img + (size_t)np * 10 * c0 + ((size_t)b * kS * w + i * w + (a0 - c0)) * 2) =
-                make_uint4(pack2(sl[0][i], sl[1][i]), pack2(sl[2][i], sl[3][i]), pack2(sl[4][i], sl[5][i]),
-                           pack2(sl[6][i], sl[7][i]));
+    const int b = t / n8, a0 = t % n8 * 8, c0 = a0 / kNC * kNC, w = min(kNC, npad - c0);
+    const int kb = act ? act[b] : b, f = dexp_field(scale);
+    float sl[8][kS];
+    for (int e = 0; e < 8; e++) {
+        const int a = a0 + e;
+        const double x = a < np ? p.W[(long long)(act ? act[a] : a) * p.ld + kb] : 0.0;
+        if (f > 0 && f < 2047 && dexp_field(x) < 2047) slice5_pow2(x, f - 1023, sl[e]);
+        else slice5(x / scale, sl[e]);
     }
+    for (int i = 0; i < kS; i++)
+        *(uint4 *)(img + (size_t)np * 10 * c0 + ((size_t)b * kS * w + i * w + (a0 - c0)) * 2) =
+            make_uint4(pack2(sl[0][i], sl[1][i]), pack2(sl[2][i], sl[3][i]), pack2(sl[4][i], sl[5][i]),
+                       pack2(sl[6][i], sl[7][i]));
+}
+
+// Blocks (problem, part).
+__global__ void __launch_bounds__(256) oz_pack_w_kernel(const SigmaProb *__restrict__ probs) {
+    const SigmaProb &p = probs[blockIdx.x];
+    const int np = p.act ? p.npc : p.np;
+    for (int t = blockIdx.y * 256 + threadIdx.x; t < np * (np_pad(np) / 8); t += gridDim.y * 256) pack_group(p, t, p.Wexp[0]);
 }
 
 // Excitation map of a string class: entry of output pair A and string I at
 // [A / 4][I][A % 4] (one 8-byte load per thread and four columns), sign << 15 | J
 // of E+_A |I> = +-|J>, kNoMap where there is none, beyond np and beyond nstr
-// (ldj strings, np_pad(np) pairs).
-__global__ void __launch_bounds__(128) oz_map_kernel(int nstr, int nexc, int np, int ldj, const int32_t *__restrict__ exc,
-                                                     uint16_t *__restrict__ jmap) {
-    // one thread per string: its list is sorted by pair
-    const int I = blockIdx.x * 128 + threadIdx.x;
-    if (I >= ldj) return;
-    const int32_t *row = exc + (size_t)I * nexc;
-    int e = 0;
-    int32_t x = I < nstr ? row[0] : -1;
-    for (int A0 = 0; A0 < np_pad(np); A0 += 4) {
-        uint32_t v[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            v[u] = kNoMap;
-            if (I < nstr && e < nexc && exc_pair(x) == A0 + u) {
-                v[u] = (uint32_t)exc_J(x) | (uint32_t)(x & 1) << 15;
-                if (++e < nexc) x = row[e];
-            }
-        }
-        reinterpret_cast<uint2 *>(jmap)[(size_t)(A0 >> 2) * ldj + I] = make_uint2(v[0] | v[1] << 16, v[2] | v[3] << 16);
+// (ldj strings, np_pad(np) pairs).  kMapRows strings, built in shared memory so
+// that the table is read and the map written in whole lines (220 strings of 30
+// entries: 11.4 us with one thread walking each list).
+constexpr int kMapRows = 32;
+
+__device__ __forceinline__ void map_rows(int I0, int nstr, int nexc, int np, int ldj, const int32_t *__restrict__ exc,
+                                         uint16_t *__restrict__ jmap, uint16_t (*tile)[kMaxNp + 2]) {
+    const int npad = np_pad(np), rows = min(kMapRows, nstr - I0);
+    for (int t = threadIdx.x; t < kMapRows * (npad / 2); t += 256)
+        *reinterpret_cast<uint32_t *>(&tile[t / (npad / 2)][2 * (t % (npad / 2))]) = kNoMap << 16 | kNoMap;
+    __syncthreads();
+    for (int t = threadIdx.x; t < rows * nexc; t += 256) {
+        const int32_t x = exc[(size_t)I0 * nexc + t];
+        tile[t / nexc][exc_pair(x)] = (uint16_t)((uint32_t)exc_J(x) | (uint32_t)(x & 1) << 15);
     }
+    __syncthreads();
+    for (int t = threadIdx.x; t < kMapRows * (npad / 4); t += 256) {
+        const int g = t / kMapRows, i = t % kMapRows;
+        const uint32_t *v = reinterpret_cast<const uint32_t *>(&tile[i][4 * g]);
+        reinterpret_cast<uint2 *>(jmap)[(size_t)g * ldj + I0 + i] = make_uint2(v[0], v[1]);
+    }
+}
+
+__global__ void __launch_bounds__(256) oz_map_kernel(int nstr, int nexc, int np, int ldj, const int32_t *__restrict__ exc,
+                                                     uint16_t *__restrict__ jmap) {
+    __shared__ __align__(8) uint16_t tile[kMapRows][kMaxNp + 2];
+    map_rows(blockIdx.x * kMapRows, nstr, nexc, np, ldj, exc, jmap, tile);
 }
 
 // maps of the sectored units: their class's map restricted to the active pairs
@@ -812,23 +849,81 @@ __global__ void __launch_bounds__(256) oz_compact_maps_kernel(const OzMapDesc *_
     }
 }
 
-// dscale of a caller's vector: the smallest power of two >= 2 max|c| with
-// spin-flip symmetry, >= max|c| without (two passes, each with its own
-// rounding: half the scale keeps their sum below the error of one pass over
-// alpha and beta sums; the top digit stays below 65)
-__global__ void oz_absmax_kernel(const double *__restrict__ c, long long n, unsigned long long *__restrict__ out) {
-    double m = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        m = fmax(m, fabs(c[i]));
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
+// A single problem is prepared in two launches around its two maxima: CAS(6e,12o)
+// takes 41 us a call, 92 us with one launch per step (fold, max W, pack, map,
+// max c, scale, quantise: 62 us of device time before the contraction).
+
+// Largest |x| of the block's values to *out (as ordered bits; NaN left out).
+__device__ __forceinline__ void block_max_bits(long long m, unsigned long long *out) {
+    __shared__ long long red[8];
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; w++) m = max(m, red[w]);
+        if (m > 0) atomicMax(out, (unsigned long long)m);
+    }
+}
+__device__ __forceinline__ long long number_mag(double x) { return dmag(x) <= 0x7FF0000000000000ll ? dmag(x) : 0ll; }
+
+// smallest power of two > m (1 for 0)
+__device__ __forceinline__ double pow2_above(double m) {
+    int e = 0;
+    if (m > 0.0) frexp(m, &e);   // m = f 2^e, f in [0.5, 1)
+    return ldexp(1.0, e);
 }
 
-__global__ void oz_set_dscale_kernel(SigmaProb *__restrict__ p, const unsigned long long *__restrict__ mx) {
-    double m = __longlong_as_double((long long)*mx);
-    int e = 0;
-    if (m > 0.0) frexp((p->sym ? 2.0 : 1.0) * m, &e);
-    p->dscale = m > 0.0 ? ldexp(1.0, e) : 1.0;
+// Blocks [0, nfold): W and max |W| (mx[0]); [nfold, nfold + nabs): max |c|
+// (mx[1]); the others: kMapRows strings each of the excitation map.
+__global__ void __launch_bounds__(256) oz_prepare_one_kernel(FoldDesc d, int nfold, const double *__restrict__ c, long long n,
+                                                             int nabs, unsigned long long *__restrict__ mx, int nstr, int nexc,
+                                                             int ldj, const int32_t *__restrict__ exc,
+                                                             uint16_t *__restrict__ jmap) {
+    __shared__ __align__(8) uint16_t tile[kMapRows][kMaxNp + 2];
+    const int np = d.n * (d.n + 1) / 2;
+    int blk = blockIdx.x;
+    long long m = 0;
+    if (blk < nfold) {
+        double *kpair = reinterpret_cast<double *>(&tile[0][0]);   // np <= kMaxNp
+        for (int A = threadIdx.x; A < np; A += 256) kpair[A] = fold_pair(d, A);
+        __syncthreads();
+        const double invN = d.nelec > 0 ? 1.0 / (double)d.nelec : 0.0;
+        for (int t = blk * 256 + threadIdx.x; t < np * np; t += nfold * 256) {
+            const int A = t / np, B = t % np;
+            const double w = fold_element(d, kpair, invN, A, B);
+            d.W[(long long)A * d.ld + B] = w;
+            m = max(m, number_mag(w));
+        }
+        block_max_bits(m, mx);
+    } else if ((blk -= nfold) < nabs) {
+        for (long long i = blk * 256ll + threadIdx.x; i < n; i += nabs * 256ll) m = max(m, number_mag(c[i]));
+        block_max_bits(m, mx + 1);
+    } else {
+        map_rows((blk - nabs) * kMapRows, nstr, nexc, np, ldj, exc, jmap, tile);
+    }
+}
+
+// Blocks [0, nquant): the digit planes of c, the others the image of W, both
+// scaled by the maxima.  dscale of a caller's vector: the smallest power of two
+// above 2 max|c| with spin-flip symmetry, above max|c| without (two passes, each
+// with its own rounding: half the scale keeps their sum below the error of one
+// pass over alpha and beta sums; the top digit stays below 65).
+__global__ void __launch_bounds__(kGatherChunk)
+oz_quantise_pack_one_kernel(SigmaProb *probs, int nquant, const unsigned long long *__restrict__ mx, __half *__restrict__ Q,
+                            long long *__restrict__ S) {
+    const SigmaProb &p = probs[0];
+    const int blk = blockIdx.x;
+    if (blk < nquant) {
+        const double dscale = pow2_above((p.sym ? 2.0 : 1.0) * __longlong_as_double((long long)mx[1]));
+        if (blk == 0 && threadIdx.x == 0) probs[0].dscale = dscale;   // for the finish
+        const long long I = (long long)blk * kGatherChunk + threadIdx.x;
+        if (I < p.ndet) quantise_one(p, I, dscale, Q, S);
+    } else {
+        const double scale = pow2_above(__longlong_as_double((long long)mx[0]));
+        const int t = (blk - nquant) * kGatherChunk + threadIdx.x;
+        if (t == 0) p.Wexp[0] = scale;
+        if (t < p.np * (np_pad(p.np) / 8)) pack_group(p, t, scale);
+    }
 }
 
 int contracted_pairs(const SigmaProb &p) { return p.act ? p.npc : p.np; }
@@ -865,7 +960,7 @@ bool oz_wide(int nexc) { return nexc > kNarrowK; }
 
 int launch_oz_map(ifci_handle_t h, int nstr, int nexc, int np, const int32_t *exc, uint16_t *jmap, cudaStream_t s) {
     const int ldj = oz_map_ld(nstr);
-    oz_map_kernel<<<ldj / 128, 128, 0, s>>>(nstr, nexc, np, ldj, exc, jmap);
+    oz_map_kernel<<<ldj / kMapRows, 256, 0, s>>>(nstr, nexc, np, ldj, exc, jmap);
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;
 }
@@ -889,27 +984,7 @@ int launch_oz_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, int m
     return IFCI_OK;
 }
 
-int launch_oz_dscale(ifci_handle_t h, SigmaProb *d_prob, const double *c, long long n, cudaStream_t s) {
-    unsigned long long *mx = ws_take<unsigned long long>(h, 1);
-    if (!mx) return set_error(h, IFCI_ERR_OOM, "FP64E: workspace (scale)");
-    IFCI_CUDA_TRY(h, cudaMemsetAsync(mx, 0, sizeof(*mx), s));
-    int blocks = (int)std::min<long long>(1024, (n + 255) / 256);
-    oz_absmax_kernel<<<std::max(blocks, 1), 256, 0, s>>>(c, n, mx);
-    IFCI_LAUNCH_CHECK(h);
-    oz_set_dscale_kernel<<<1, 1, 0, s>>>(d_prob, mx);
-    IFCI_LAUNCH_CHECK(h);
-    return IFCI_OK;
-}
-
-int run_sigma_oz(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, void *D, void *G, cudaStream_t s) {
-    if (!h->d_err) return set_error(h, IFCI_ERR_INVALID_ARG, "FP64E: no error flag");
-    auto *Q = static_cast<__half *>(D);
-    auto *S = static_cast<long long *>(G);
-    {
-        ProfScope ps(h, s, PK_GATHER);
-        oz_quantise_kernel<<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0, Q, S);
-        IFCI_LAUNCH_CHECK(h);
-    }
+static int contract_oz(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, __half *Q, long long *S, cudaStream_t s) {
     static SmemOptIn opt_n, opt_w, opt_g;
     for (int wide = 0; wide < 2; wide++) {
         const int i0 = wide ? w.tc0 + w.ntc : w.tc0, ni = wide ? w.nwide : w.ntc;
@@ -944,6 +1019,40 @@ int run_sigma_oz(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, voi
     oz_finish_kernel<<<w.nfin, 256, 0, s>>>(plan.d_probs, plan.d_tiles + w.tile0, S);
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;
+}
+
+int run_sigma_oz(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, void *D, void *G, cudaStream_t s) {
+    if (!h->d_err) return set_error(h, IFCI_ERR_INVALID_ARG, "FP64E: no error flag");
+    auto *Q = static_cast<__half *>(D);
+    auto *S = static_cast<long long *>(G);
+    {
+        ProfScope ps(h, s, PK_GATHER);
+        oz_quantise_kernel<<<w.nitem, kGatherChunk, 0, s>>>(plan.d_probs, plan.d_items + w.item0, Q, S);
+        IFCI_LAUNCH_CHECK(h);
+    }
+    return contract_oz(h, plan, w, Q, S, s);
+}
+
+int run_sigma_oz_one(ifci_handle_t h, const SigmaPlan &plan, const FoldDesc &f, const double *c, uint16_t *jmap,
+                     unsigned long long *mx, void *D, void *G, cudaStream_t s) {
+    if (!h->d_err) return set_error(h, IFCI_ERR_INVALID_ARG, "FP64E: no error flag");
+    const SigmaProb &p = plan.probs[0];
+    auto *Q = static_cast<__half *>(D);
+    auto *S = static_cast<long long *>(G);
+    {
+        ProfScope ps(h, s, PK_GATHER);
+        IFCI_CUDA_TRY(h, cudaMemsetAsync(mx, 0, 2 * sizeof(*mx), s));
+        const int nfold = (p.np * p.np + 511) / 512;   // two elements a thread
+        const int nabs = (int)std::min<long long>(2 * device_sm_count(h->device), (p.ndet + 511) / 512);
+        oz_prepare_one_kernel<<<nfold + nabs + p.ldj / kMapRows, 256, 0, s>>>(f, nfold, c, p.ndet, nabs, mx, p.nstr, p.nexc,
+                                                                              p.ldj, p.exc, jmap);
+        IFCI_LAUNCH_CHECK(h);
+        const int nquant = (int)((p.ndet + kGatherChunk - 1) / kGatherChunk);
+        const int npack = (p.np * (np_pad(p.np) / 8) + kGatherChunk - 1) / kGatherChunk;
+        oz_quantise_pack_one_kernel<<<nquant + npack, kGatherChunk, 0, s>>>(plan.d_probs, nquant, mx, Q, S);
+        IFCI_LAUNCH_CHECK(h);
+    }
+    return contract_oz(h, plan, plan.waves[0], Q, S, s);
 }
 
 }  // namespace ifci
