@@ -128,11 +128,32 @@ contract_simt_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__rest
     }
 }
 
-// +-(double)g for an excitation entry x.  The conversion of an FP32 G and the
-// sign run on the integer pipe: the sum itself is the only FP64 instruction per
-// element (CAS(6e,17o): 139 us, with a conversion and a product by +-1 256 us).
-__device__ __forceinline__ double signed_g(double g, int32_t x) { return dflip(g, (uint32_t)x << 31); }
-__device__ __forceinline__ double signed_g(float g, int32_t x) { return f2d(__uint_as_float(__float_as_uint(g) ^ (uint32_t)x << 31)); }
+// Sum of signed entries of G: FP64 for an FP64 G.  An FP32 G is added up in
+// two floats, each rounding error of the first kept in the second (TwoSum, exact
+// per step; Knuth, The Art of Computer Programming 2, 4.2.2): ~48 bits, and an
+// FP64 addition takes the pipe 64 clk a warp (CAS(6e,17o): 73 us, in FP64
+// 119 us).  The error of sigma against 64 bits is that of G in either form.
+template <typename TG>
+struct SignedSum;
+template <>
+struct SignedSum<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double g, int32_t x) { v += dflip(g, (uint32_t)x << 31); }
+    __device__ __forceinline__ bool good() const { return true; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <>
+struct SignedSum<float> {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float g, int32_t x) {
+        const float b = __uint_as_float(__float_as_uint(g) ^ (uint32_t)x << 31);
+        const float s = __fadd_rn(hi, b), t = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(b, t)));
+        hi = s;
+    }
+    __device__ __forceinline__ bool good() const { return isfinite(hi) && isfinite(lo); }   // else: FP64 throughout
+    __device__ __forceinline__ double value() const { return f2d(hi) + f2d(lo); }
+};
 
 template <typename TG>
 __global__ void __launch_bounds__(kGatherChunk)
@@ -148,15 +169,16 @@ scatter_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__
     const int32_t *__restrict__ ea = p.exc + (size_t)ia * nexc;
     const int32_t *__restrict__ eb = p.exc + (size_t)ib * nexc;
     const TG *__restrict__ Gp = G + p.doff;
-    double v = 0.0;
-    for (int e = 0; e < nexc; e++) {
-        int32_t x = ea[e];
-        v += signed_g(Gp[(long long)exc_pair(x) * ndet + (long long)exc_J(x) * nstr + ib], x);
-    }
-    const long long rowb = (long long)ia * nstr;
-    for (int e = 0; e < nexc; e++) {
-        int32_t x = eb[e];
-        v += signed_g(Gp[(long long)exc_pair(x) * ndet + rowb + exc_J(x)], x);
+    const TG *__restrict__ Ga = Gp + ib, *__restrict__ Gb = Gp + (long long)ia * nstr;
+    SignedSum<TG> sum;
+    for (int e = 0; e < nexc; e++) sum.add(Ga[(long long)exc_pair(ea[e]) * ndet + (long long)exc_J(ea[e]) * nstr], ea[e]);
+    for (int e = 0; e < nexc; e++) sum.add(Gb[(long long)exc_pair(eb[e]) * ndet + exc_J(eb[e])], eb[e]);
+    double v = sum.value();
+    if (!sum.good()) {
+        SignedSum<double> wide;
+        for (int e = 0; e < nexc; e++) wide.add((double)Ga[(long long)exc_pair(ea[e]) * ndet + (long long)exc_J(ea[e]) * nstr], ea[e]);
+        for (int e = 0; e < nexc; e++) wide.add((double)Gb[(long long)exc_pair(eb[e]) * ndet + exc_J(eb[e])], eb[e]);
+        v = wide.value();
     }
     double *s = p.sbase + (p.sslot ? (long long)*p.sslot : 0ll) * p.stride;
     s[I] = v;
