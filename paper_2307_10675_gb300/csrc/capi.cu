@@ -98,11 +98,11 @@ int ifci_sigma(ifci_handle_t h, const ifci_strings_t *str, const double *h1, con
     }
     IFCI_CUDA_TRY(h, cudaMemcpyAsync(fd, &f, sizeof(f), cudaMemcpyHostToDevice, s));
     IFCI_TRY(launch_fold(h, 1, fd, np, s));
-    if (blk) IFCI_TRY(launch_exc_blocks(h, nstr, nexc, str->exc, blk, s));
+    if (blk && !pmap) IFCI_TRY(launch_exc_blocks(h, nstr, nexc, str->exc, blk, s));
     if (pmap) IFCI_TRY(launch_pair_map(h, nstr, nexc, np, str->exc, pmap, s));
     IFCI_TRY(upload_plan(h, plan, s));
     if (precision == IFCI_FP32) IFCI_TRY(launch_convert_w(h, 1, plan.d_probs, s));
-    if (tc) IFCI_TRY(launch_tc_pack_w(h, 1, plan.d_probs, precision, s));
+    if (tc) IFCI_TRY(launch_tc_pack_w(h, 1, plan.d_probs, precision, np, s));
     D = ws_take<char>(h, (size_t)delems_D * eb);
     G = ws_take<char>(h, (size_t)plan.max_delems * eb);
     if (!D || !G) return set_error(h, IFCI_ERR_OOM, "ifci_sigma: workspace");

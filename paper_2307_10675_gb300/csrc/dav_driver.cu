@@ -472,7 +472,7 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
         if (lo || oz) IFCI_TRY(launch_fold(h, nu, mem.fold, maxnp, s));
         if (f64) IFCI_TRY(launch_string_h_batch(h, mem.hdesc, mem.hitems, (int)hitems.size(), s));
         if (lo) IFCI_TRY(launch_convert_w(h, nu, lop.d_probs, s));
-        if (tc) IFCI_TRY(launch_tc_pack_w(h, nu, lop.d_probs, o.precision, s));
+        if (tc) IFCI_TRY(launch_tc_pack_w(h, nu, lop.d_probs, o.precision, maxnp, s));
         if (oz) IFCI_TRY(launch_oz_pack_w(h, nu, hi.d_probs, maxnp, s));
         IFCI_TRY(launch_hdiag(h, mem.hdu, mem.hwp, mem.hws, (int)hw_prob.size(), kVecChunk, s));
         if (b.any_sector) IFCI_TRY(launch_sector_hd(h, b, s));

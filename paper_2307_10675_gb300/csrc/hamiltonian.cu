@@ -152,8 +152,8 @@ int launch_frozen_core(ifci_handle_t h, int nprob, const FrozenDesc *d_desc, con
 
 int launch_fold(ifci_handle_t h, int nprob, const FoldDesc *d_desc, int max_np, cudaStream_t s) {
     if (nprob <= 0) return IFCI_OK;
-    // about four elements per thread while there are few problems
-    const int parts = std::max(1, std::min((max_np * max_np + 1023) / 1024, 16 * device_sm_count(h->device) / nprob));
+    // about two elements per thread while there are few problems
+    const int parts = std::max(1, std::min((max_np * max_np + 511) / 512, 16 * device_sm_count(h->device) / nprob));
     fold_kernel<<<dim3(nprob, parts), 256, max_np * sizeof(double), s>>>(d_desc);
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;

@@ -140,7 +140,7 @@ int run_sigma_oz_one(ifci_handle_t h, const SigmaPlan &plan, const FoldDesc &f, 
 // tensor-core contraction (sigma_tc.cu)
 int tc_supported(int precision);
 int tc_operand_bytes(int np, int precision);   // bytes of one problem's W image
-int launch_tc_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, int precision, cudaStream_t s);
+int launch_tc_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, int precision, int max_np, cudaStream_t s);
 int launch_tc_contract(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, int precision,
                        const void *D, void *G, cudaStream_t s);
 

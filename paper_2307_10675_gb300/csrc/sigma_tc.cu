@@ -28,7 +28,7 @@ using namespace tc;
 
 constexpr int kBfThreads = 512;   // four threads per determinant row
 
-__global__ void __launch_bounds__(kBfThreads, 1)
+__global__ void __launch_bounds__(kBfThreads, 2)
 tc_contract_bf16_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ tiles, int ntile,
                         size_t w_bytes_max, size_t a_bytes_max, const float *__restrict__ Q,
                         float *__restrict__ G, int *__restrict__ err, int *__restrict__ counter) {
@@ -152,12 +152,13 @@ tc_contract_bf16_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__r
 }
 
 // BF16 image of W in the B-operand layout: [atom a][row n < N][128 B], the
-// 16-byte chunk c of row n stored at chunk c ^ (n % 8); zero padding.
+// 16-byte chunk c of row n stored at chunk c ^ (n % 8); zero padding.  Blocks
+// (problem, part).
 __global__ void pack_w_bf16_kernel(const SigmaProb *__restrict__ probs) {
     const SigmaProb &p = probs[blockIdx.x];
     const int np = p.np, N = n_pad(np), KA = k_atoms(np);
     uint8_t *img = (uint8_t *)const_cast<void *>(p.Wtc);
-    for (int t = threadIdx.x; t < N * KA * 8; t += blockDim.x) {
+    for (int t = blockIdx.y * blockDim.x + threadIdx.x; t < N * KA * 8; t += gridDim.y * blockDim.x) {
         const int n = t / (KA * 8), ch = t % (KA * 8);
         uint32_t pk[4];
         for (int e = 0; e < 8; e += 2) {
@@ -208,7 +209,7 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64
         : "memory");
 }
 
-__global__ void __launch_bounds__(kBfThreads, 1)
+__global__ void __launch_bounds__(kBfThreads, 2)
 tc_contract_tf32_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__ tiles, int ntile,
                         size_t w_stage_max, const float *__restrict__ Q, float *__restrict__ G,
                         int *__restrict__ err, int *__restrict__ counter) {
@@ -360,7 +361,7 @@ __global__ void pack_w_tf32_kernel(const SigmaProb *__restrict__ probs) {
     const SigmaProb &p = probs[blockIdx.x];
     const int np = p.np, N = n_pad(np), KA = tf_atoms(np);
     uint8_t *img = (uint8_t *)const_cast<void *>(p.Wtc);
-    for (int t = threadIdx.x; t < N * KA * 8; t += blockDim.x) {
+    for (int t = blockIdx.y * blockDim.x + threadIdx.x; t < N * KA * 8; t += gridDim.y * blockDim.x) {
         const int n = t / (KA * 8), ch = t % (KA * 8);
         uint32_t pk[4];
         for (int e = 0; e < 4; e++) {
@@ -372,6 +373,13 @@ __global__ void pack_w_tf32_kernel(const SigmaProb *__restrict__ probs) {
         *dst = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
 }
+
+// Two CTAs share an SM while their buffers fit (BF16: up to 160 pairs, TF32: 128),
+// so that one gathers while the other multiplies or stores: CAS(6e,17o) in BF16
+// 166 us with one CTA per SM, 120 us with two.  Their 2 x 256 TMEM columns are
+// all there are; at least 76 KB of shared memory keeps a third one out, so TMEM
+// allocation never waits.
+constexpr size_t kTwoPerSm = (size_t)76 * 1024, kHalfSm = (size_t)112 * 1024;
 
 size_t tc_smem_bytes(int max_np) {
     size_t w = (size_t)k_atoms(max_np) * n_pad(max_np) * kAtomBytes;
@@ -387,11 +395,14 @@ int tc_operand_bytes(int np, int precision) {
     return (precision == IFCI_TF32 ? tf_atoms(np) : k_atoms(np)) * n_pad(np) * kAtomBytes;
 }
 
-int launch_tc_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, int precision, cudaStream_t s) {
+int launch_tc_pack_w(ifci_handle_t h, int nprob, const SigmaProb *d_probs, int precision, int max_np, cudaStream_t s) {
     if (!tc_supported(precision)) return set_error(h, IFCI_ERR_UNSUPPORTED, "tensor-core precision %d", precision);
     if (nprob <= 0) return IFCI_OK;
-    if (precision == IFCI_TF32) pack_w_tf32_kernel<<<nprob, 256, 0, s>>>(d_probs);
-    else pack_w_bf16_kernel<<<nprob, 256, 0, s>>>(d_probs);
+    // one 16-byte chunk per thread while there are few problems
+    const int parts = (tc_operand_bytes(max_np, precision) / 16 + 255) / 256;
+    const dim3 grid(nprob, std::max(1, std::min(parts, 16 * device_sm_count(h->device) / nprob)));
+    if (precision == IFCI_TF32) pack_w_tf32_kernel<<<grid, 256, 0, s>>>(d_probs);
+    else pack_w_bf16_kernel<<<grid, 256, 0, s>>>(d_probs);
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;
 }
@@ -407,14 +418,14 @@ int launch_tc_contract(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &
     if (!h->d_err) return set_error(h, IFCI_ERR_INVALID_ARG, "tensor-core path: no error flag");
     if (!h->d_counter) return set_error(h, IFCI_ERR_INVALID_ARG, "tensor-core path: no tile counter");
     if (precision == IFCI_TF32) {
-        // two W atom stages + the whole A tile; at least 116 KB so that one CTA runs per SM
+        // two W atom stages + the whole A tile
         const size_t wst = (size_t)n_pad(max_np) * kAtomBytes;
         const size_t smem = std::max(1024 + 2 * ((wst + 1023) & ~(size_t)1023) +
                                          (size_t)tf_atoms(max_np) * kTM * kAtomBytes,
-                                     (size_t)116 * 1024);
+                                     kTwoPerSm);
         static SmemOptIn opt_tf;
         IFCI_CUDA_TRY(h, ensure_smem(opt_tf, h->device, tc_contract_tf32_kernel, (int)smem));
-        const int grid = std::min(w.ntc, device_sm_count(h->device));
+        const int grid = std::min(w.ntc, (smem <= kHalfSm ? 2 : 1) * device_sm_count(h->device));
         IFCI_CUDA_TRY(h, cudaMemsetAsync(h->d_counter, 0, sizeof(int), s));
         ProfScope ps(h, s, PK_CONTRACT);
         tc_contract_tf32_kernel<<<grid, kBfThreads, smem, s>>>(plan.d_probs, plan.d_tctiles + w.tc0, w.ntc, wst,
@@ -422,13 +433,12 @@ int launch_tc_contract(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &
         IFCI_LAUNCH_CHECK(h);
         return IFCI_OK;
     }
-    // at least 116 KB of shared memory: one CTA per SM, so TMEM allocation never waits
-    const size_t smem = std::max(tc_smem_bytes(max_np), (size_t)116 * 1024);
+    const size_t smem = std::max(tc_smem_bytes(max_np), kTwoPerSm);
     const size_t wmax = (size_t)k_atoms(max_np) * n_pad(max_np) * kAtomBytes;
     const size_t amax = (size_t)k_atoms(max_np) * kTM * kAtomBytes;
     static SmemOptIn opt;
     IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, tc_contract_bf16_kernel, (int)smem));
-    const int grid = std::min(w.ntc, device_sm_count(h->device));
+    const int grid = std::min(w.ntc, (smem <= kHalfSm ? 2 : 1) * device_sm_count(h->device));
     IFCI_CUDA_TRY(h, cudaMemsetAsync(h->d_counter, 0, sizeof(int), s));
     ProfScope ps(h, s, PK_CONTRACT);
     tc_contract_bf16_kernel<<<grid, kBfThreads, smem, s>>>(plan.d_probs, plan.d_tctiles + w.tc0, w.ntc, wmax, amax,
