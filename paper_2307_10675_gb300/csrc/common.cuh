@@ -165,23 +165,26 @@ struct StringBinom {
     int c[32][32];
 };
 StringBinom string_binom();
-__device__ __forceinline__ int string_rank_of(uint32_t mask, const StringBinom &B) {
+// (c: binomials [n][m + 1] or more, row stride LD)
+template <int LD>
+__device__ __forceinline__ int string_rank_of(uint32_t mask, const int (&c)[32][LD]) {
     int r = 0, k = 1;
     while (mask) {
         int p = __ffs(mask) - 1;
-        r += B.c[p][k];
+        r += c[p][k];
         k++;
         mask &= mask - 1;
     }
     return r;
 }
-__device__ __forceinline__ uint32_t string_of_rank(int rank, int n, int m, const StringBinom &B) {
+template <int LD>
+__device__ __forceinline__ uint32_t string_of_rank(int rank, int n, int m, const int (&c)[32][LD]) {
     uint32_t mask = 0;
     int rem = rank;
     for (int k = m; k >= 1; k--) {
         int p = k - 1;
-        while (p + 1 < n && B.c[p + 1][k] <= rem) p++;
-        rem -= B.c[p][k];
+        while (p + 1 < n && c[p + 1][k] <= rem) p++;
+        rem -= c[p][k];
         mask |= 1u << p;
     }
     return mask;

@@ -23,7 +23,7 @@
 // the accumulator's sign bit instead of costing a multiplication.  56 KB per
 // block leave four blocks on an SM, whose loads overlap another's FMAs.
 //
-// Measured: CAS(6e,13o) 253 us (dense contraction 1634 us, gather and scatter
+// Measured: CAS(6e,13o) 240 us and 9 us for the lists (dense contraction 1634 us, gather and scatter
 // 103 us before), 1.1e8 FMAs at 0.44 of a DGEMM's rate.
 #include <algorithm>
 
@@ -36,6 +36,7 @@ namespace {
 
 constexpr int kMaxThreads64 = 512;
 constexpr int kList = 128;              // alpha-alpha elements staged at a time
+constexpr int kMaxExc = (kMaxNorb + 1) * (kMaxNorb + 1) / 4;   // most excitations m (n - m + 1) of a string
 constexpr int kCapSmall = 6912, kCapMid = 13824, kCapLarge = 28160;   // doubles: 4, 2 or 1 blocks per SM
 
 // the input row and the sums are kept in shared memory too, unless the strings
@@ -56,7 +57,7 @@ __host__ __device__ inline int fit64(int nstr, int np, int nexc, long long cap) 
 __device__ __forceinline__ void sigma64_body(const SigmaProb &p, int ka, int cap) {
     extern __shared__ double sm[];
     __shared__ double lv[kList];
-    __shared__ int lj[kList];
+    __shared__ int lj[kList], lx[kMaxExc];
     if (p.active && !*p.active) return;
     const int nstr = p.nstr, nexc = p.nexc, np = p.np, nnz = p.nnz, t = threadIdx.x, nt = blockDim.x;
     const double *__restrict__ c = p.cbase + (p.cslot ? (long long)*p.cslot : 0ll) * p.stride;
@@ -71,11 +72,13 @@ __device__ __forceinline__ void sigma64_body(const SigmaProb &p, int ka, int cap
     double *Vs = Cs + (size_t)kb * nstr;
     if (rows)
         for (int i = t; i < nstr; i += nt) sm[i] = c[(long long)ka * nstr + i];
+    for (int i = t; i < nexc; i += nt) lx[i] = exc[(size_t)ka * nexc + i];
     __syncthreads();
     // beta beta: the string's own elements, the row from shared memory
     for (int ib = t; ib < nstr; ib += nt) {
         double a0 = 0.0, a1 = 0.0;
         int e = 0;
+#pragma unroll 4
         for (; e + 1 < nnz; e += 2) {
             a0 = fma(hval[(size_t)e * nstr + ib], row[hidx[(size_t)e * nstr + ib]], a0);
             a1 = fma(hval[(size_t)(e + 1) * nstr + ib], row[hidx[(size_t)(e + 1) * nstr + ib]], a1);
@@ -108,8 +111,9 @@ __device__ __forceinline__ void sigma64_body(const SigmaProb &p, int ka, int cap
     for (int k0 = 0; k0 < nexc; k0 += kb) {
         const int kn = min(kb, nexc - k0);
         __syncthreads();
-        for (int k = 0; k < kn; k++) {
-            const int32_t x = exc[(size_t)ka * nexc + k0 + k];
+#pragma unroll 4
+        for (int k = 0; k < kn; k++) {   // loads of several excitations in flight
+            const int32_t x = lx[k0 + k];
             const uint32_t neg = (uint32_t)(x & 1) << 31;
             const double *src = c + (long long)exc_J(x) * nstr, *v = p.eri + (long long)exc_pair(x) * np;
             for (int i = t; i < nstr; i += nt) Cs[(size_t)k * nstr + i] = dflip(src[i], neg);
@@ -154,20 +158,27 @@ sigma64_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict__
 
 // Element list of the string Hamiltonian: entry 0 the diagonal, then the
 // single, then the double excitations (occupied major), at [entry][string].
-// val and idx may each be nullptr.
+// val and idx may each be nullptr.  A lane owns one of kStringHChunk strings,
+// a warp one entry at a time (the same kind of element in all lanes); the
+// gridDim.y parts of a problem share its entries.  The binomials that rank and
+// unrank strings sit in shared memory: lanes read them at addresses of their
+// own, which a kernel parameter serves one after the other.
+// CAS(6e,13o), 166 entries of 286 strings: 9.4 us; 9 blocks, a string unranked for
+// each element from the parameter, took 56 us.
 __device__ __forceinline__ void string_h_body(const StringHDesc &d, int I0, const StringBinom &B) {
-    const int n = d.n, m = d.m, nv = n - m, ns = m * nv, nvp = nv * (nv - 1) / 2;
-    for (int w = threadIdx.x; w < d.nnz * kStringHChunk; w += 256) {
-        // consecutive threads: consecutive strings of one entry
-        const int e = w / kStringHChunk, I = I0 + w % kStringHChunk;
-        if (I >= d.nstr) continue;
-        const uint32_t bra = string_of_rank(I, n, m, B);
+    const int n = d.n, m = d.m, nv = n - m, ns = m * nv, nvp = nv * (nv - 1) / 2, lane = threadIdx.x % kStringHChunk;
+    __shared__ int bin[32][33];
+    for (int t = threadIdx.x; t < n * (m + 1); t += 256) bin[t / (m + 1)][t % (m + 1)] = B.c[t / (m + 1)][t % (m + 1)];
+    __syncthreads();
+    const int I = I0 + lane;
+    if (I >= d.nstr) return;
+    const uint32_t bra = string_of_rank(I, n, m, bin), vir = ~bra & (n == 32 ? ~0u : (1u << n) - 1u);
+    auto nth = [](uint32_t x, int k) {
+        for (; k > 0; k--) x &= x - 1;
+        return x & (~x + 1u);
+    };
+    for (int e = blockIdx.y * (256 / kStringHChunk) + threadIdx.x / kStringHChunk; e < d.nnz; e += gridDim.y * (256 / kStringHChunk)) {
         uint32_t ket = bra;
-        auto nth = [](uint32_t x, int k) {
-            for (; k > 0; k--) x &= x - 1;
-            return x & (~x + 1u);
-        };
-        const uint32_t vir = ~bra & (n == 32 ? ~0u : (1u << n) - 1u);
         if (e > ns) {
             int o = (e - 1 - ns) / nvp, v = (e - 1 - ns) % nvp, i = 0, a = 0;
             while (o >= m - 1 - i) o -= m - 1 - i++;       // pair (i, i + 1 + o) of the occupied
@@ -176,7 +187,7 @@ __device__ __forceinline__ void string_h_body(const StringHDesc &d, int I0, cons
         } else if (e > 0) {
             ket ^= nth(bra, (e - 1) / nv) | nth(vir, (e - 1) % nv);
         }
-        if (d.idx) d.idx[(size_t)e * d.nstr + I] = string_rank_of(ket, B);
+        if (d.idx) d.idx[(size_t)e * d.nstr + I] = string_rank_of(ket, bin);
         if (d.val) d.val[(size_t)e * d.nstr + I] = h_element(n, d.h1, d.eri, bra, 0u, ket, 0u);
     }
 }
@@ -188,6 +199,11 @@ __global__ void __launch_bounds__(256) string_h_kernel(const StringHDesc *__rest
                                                        const StringBinom B) {
     const WorkItem it = items[blockIdx.x];
     string_h_body(desc[it.prob], (int)it.start, B);
+}
+
+// parts of a problem's entries: about two blocks per SM, eight entries to a part
+static int string_h_parts(ifci_handle_t h, int nblk, int nnz) {
+    return std::max(1, std::min((nnz + 7) / 8, 2 * device_sm_count(h->device) / nblk));
 }
 
 int cap64(const SigmaProb *probs, int nprob) {
@@ -214,14 +230,15 @@ StringBinom string_binom() {
 int string_h_nnz(int n, int m) { return 1 + m * (n - m) + m * (m - 1) / 2 * ((n - m) * (n - m - 1) / 2); }
 
 int launch_string_h(ifci_handle_t h, const StringHDesc &one, cudaStream_t s) {
-    string_h_one_kernel<<<(one.nstr + kStringHChunk - 1) / kStringHChunk, 256, 0, s>>>(one, string_binom());
+    const int nblk = (one.nstr + kStringHChunk - 1) / kStringHChunk;
+    string_h_one_kernel<<<dim3(nblk, string_h_parts(h, nblk, one.nnz)), 256, 0, s>>>(one, string_binom());
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;
 }
 
 int launch_string_h_batch(ifci_handle_t h, const StringHDesc *d_desc, const WorkItem *d_items, int nitem, cudaStream_t s) {
     if (nitem <= 0) return IFCI_OK;
-    string_h_kernel<<<nitem, 256, 0, s>>>(d_desc, d_items, string_binom());
+    string_h_kernel<<<dim3(nitem, string_h_parts(h, nitem, 64)), 256, 0, s>>>(d_desc, d_items, string_binom());
     IFCI_LAUNCH_CHECK(h);
     return IFCI_OK;
 }

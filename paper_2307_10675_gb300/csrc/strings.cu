@@ -13,9 +13,13 @@ namespace ifci {
 // ascending pair order.
 __global__ void build_strings_kernel(int n, int m, int nstr, int nexc, StringBinom B,
                                      uint64_t *__restrict__ strings, int32_t *__restrict__ exc) {
+    // read at lane-dependent addresses: a kernel parameter would serve them one by one
+    __shared__ int bin[32][33];
+    for (int t = threadIdx.x; t < n * (m + 1); t += blockDim.x) bin[t / (m + 1)][t % (m + 1)] = B.c[t / (m + 1)][t % (m + 1)];
+    __syncthreads();
     int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nstr) return;
-    uint32_t mask = string_of_rank(I, n, m, B);
+    uint32_t mask = string_of_rank(I, n, m, bin);
     strings[I] = mask;
     int32_t *row = exc + (size_t)I * nexc;
     int k = 0;
@@ -32,7 +36,7 @@ __global__ void build_strings_kernel(int n, int m, int nstr, int nexc, StringBin
                 uint32_t J = mask ^ (1u << P) ^ (1u << Q);
                 uint32_t between = ((1u << P) - 1u) & ~((2u << Q) - 1u);
                 int neg = __popc(mask & between) & 1;
-                if (k < nexc) row[k++] = (string_rank_of(J, B) << 10) | (A << 1) | neg;
+                if (k < nexc) row[k++] = (string_rank_of(J, bin) << 10) | (A << 1) | neg;
             }
         }
     }
