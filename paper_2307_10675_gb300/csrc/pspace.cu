@@ -355,24 +355,41 @@ __device__ __forceinline__ void psp_jacobi_ahead(double *A, double *V, int P, do
 // the diagonal (the other half is its mirror image) and 4 per element pair of
 // V.  n4 = P rounded up to a multiple of 4; the padding rows are zero and never
 // rotate.
-template <int MAXP, int NT>
-__device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, double *red, double *red2) {
+// T = float: a first pass that leaves few FP64 sweeps to do (psp_jacobi_refined);
+// it stops at 1e-11 of |A|_F^2, near FP32's own rounding.
+__device__ __forceinline__ bool pair_rotation(double app, double aqq, double apq, double &c, double &s, bool &zero) {
+    if (dmag(apq) < dbits(1e-300)) return false;
+    zero = jacobi_negligible(app, aqq, apq);
+    if (!zero) jacobi_rotation(app, aqq, apq, c, s);
+    return !zero;
+}
+__device__ __forceinline__ bool pair_rotation(float app, float aqq, float apq, float &c, float &s, bool &) {
+    if (!(fabsf(apq) > 1e-9f * (fabsf(app) + fabsf(aqq)))) return false;
+    const float tau = (aqq - app) / (2.0f * apq);
+    const float t = (tau >= 0.0f ? 1.0f : -1.0f) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
+    c = rsqrtf(1.0f + t * t);
+    s = t * c;
+    return true;
+}
+
+template <int MAXP, int NT, typename T>
+__device__ __forceinline__ void psp_jacobi_pairs(T *A, T *V, int P, int sweeps, T small, T *red, T *red2) {
     static_assert(MAXP % 4 == 0 && NT >= MAXP && NT / 32 <= MAXP, "P-space sizes");
     constexpr int LD = MAXP + 1;
-    __shared__ double rc[MAXP / 2], rsn[MAXP / 2];
+    __shared__ T rc[MAXP / 2], rsn[MAXP / 2];
     __shared__ int rp[MAXP / 2], rq[MAXP / 2];       // the step's index pairs; rq < 0: no rotation
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int n4 = (P + 3) & ~3, npr = n4 / 2;
     for (int e = t; e < n4 * n4; e += NT) {
         const int r = e / n4, c = e % n4;
-        if (r >= P || c >= P) A[r * LD + c] = 0.0;
+        if (r >= P || c >= P) A[r * LD + c] = T(0);
     }
     __syncthreads();
-    for (int sweep = 0; sweep < 40; sweep++) {
-        double off = 0.0, all = 0.0;
+    for (int sweep = 0; sweep < sweeps; sweep++) {
+        T off = T(0), all = T(0);
         for (int e = t; e < P * P; e += NT) {
             const int r = e / P, c = e % P;
-            const double a = A[r * LD + c];
+            const T a = A[r * LD + c];
             all += a * a;
             if (c != r) off += a * a;
         }
@@ -386,35 +403,30 @@ __device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, do
             red2[warp] = all;
         }
         __syncthreads();
-        off = all = 0.0;
+        off = all = T(0);
         for (int w = 0; w < NT / 32; w++) {
             off += red[w];
             all += red2[w];
         }
-        if (off <= 1e-26 * all || off == 0.0) break;
+        if (off <= small * all || off == T(0)) break;
         for (int step = 0; step < n4 - 1; step++) {
             if (t < npr) {
                 // index n4 - 1 stays, the others turn
                 const int a = t == 0 ? n4 - 1 : (step + t) % (n4 - 1), b = t == 0 ? step : (step + n4 - 1 - t) % (n4 - 1);
                 const int pp = min(a, b), q = max(a, b);
-                const double apq = A[pp * LD + q];
-                int rot = 0;
-                if (dmag(apq) >= dbits(1e-300)) {
-                    const double app = A[pp * LD + pp], aqq = A[q * LD + q];
-                    if (jacobi_negligible(app, aqq, apq)) {
-                        A[pp * LD + q] = A[q * LD + pp] = 0.0;
-                    } else {
-                        double c, sn;
-                        jacobi_rotation(app, aqq, apq, c, sn);
-                        const double xp = c * app - sn * apq, xq = sn * app + c * apq;   // columns of row p
-                        const double yp = c * apq - sn * aqq, yq = sn * apq + c * aqq;   // columns of row q
-                        A[pp * LD + pp] = c * xp - sn * yp;
-                        A[q * LD + q] = sn * xq + c * yq;
-                        A[pp * LD + q] = A[q * LD + pp] = c * xq - sn * yq;
-                        rc[t] = c;
-                        rsn[t] = sn;
-                        rot = 1;
-                    }
+                const T app = A[pp * LD + pp], aqq = A[q * LD + q], apq = A[pp * LD + q];
+                T c = T(1), sn = T(0);
+                bool zero = false;
+                const bool rot = pair_rotation(app, aqq, apq, c, sn, zero);
+                if (zero) A[pp * LD + q] = A[q * LD + pp] = T(0);
+                if (rot) {
+                    const T xp = c * app - sn * apq, xq = sn * app + c * apq;   // columns of row p
+                    const T yp = c * apq - sn * aqq, yq = sn * apq + c * aqq;   // columns of row q
+                    A[pp * LD + pp] = c * xp - sn * yp;
+                    A[q * LD + q] = sn * xq + c * yq;
+                    A[pp * LD + q] = A[q * LD + pp] = c * xq - sn * yq;
+                    rc[t] = c;
+                    rsn[t] = sn;
                 }
                 rp[t] = pp;
                 rq[t] = rot ? q : -1 - q;
@@ -427,16 +439,16 @@ __device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, do
                 const int i = c >= r ? r : npr - 1 - r, j = c >= r ? c + 1 : npr - 1 - c;
                 int qi = rq[i], qj = rq[j];
                 if (qi < 0 && qj < 0) continue;
-                const double ci = qi >= 0 ? rc[i] : 1.0, si = qi >= 0 ? rsn[i] : 0.0;
-                const double cj = qj >= 0 ? rc[j] : 1.0, sj = qj >= 0 ? rsn[j] : 0.0;
+                const T ci = qi >= 0 ? rc[i] : T(1), si = qi >= 0 ? rsn[i] : T(0);
+                const T cj = qj >= 0 ? rc[j] : T(1), sj = qj >= 0 ? rsn[j] : T(0);
                 const int pi = rp[i], pj = rp[j];
                 if (qi < 0) qi = -1 - qi;
                 if (qj < 0) qj = -1 - qj;
-                const double a00 = A[pi * LD + pj], a01 = A[pi * LD + qj], a10 = A[qi * LD + pj], a11 = A[qi * LD + qj];
-                const double x00 = cj * a00 - sj * a01, x01 = sj * a00 + cj * a01;
-                const double x10 = cj * a10 - sj * a11, x11 = sj * a10 + cj * a11;
-                const double b00 = ci * x00 - si * x10, b10 = si * x00 + ci * x10;
-                const double b01 = ci * x01 - si * x11, b11 = si * x01 + ci * x11;
+                const T a00 = A[pi * LD + pj], a01 = A[pi * LD + qj], a10 = A[qi * LD + pj], a11 = A[qi * LD + qj];
+                const T x00 = cj * a00 - sj * a01, x01 = sj * a00 + cj * a01;
+                const T x10 = cj * a10 - sj * a11, x11 = sj * a10 + cj * a11;
+                const T b00 = ci * x00 - si * x10, b10 = si * x00 + ci * x10;
+                const T b01 = ci * x01 - si * x11, b11 = si * x01 + ci * x11;
                 A[pi * LD + pj] = A[pj * LD + pi] = b00;
                 A[pi * LD + qj] = A[qj * LD + pi] = b01;
                 A[qi * LD + pj] = A[pj * LD + qi] = b10;
@@ -445,7 +457,7 @@ __device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, do
             for (int e = t; e < npr * P; e += NT) {
                 const int i = e / P, r = e % P, q = rq[i];
                 if (q < 0) continue;
-                const double c = rc[i], sn = rsn[i], vp = V[r * LD + rp[i]], vq = V[r * LD + q];
+                const T c = rc[i], sn = rsn[i], vp = V[r * LD + rp[i]], vq = V[r * LD + q];
                 V[r * LD + rp[i]] = c * vp - sn * vq;
                 V[r * LD + q] = sn * vp + c * vq;
             }
@@ -454,13 +466,102 @@ __device__ __forceinline__ void psp_jacobi_pairs(double *A, double *V, int P, do
     }
 }
 
+// P x P product X^T Y (or X Y with TX = false), every thread its elements into
+// registers: element e = t + NT i of the result is (e / P, e % P).
+template <int MAXP, int NT, bool TX>
+__device__ __forceinline__ void psp_product(const double *X, const double *Y, int P, double (&out)[MAXP * MAXP / NT]) {
+    constexpr int LD = MAXP + 1;
+#pragma unroll
+    for (int i = 0; i < MAXP * MAXP / NT; i++) {
+        const int e = threadIdx.x + NT * i, r = e / P, c = e % P;
+        out[i] = 0.0;
+        if (e < P * P)
+            for (int k = 0; k < P; k++) out[i] = fma(X[TX ? k * LD + r : r * LD + k], Y[k * LD + c], out[i]);
+    }
+}
+template <int MAXP, int NT>
+__device__ __forceinline__ void psp_store(double *X, int P, const double (&v)[MAXP * MAXP / NT]) {
+    __syncthreads();   // every thread has read the operands
+#pragma unroll
+    for (int i = 0; i < MAXP * MAXP / NT; i++) {
+        const int e = threadIdx.x + NT * i;
+        if (e < P * P) X[e / P * (MAXP + 1) + e % P] = v[i];
+    }
+    __syncthreads();
+}
+
+// The FP64 sweeps from the eigenvectors of an FP32 solve: those, made orthogonal
+// in FP64 by two Newton-Schulz steps X <- X + X (1 - X^T X) / 2 (1e-6 -> 1e-12
+// -> rounding; E32 holds 1 - X^T X, whose own rounding the second step sees),
+// turn A into X^T A X with off-diagonal elements ~1e-6 of the others, and about
+// two FP64 sweeps are left of seven.  32 problems of 64 functions: 2.4 ms, 3.5 ms
+// in FP64 throughout.  Blocks of A stay blocks (zeros stay zero in every step).  An
+// FP32 solve that went wrong (numbers beyond its range) is dropped.
+template <int MAXP, int NT>
+__device__ __forceinline__ void psp_jacobi_refined(double *A, double *V, float *E32, int P, double *red, double *red2) {
+    constexpr int LD = MAXP + 1, R = MAXP * MAXP / NT;
+    const int t = threadIdx.x;
+    if (P >= 8) {
+        float *A32 = reinterpret_cast<float *>(V), *V32 = A32 + MAXP * LD;   // V is not needed yet
+        for (int e = t; e < P * P; e += NT) {
+            const int r = e / P, c = e % P;
+            A32[r * LD + c] = d2f(A[r * LD + c]);
+            V32[r * LD + c] = r == c ? 1.0f : 0.0f;
+        }
+        __syncthreads();
+        psp_jacobi_pairs<MAXP, NT, float>(A32, V32, P, 12, 1e-11f, reinterpret_cast<float *>(red), reinterpret_cast<float *>(red2));
+        __syncthreads();
+        double v[R];
+#pragma unroll
+        for (int i = 0; i < R; i++) {
+            const int e = t + NT * i;
+            v[i] = e < P * P ? f2d(V32[e / P * LD + e % P]) : 0.0;
+        }
+        psp_store<MAXP, NT>(V, P, v);
+        bool bad = false;
+        for (int step = 0; step < 2 && !bad; step++) {
+            psp_product<MAXP, NT, true>(V, V, P, v);
+#pragma unroll
+            for (int i = 0; i < R; i++) {
+                const int e = t + NT * i;
+                if (e >= P * P) continue;
+                const float d = d2f((e / P == e % P ? 1.0 : 0.0) - v[i]);
+                E32[e / P * LD + e % P] = d;
+                if (!(fabsf(d) < 1e-3f)) bad = true;
+            }
+            bad = __syncthreads_or(bad);
+            // X + X E / 2
+#pragma unroll
+            for (int i = 0; i < R; i++) {
+                const int e = t + NT * i, r = e / P, c = e % P;
+                v[i] = 0.0;
+                if (e >= P * P) continue;
+                float x = 0.0f;   // X E is at most 1e-3: FP32 keeps the first step's result to 1e-9, the second's to 1e-16
+                for (int k = 0; k < P; k++) x = fmaf(d2f(V[r * LD + k]), E32[k * LD + c], x);
+                v[i] = V[r * LD + c] + 0.5 * f2d(x);
+            }
+            psp_store<MAXP, NT>(V, P, v);
+        }
+        if (!bad) {
+            psp_product<MAXP, NT, false>(A, V, P, v);
+            psp_store<MAXP, NT>(A, P, v);
+            psp_product<MAXP, NT, true>(V, A, P, v);
+            psp_store<MAXP, NT>(A, P, v);
+        } else {
+            for (int e = t; e < P * P; e += NT) V[e / P * LD + e % P] = e / P == e % P ? 1.0 : 0.0;
+            __syncthreads();
+        }
+    }
+    psp_jacobi_pairs<MAXP, NT, double>(A, V, P, 40, 1e-26, red, red2);
+}
+
 // Per problem (one block of NT threads): H in the pair functions, its lowest
 // eigenvectors, written to the start slots 0..nv-1; the random start vector is
 // cleared on the P-space determinants.
 //
 // NT = 256 runs the round-robin sweeps, the others the cyclic ones.  The
 // round-robin order is the faster one for a 64-function problem (2.2 ms, against
-// 20.1 ms with one rotation at a time) and serves the whole spaces of an FP64
+// 20.1 ms with one rotation at a time; less after an FP32 solve) and serves the whole spaces of an FP64
 // solve, where a last-bit change of the start vector stays one.  With a
 // quantised contraction (FP64E and the mixed modes that end on it) such a change
 // turns up at the contraction's own level, ~5e-11 Eh, so those solves keep the
@@ -541,7 +642,7 @@ __device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict_
     __syncthreads();
     if constexpr (NT == 32) psp_jacobi_cyclic<MAXP>(A, V, P, red, red2);
     else if constexpr (NT == kPairThreads) psp_jacobi_ahead<MAXP>(A, V, P, red, red2);
-    else psp_jacobi_pairs<MAXP, NT>(A, V, P, red, red2);
+    else psp_jacobi_refined<MAXP, NT>(A, V, reinterpret_cast<float *>(psm + 2 * MAXP * LD), P, red, red2);
     __syncthreads();
     int nv, ns;
     start_block(p.ndim, max_space, false, &nv, &ns);
@@ -719,9 +820,10 @@ int launch_pspace_start(ifci_handle_t h, const DavBatch &b, const HdiagDesc *d_h
     constexpr int smem = 2 * kPsp * (kPsp + 1) * (int)sizeof(double);   // 65 KB
     if (whole && b.precision == IFCI_FP64) {
         static SmemOptIn opt;
-        IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel<kPsp, 256>, smem));
+        constexpr int smem_refined = smem + kPsp * (kPsp + 1) * (int)sizeof(float);   // 82 KB
+        IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel<kPsp, 256>, smem_refined));
         ProfScope ps(h, s, PK_PSPACE);
-        psp_solve_kernel<kPsp, 256><<<stride_grid(h->device, b.nprob, 3), 256, smem, s>>>(
+        psp_solve_kernel<kPsp, 256><<<stride_grid(h->device, b.nprob, 2), 256, smem_refined, s>>>(
             b.d_probs, d_hd, pidx, pcount, b.max_space, b.d_blk_energy, b.nprob);
         IFCI_LAUNCH_CHECK(h);
     } else if (whole) {
