@@ -23,6 +23,7 @@
 // unchanged scatter on G_a to get S, and add the transpose of S.  The FP64E
 // path (sigma_oz.cu) builds S in one kernel without D and G.
 #include <algorithm>
+#include <cstring>
 
 #include "fp64int.cuh"
 #include "sigma.cuh"
@@ -358,18 +359,23 @@ int upload_plan(ifci_handle_t h, SigmaPlan &plan, cudaStream_t s) {
     plan.d_tctiles = ws_take<WorkItem>(h, std::max<size_t>(1, plan.tctiles.size()));
     if (!plan.d_probs || !plan.d_items || !plan.d_tiles || !plan.d_tctiles)
         return set_error(h, IFCI_ERR_OOM, "sigma plan: workspace too small");
-    IFCI_CUDA_TRY(h, cudaMemcpyAsync(plan.d_probs, plan.probs.data(), plan.probs.size() * sizeof(SigmaProb),
-                                     cudaMemcpyHostToDevice, s));
-    if (!plan.items.empty())
-        IFCI_CUDA_TRY(h, cudaMemcpyAsync(plan.d_items, plan.items.data(), plan.items.size() * sizeof(WorkItem),
-                                         cudaMemcpyHostToDevice, s));
-    if (!plan.tiles.empty())
-        IFCI_CUDA_TRY(h, cudaMemcpyAsync(plan.d_tiles, plan.tiles.data(), plan.tiles.size() * sizeof(WorkItem),
-                                         cudaMemcpyHostToDevice, s));
-    if (!plan.tctiles.empty())
-        IFCI_CUDA_TRY(h, cudaMemcpyAsync(plan.d_tctiles, plan.tctiles.data(),
-                                         plan.tctiles.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, s));
-    return IFCI_OK;
+    // the arrays lie one after another: small plans go over in one copy (each costs
+    // the host ~2 us; a pageable copy of up to 64 KB is staged without waiting)
+    char *lo = (char *)plan.d_probs;
+    const size_t span = (char *)(plan.d_tctiles + plan.tctiles.size()) - lo;
+    if (span <= 65536 && span <= plan_device_bytes(plan) + 4 * ws_round(1)) {
+        std::vector<char> st(span);
+        auto put = [&](const void *dst, const void *src, size_t bytes) {
+            if (bytes) memcpy(st.data() + ((const char *)dst - lo), src, bytes);
+        };
+        put(plan.d_probs, plan.probs.data(), plan.probs.size() * sizeof(SigmaProb));
+        put(plan.d_items, plan.items.data(), plan.items.size() * sizeof(WorkItem));
+        put(plan.d_tiles, plan.tiles.data(), plan.tiles.size() * sizeof(WorkItem));
+        put(plan.d_tctiles, plan.tctiles.data(), plan.tctiles.size() * sizeof(WorkItem));
+        IFCI_CUDA_TRY(h, cudaMemcpyAsync(lo, st.data(), span, cudaMemcpyHostToDevice, s));
+        return IFCI_OK;
+    }
+    return upload_plan_to(h, plan, s);
 }
 
 // Copies the plan's descriptor arrays to the device arrays the caller set in
