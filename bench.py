@@ -40,7 +40,7 @@ METRIC = "iFCI increments/s & sigma TFLOP/s, 1 GB300, batched+mixed vs plain FP6
 # dram__bytes_read.sum + dram__bytes_write.sum of one oz_sigma_kernel launch on
 # CAS(6e,18o) per determinant (ncu capture of one FP64E sigma); set to None
 # whenever that kernel changes until it is captured again
-OZ_DRAM_BYTES_PER_DET = 19.46e6 / 665856
+OZ_DRAM_BYTES_PER_DET = None
 UNIT = "increments/s"
 
 
