@@ -59,9 +59,13 @@
 // reductions (3.4 clocks a warp).  Sixteen warps share it, twelve for the beta
 // sums and four for the alpha sums; eight warps with both took 612 us.
 //
-// Measured, one sigma: CAS(6e,18o) 403 us (1282 us contraction + 254 us scatter
-// before), CAS(8e,20o) 29.4 ms (96.0 + 9.8 ms in three waves of 16 GB, now 0.7 GB
-// at once).
+// The producers' copies go out in batches of ten and eight after their row
+// numbers are read: one row number and one copy at a time took a warp 240 clocks
+// a copy, and the W chunks of CAS(8e,20o), reloaded for every tile, bounded it.
+//
+// Measured, one sigma: CAS(6e,18o) 382 us (1282 us contraction + 254 us scatter
+// before), CAS(8e,20o) 17.0 ms (96.0 + 9.8 ms in three waves of 16 GB, now 0.7 GB
+// at once; 29.4 ms with the copies one at a time).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -554,12 +558,22 @@ oz_sigma_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict_
                 if (!okA[an & 1]) { ok = false; break; }
                 const uint32_t dst = smem_u32(Asm) + slot * stageA + (ch >> 3) * (uint32_t)Kp * 128;
                 const int col = mt * kTM + ch * 8;
-                for (int j = 0; j < kS; j++)
-                    for (int k = t >> 4; k < Kp; k += 2 * kAWarps) {
-                        const bool lv = k < kc && col < nstr;
-                        const __half *s = lv ? src + ((size_t)lstA[k] + (size_t)j * nstr) * ldq + col : Q;
-                        cp_async16(dst + (uint32_t)(j * Kp * 256 + k * 128 + (((ch & 7) ^ (k & 7)) << 4)), s, lv);
+                // two K rows (of this thread's Kp / 8, an even number) and all digits at a time
+                const size_t plane = (size_t)nstr * ldq;
+                const bool in = col < nstr;
+                for (int k0 = t >> 4; k0 < Kp; k0 += 4 * kAWarps) {
+                    const int k1 = k0 + 2 * kAWarps, r0 = lstA[k0], r1 = lstA[k1];
+                    const bool lv0 = in && k0 < kc, lv1 = in && k1 < kc;
+                    const __half *s0 = lv0 ? src + (size_t)r0 * ldq + col : Q, *s1 = lv1 ? src + (size_t)r1 * ldq + col : Q;
+                    const size_t p0 = lv0 ? plane : 0, p1 = lv1 ? plane : 0;
+                    const uint32_t d0 = dst + (uint32_t)(k0 * 128 + (((ch & 7) ^ (k0 & 7)) << 4));
+                    const uint32_t d1 = dst + (uint32_t)(k1 * 128 + (((ch & 7) ^ (k1 & 7)) << 4));
+#pragma unroll
+                    for (int j = 0; j < kS; j++) {
+                        cp_async16(d0 + (uint32_t)(j * Kp * 256), s0 + j * p0, lv0);
+                        cp_async16(d1 + (uint32_t)(j * Kp * 256), s1 + j * p1, lv1);
                     }
+                }
                 if (t == 0) kp_of[slot] = Kp;
                 cp_async_done();
                 mbar_arrive(smem_u32(&b_fullA[slot]));
@@ -589,10 +603,17 @@ oz_sigma_kernel(const SigmaProb *__restrict__ probs, const WorkItem *__restrict_
                     const int n8 = lane;                       // 16-byte chunk of a row (5 w / 8 <= 30 of them)
                     const uint32_t dst = smem_u32(Wsm) + slot * stageW + (uint32_t)(n8 >> 3) * Kp * 128;
                     if (n8 < kS * w / 8)
-                        for (int k = wi; k < Kp; k += kWWarps) {
-                            const bool lv = k < kc;
-                            const uint8_t *s = lv ? cimg + (size_t)lstW[k] * 10 * w + n8 * 16 : img;
-                            cp_async16(dst + (uint32_t)(k * 128 + (((n8 & 7) ^ (k & 7)) << 4)), s, lv);
+                        for (int k0 = wi; k0 < Kp; k0 += 8 * kWWarps) {   // Kp / 2 rows a warp, a multiple of 8
+                            int b[8];
+#pragma unroll
+                            for (int u = 0; u < 8; u++) b[u] = lstW[k0 + u * kWWarps];
+#pragma unroll
+                            for (int u = 0; u < 8; u++) {
+                                const int k = k0 + u * kWWarps;
+                                const bool lv = k < kc;
+                                cp_async16(dst + (uint32_t)(k * 128 + (((n8 & 7) ^ (k & 7)) << 4)),
+                                           lv ? cimg + (uint32_t)(b[u] * 10 * w) + n8 * 16 : img, lv);
+                            }
                         }
                     cp_async_done();
                     mbar_arrive(smem_u32(&b_fullW[slot]));
