@@ -88,7 +88,12 @@ constexpr int kOzTmemCols = 512;
 constexpr int kMaxK = 112;                  // contracted pairs of one string, rounded to 16
 constexpr int kMaxNp = 304;                 // pairs (norb <= 24)
 constexpr int kMaxStrings = 32767;          // 16-bit map entries (sign << 15 | J), 0xFFFF = none
-constexpr int kNarrowK = 51;                // up to here a level stays below 2^22 and a row sum of 26-bit words below 2^32
+// Longest lists of the narrow epilogue.  A digit is at most 128, the top one of c
+// at most 65, so a level over K rows is at most K (65 + 4 128) 128: below 2^22 up
+// to K = 56, as is a row sum of K 26-bit words below 2^32 and of K T's below 2^57.
+// Lists of 54 to 56 entries: 1 to 8 % off a sigma against the wide form (6e,20o:
+// 1044 us, 973 us).  A third form for up to 72, with four levels narrow, gave 1 %.
+constexpr int kNarrowK = 56;
 constexpr int kMaxW = 8;                    // W chunk buffers
 constexpr int kBetaWarps = 12, kAlphaWarps = 4, kAWarps = 4, kWWarps = 2;
 constexpr int kEpiWarps = kBetaWarps + kAlphaWarps;
