@@ -287,7 +287,7 @@ int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision
         if (tc) {
             // one tile = up to 128 determinants of whole alpha rows x all pairs (sigma_tc.cu)
             size_t before = plan.tctiles.size();
-            tcg::append_row_tiles(plan.tctiles, (int)i, 0, p.nstr);
+            tcg::append_row_tiles(plan.tctiles, (int)i, p.nstr);
             w.ntc += (int)(plan.tctiles.size() - before);
         } else {
             for (int m0 = 0; m0 < p.np; m0 += kGemmTM)

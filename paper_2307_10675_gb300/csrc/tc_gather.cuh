@@ -47,18 +47,14 @@ inline int rows_per_tile(int nstr) {
     return rmax > kRows ? kRows : rmax;
 }
 
-// Host: the row-aligned tiles of alpha rows [r0, r1) of one problem (all rows
-// when r1 < 0), in order; r0 and r1 are multiples of rows_per_tile(nstr)
-// (r1 may be nstr).
-inline void append_row_tiles(std::vector<WorkItem> &out, int prob, int sub, int nstr, int r0 = 0, int r1 = -1) {
-    if (r1 < 0) r1 = nstr;
+// Host: the row-aligned tiles of one problem, in order.
+inline void append_row_tiles(std::vector<WorkItem> &out, int prob, int nstr) {
     if (nstr >= kTileDets) {
-        for (int ka = r0; ka < r1; ka++)
-            for (int kb0 = 0; kb0 < nstr; kb0 += kTileDets)
-                out.push_back(WorkItem{prob, sub, (long long)ka * nstr + kb0});
+        for (int ka = 0; ka < nstr; ka++)
+            for (int kb0 = 0; kb0 < nstr; kb0 += kTileDets) out.push_back(WorkItem{prob, 0, (long long)ka * nstr + kb0});
     } else {
         const int rmax = rows_per_tile(nstr);
-        for (int ka0 = r0; ka0 < r1; ka0 += rmax) out.push_back(WorkItem{prob, sub, (long long)ka0 * nstr});
+        for (int ka0 = 0; ka0 < nstr; ka0 += rmax) out.push_back(WorkItem{prob, 0, (long long)ka0 * nstr});
     }
 }
 
@@ -74,13 +70,6 @@ __device__ __forceinline__ int claim_tile(int *counter, const SigmaProb *probs, 
     }
 }
 
-inline long long row_tile_count(int nstr) {
-    if (nstr >= kTileDets) return (long long)nstr * ((nstr + kTileDets - 1) / kTileDets);
-    int rmax = kTileDets / nstr;
-    if (rmax > kRows) rmax = kRows;
-    return (nstr + rmax - 1) / rmax;
-}
-
 }  // namespace tcg
 }  // namespace ifci
 
@@ -88,7 +77,7 @@ namespace ifci {
 namespace tcg {
 
 // Sum of the alpha and beta contributions of determinant (ka, kb) to the 16
-// pairs [16 b, 16 b + 16): x[i] += sign * c.  T = float or long long.
+// pairs [16 b, 16 b + 16): x[i] += sign * c.
 template <typename T>
 __device__ __forceinline__ void gather_block16(const SigmaProb &p, const T *__restrict__ c, int ka, int kb, int b,
                                                T (&x)[16]) {
