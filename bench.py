@@ -40,7 +40,7 @@ METRIC = "iFCI increments/s & sigma TFLOP/s, 1 GB300, batched+mixed vs plain FP6
 # dram__bytes_read.sum + dram__bytes_write.sum of one oz_sigma_kernel launch on
 # CAS(6e,18o) per determinant (ncu capture of one FP64E sigma); set to None
 # whenever that kernel changes until it is captured again
-OZ_DRAM_BYTES_PER_DET = None
+OZ_DRAM_BYTES_PER_DET = 19.46e6 / 665856
 UNIT = "increments/s"
 
 
@@ -488,7 +488,7 @@ def main():
         hi_ms = prof["contract_hi"][0]
         ach = flops_step / ((lo_ms + hi_ms) / 1000.0) / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": bf, "unit": "TFLOP/s", "frac": ach / bf,
-                "traffic": None, "kernel": "tc_contract_bf16_kernel + oz_contract_kernel", "peak_source": bf_src}
+                "traffic": None, "kernel": "tc_contract_bf16_kernel + oz_sigma_kernel", "peak_source": bf_src}
         dtype = args.precision + "+f64"
 
     line = {
