@@ -98,6 +98,8 @@ int dav_run(ifci_handle_t h, std::vector<Unit> &units, const std::vector<BlockSp
     b.keep = std::min(kKeep, ms - 2);
     b.precision = o.precision;
     b.hi_precision = hi_prec;
+    b.any_order = o.precision == IFCI_FP64 ||
+                  std::all_of(units.begin(), units.end(), [](const Unit &u) { return u.spec.any_order; });
     b.max_iter = o.max_iter;
     b.graph_iters = o.graph_iters > 0 ? o.graph_iters : 0;
     b.e_tol = o.e_tol;
@@ -881,6 +883,7 @@ int ifci_davidson_batched(ifci_handle_t h, int nprob, const ifci_problem_t *prob
         if (!p.h1 || !p.eri || p.nelec_spin < 1 || ifci_string_counts(p.norb, p.nelec_spin, nullptr, nullptr))
             return set_error(h, IFCI_ERR_INVALID_ARG, "davidson_batched: problem %d invalid", i);
         specs.push_back(ProbSpec{p.norb, p.nelec_spin, p.h1, p.eri, p.e_core, p.c_out});
+        specs.back().any_order = true;
     }
     IFCI_TRY(check_opts(h, o));
     IFCI_CUDA_TRY(h, cudaSetDevice(h->device));

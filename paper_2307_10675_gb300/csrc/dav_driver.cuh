@@ -20,6 +20,11 @@ struct ProbSpec {
     const double *seed = nullptr;
     const unsigned char *mask = nullptr;
     long long ndim = 0;
+    // its energy is a result by itself: the small eigenproblems may take the faster
+    // order of rotations, whose other rounding a quantised sigma turns into
+    // ~1e-10 Eh.  An expansion, which takes differences of such energies, and HBCI
+    // keep the serial order.
+    bool any_order = false;
 };
 
 // coupling graph of one problem's orbitals (sectors.cu)

@@ -328,10 +328,11 @@ __device__ void jacobi_warp(double *A, double *V, int k, int lane) {
 // is one lane's two multiplies and two FMAs; the (pair, row)s of V follow while
 // the next step's rotations are derived (those of step `step` in buffer step & 1).
 // The chain of a step (~1200 clk to derive, 2 x 256 to mix) bounds it: 32 problems
-// of up to 12 vectors take 62 us on average, 194 us one rotation at a time.  Only
-// FP64 solves take it: with a quantised sigma another rounding here turns up at
-// the contraction's own level (energies of selected spaces moved by 7e-10 of
-// themselves), so those keep the serial order and every bit.
+// of up to 12 vectors take 62 us on average, 194 us one rotation at a time.  FP64
+// solves and direct batches take it; in expansions and HBCI with a quantised
+// sigma another rounding here turns up at the contraction's own level (energies
+// of selected spaces moved by 7e-10 of themselves), so those keep the serial
+// order and every bit.
 constexpr int kPairSolveThreads = 128;
 
 template <int LD>
@@ -1081,7 +1082,7 @@ static int dav_step(ifci_handle_t h, DavBatch &b, SigmaPlan &hi_plan, SigmaPlan 
     const bool small = b.max_space <= kSmallSpace;
     (small ? dots_kernel<kSmallSpace> : dots_kernel<kMaxSpace>)<<<gi, 256, 0, s>>>(b.d_probs, b.d_state, b.d_vitems, b.d_part, nitem);
     IFCI_LAUNCH_CHECK(h);
-    if (b.precision == IFCI_FP64)
+    if (b.any_order)
         solve_pairs_kernel<<<stride_grid(h->device, b.nprob, 16), kPairSolveThreads, 0, s>>>(b.d_probs, b.d_state, b.d_part,
                                                                                      b.d_gs, b.d_y, b.nprob);
     else if (b.max_space <= 16)

@@ -111,6 +111,7 @@ struct DavBatch {
     double *d_blk_energy = nullptr;   // [nprob][2] lowest eigenvalue of the two lowest P-space blocks
     int precision = IFCI_FP64;
     int hi_precision = IFCI_FP64;
+    bool any_order = false;       // small eigenproblems in round-robin order (FP64, or ProbSpec::any_order)
     int max_iter = 100;
     double e_tol = 1e-10, r_tol = 1e-6;
     std::vector<DavProb> probs;

@@ -561,15 +561,19 @@ __device__ __forceinline__ void psp_jacobi_refined(double *A, double *V, float *
 //
 // NT = 256 runs the round-robin sweeps, the others the cyclic ones.  The
 // round-robin order is the faster one for a 64-function problem (2.2 ms, against
-// 20.1 ms with one rotation at a time; less after an FP32 solve) and serves the whole spaces of an FP64
-// solve, where a last-bit change of the start vector stays one.  With a
-// quantised contraction (FP64E and the mixed modes that end on it) such a change
-// turns up at the contraction's own level, ~5e-11 Eh, so those solves keep the
-// order of rotations, and with it every bit of their start vectors, on five
-// warps a problem: 64 functions 20.1 ms on one warp, 13.8 ms; 298 such problems
-// at once 21.9 ms, 15.7 ms; the P-space solves of an expansion of 298 sets
-// 58.9 ms, 42.9 ms.  So do the blocks of sectored spaces (MAXP = 24), which come
-// by the hundred thousand and share an SM sixteen at a time, a warp each.
+// 20.1 ms with one rotation at a time; less after an FP32 solve) and serves the
+// whole spaces of FP64 solves, where a last-bit change of the start vector stays
+// one, and of direct batches in every precision, whose energies it moves by
+// 1e-13 (FP64E) to 3e-11 (mixed) of themselves (a batch of two-body spaces in
+// FP64E: 18.9 ms, 4.2 ms with the Rayleigh-Ritz problems in that order too).  In
+// an expansion with a quantised contraction (FP64E and the mixed modes that end
+// on it) such a change turns up at the contraction's own level, ~5e-11 Eh, in
+// increments that are differences of energies, so those and HBCI keep the order
+// of rotations, and with it every bit of their start vectors, on five warps a
+// problem: 64 functions 20.1 ms on one warp, 13.8 ms; 298 such problems at once
+// 21.9 ms, 15.7 ms; the P-space solves of an expansion of 298 sets 58.9 ms,
+// 42.9 ms.  So do the blocks of sectored spaces (MAXP = 24), which come by the
+// hundred thousand and share an SM sixteen at a time, a warp each.
 template <int MAXP, int NT>
 __device__ __forceinline__ void psp_solve_kernel_body(const DavProb *__restrict__ probs, const HdiagDesc *__restrict__ hdd, const long long *__restrict__ pidx,
                  const int *__restrict__ pcount, int max_space, double *__restrict__ blk_energy, int w_) {
@@ -818,7 +822,7 @@ int launch_pspace_start(ifci_handle_t h, const DavBatch &b, const HdiagDesc *d_h
         sector = sector || (p.gc && !p.seed);
     }
     constexpr int smem = 2 * kPsp * (kPsp + 1) * (int)sizeof(double);   // 65 KB
-    if (whole && b.precision == IFCI_FP64) {
+    if (whole && b.any_order) {
         static SmemOptIn opt;
         constexpr int smem_refined = smem + kPsp * (kPsp + 1) * (int)sizeof(float);   // 82 KB
         IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, psp_solve_kernel<kPsp, 256>, smem_refined));
