@@ -37,6 +37,8 @@ int ifci_sigma(ifci_handle_t h, const ifci_strings_t *str, const double *h1, con
 
     if (precision == IFCI_FP64) {
         // string Hamiltonian, then one fused kernel; descriptors by value
+        if (!sigma64_supported(np, nstr, nexc))
+            return set_error(h, IFCI_ERR_OOM, "ifci_sigma: %d strings are beyond the shared memory of an SM", nstr);
         const int nnz = string_h_nnz(n, str->nelec_spin);
         IFCI_TRY(ws_reserve(h, ws_round((size_t)nnz * nstr * 8) + ws_round((size_t)nnz * nstr * 4)));
         double *hval = ws_take<double>(h, (size_t)nnz * nstr);

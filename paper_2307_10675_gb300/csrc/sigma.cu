@@ -266,6 +266,8 @@ int plan_sigma(ifci_handle_t h, SigmaPlan &plan, long long budget, int precision
             continue;
         }
         if (precision == IFCI_FP64) {   // no intermediates: one item per alpha string, one wave
+            if (!sigma64_supported(p.np, p.nstr, p.nexc))
+                return set_error(h, IFCI_ERR_OOM, "FP64 sigma: %d strings are beyond the shared memory of an SM", p.nstr);
             w.nprob++;
             w.nitem += p.nstr;
             continue;

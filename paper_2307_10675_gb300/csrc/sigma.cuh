@@ -107,6 +107,7 @@ struct StringHDesc {
     int *idx;                // [nnz][nstr] or nullptr
 };
 int string_h_nnz(int n, int m);
+bool sigma64_supported(int np, int nstr, int nexc);   // one excitation of every string fits an SM's shared memory
 int launch_string_h(ifci_handle_t h, const StringHDesc &one, cudaStream_t s);
 int launch_string_h_batch(ifci_handle_t h, const StringHDesc *d_desc, const WorkItem *d_items, int nitem, cudaStream_t s);
 int run_sigma64_one(ifci_handle_t h, const SigmaProb &p, cudaStream_t s);

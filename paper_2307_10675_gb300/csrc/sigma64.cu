@@ -207,15 +207,15 @@ static int string_h_parts(ifci_handle_t h, int nblk, int nnz) {
 }
 
 int cap64(const SigmaProb *probs, int nprob) {
-    for (int cap : {kCapSmall, kCapMid, kCapLarge}) {
+    for (int cap : {kCapSmall, kCapMid}) {
         bool ok = true;
         for (int i = 0; i < nprob && ok; i++) {
             const SigmaProb &p = probs[i];
-            ok = fit64(p.nstr, p.np, p.nexc, cap) >= (cap == kCapLarge ? 1 : std::min(p.nexc, 4));
+            ok = fit64(p.nstr, p.np, p.nexc, cap) >= std::min(p.nexc, 4);
         }
         if (ok) return cap;
     }
-    return 0;
+    return kCapLarge;
 }
 
 }  // namespace
@@ -226,6 +226,8 @@ StringBinom string_binom() {
         for (int j = 0; j < 32; j++) B.c[i][j] = (int)std::min<long long>(binom(i, j), 0x7fffffff);
     return B;
 }
+
+bool sigma64_supported(int np, int nstr, int nexc) { return fit64(nstr, np, nexc, kCapLarge) >= 1; }
 
 int string_h_nnz(int n, int m) { return 1 + m * (n - m) + m * (m - 1) / 2 * ((n - m) * (n - m - 1) / 2); }
 
@@ -252,14 +254,9 @@ static int threads64(ifci_handle_t h, int nstr, int nitem) {
     return std::min(most, (nstr + 31) / 32 * 32);
 }
 
-static int no_room(ifci_handle_t h) {
-    return set_error(h, IFCI_ERR_OOM, "FP64 sigma: strings beyond the shared memory of an SM");
-}
-
 // One problem, its descriptor passed by value (no copies to the device).
 int run_sigma64_one(ifci_handle_t h, const SigmaProb &p, cudaStream_t s) {
     const int cap = cap64(&p, 1);
-    if (cap == 0) return no_room(h);
     static SmemOptIn opt;
     IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, sigma64_one_kernel, cap * (int)sizeof(double)));
     ProfScope ps(h, s, PK_CONTRACT);
@@ -270,7 +267,6 @@ int run_sigma64_one(ifci_handle_t h, const SigmaProb &p, cudaStream_t s) {
 
 int run_sigma64(ifci_handle_t h, const SigmaPlan &plan, const SigmaWave &w, cudaStream_t s) {
     const int cap = cap64(plan.probs.data() + w.prob0, w.nprob);
-    if (cap == 0) return no_room(h);
     static SmemOptIn opt;
     IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, sigma64_kernel, cap * (int)sizeof(double)));
     ProfScope ps(h, s, PK_CONTRACT);
