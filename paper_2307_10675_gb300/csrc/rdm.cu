@@ -26,7 +26,8 @@ namespace ifci {
 namespace {
 
 constexpr int kSyrkT = 16;          // SYRK output tile
-constexpr int kSyrkChunk = 512;     // determinants per split-K chunk
+constexpr int kSyrkChunk = 512;     // fewest determinants of a split-K chunk
+constexpr int kSyrkJobsPerSm = 64;  // jobs a wave is cut into, about, if it has more determinants than that
 constexpr int kSyrkWarps = 4, kSyrkPer = 4;             // warps of a block, tiles each keeps in registers
 constexpr int kSyrkGroup = kSyrkWarps * kSyrkPer;       // tiles of one job
 constexpr int kSyrkK = 16;          // determinants staged at a time
@@ -90,13 +91,13 @@ __global__ void __launch_bounds__(256) rdm_gather_kernel(const RdmProb *__restri
 // 16,384, of which a gradient over 63 sets had fewer than two per SM).  The
 // gradient of 63 sets up to CAS(6e,12o): 18.2 ms before, 1.6 ms.
 __global__ void __launch_bounds__(32 * kSyrkWarps) rdm_syrk_kernel(const RdmProb *__restrict__ probs,
-                                                                   const SyrkJob *__restrict__ jobs,
+                                                                   const SyrkJob *__restrict__ jobs, int chunk,
                                                                    const double *__restrict__ D, double *__restrict__ part) {
     const SyrkJob jb = jobs[blockIdx.x];
     const RdmProb &p = probs[jb.prob];
     const int rows = p.np + 1, T = syrk_side(p.np), nt = syrk_tiles(p.np), ld = T * kSyrkT + 2;
     const long long ndet = p.ndet;
-    const long long k0 = (long long)(jb.chunk - p.chunk0) * kSyrkChunk, k1 = min(ndet, k0 + kSyrkChunk);
+    const long long k0 = (long long)(jb.chunk - p.chunk0) * chunk, k1 = min(ndet, k0 + chunk);
     const double *Dp = D + p.doff;
     extern __shared__ double Ds[];   // [kSyrkK][ld]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -270,6 +271,20 @@ long long expansion_weight(int nbody, int k, int max_order) {
     return ((max_order - k) & 1) ? -c : c;
 }
 
+// Determinants of a split-K chunk for problems [first, last): 512, which spreads
+// small sets over the chip, while that makes at most 64 jobs per SM; then the
+// least multiple of it that does.  A job leaves 32 KB of partial sums, which the
+// reduction adds up one chunk after the other: with 512 throughout, CAS(8e,20o)
+// held 10.5 GB of them next to 39.6 GB of rows and took 1,191 ms (1,067 ms so,
+// 0.3 GB), CAS(8e,16o) 0.64 GB and 74.9 ms (0.32 GB, 70.7 ms).  A wave of up to
+// 64 jobs per SM, such as 63 sets up to CAS(6e,12o), keeps 512.
+int syrk_chunk(const std::vector<RdmProb> &probs, int first, int last, int sms) {
+    long long jobs = 0;
+    for (int x = first; x < last; x++) jobs += (probs[x].ndet + kSyrkChunk - 1) / kSyrkChunk * syrk_groups(probs[x].np);
+    const long long most = (long long)kSyrkJobsPerSm * sms;
+    return (int)(kSyrkChunk * std::max(1ll, (jobs + most - 1) / most));
+}
+
 }  // namespace
 
 }  // namespace ifci
@@ -391,8 +406,9 @@ extern "C" int ifci_rdm_backward(ifci_handle_t h, const ifci_system_t *sys, int 
     size_t wave_max = 0;
     for (auto &wv : waves) {
         long long items = 0, jobs = 0;
+        const int chunk = syrk_chunk(probs, wv.first, wv.second, device_sm_count(h->device));
         for (int x = wv.first; x < wv.second; x++) {
-            const long long nch = (probs[x].ndet + kSyrkChunk - 1) / kSyrkChunk;
+            const long long nch = (probs[x].ndet + chunk - 1) / chunk;
             items += (probs[x].ndet + 255) / 256;
             jobs += nch * syrk_groups(probs[x].np);
         }
@@ -440,6 +456,7 @@ extern "C" int ifci_rdm_backward(ifci_handle_t h, const ifci_system_t *sys, int 
         std::vector<SyrkJob> jobs;
         std::vector<int> job0;
         long long doff = 0;
+        const int len = syrk_chunk(probs, wv.first, wv.second, device_sm_count(h->device));
         int chunk = 0, max_np = 0;
         for (int x = wv.first; x < wv.second; x++) {
             RdmProb &r = probs[x];
@@ -448,7 +465,7 @@ extern "C" int ifci_rdm_backward(ifci_handle_t h, const ifci_system_t *sys, int 
             for (long long s0 = 0; s0 < r.ndet; s0 += 256) items.push_back(WorkItem{x - wv.first, 0, s0});
             const int ng = syrk_groups(r.np);
             max_np = std::max(max_np, r.np);
-            r.nchunk = (int)((r.ndet + kSyrkChunk - 1) / kSyrkChunk);
+            r.nchunk = (int)((r.ndet + len - 1) / len);
             r.chunk0 = chunk;
             job0.push_back((int)jobs.size());
             for (int ch = 0; ch < r.nchunk; ch++)
@@ -471,7 +488,7 @@ extern "C" int ifci_rdm_backward(ifci_handle_t h, const ifci_system_t *sys, int 
         const int smem = kSyrkK * (syrk_side(max_np) * kSyrkT + 2) * (int)sizeof(double);   // 64 KB at 496 pairs
         static SmemOptIn opt;
         IFCI_CUDA_TRY(h, ensure_smem(opt, h->device, rdm_syrk_kernel, smem));
-        rdm_syrk_kernel<<<(int)jobs.size(), 32 * kSyrkWarps, smem, s>>>(d_wp, d_jobs, D, part);
+        rdm_syrk_kernel<<<(int)jobs.size(), 32 * kSyrkWarps, smem, s>>>(d_wp, d_jobs, len, D, part);
         IFCI_LAUNCH_CHECK(h);
         rdm_reduce_kernel<<<dim3(nw, std::max(1, std::min(32, (max_np + 1) * (max_np + 1) / 256))), 256, 0, s>>>(d_wp, d_job0, part);
         IFCI_LAUNCH_CHECK(h);
