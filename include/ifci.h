@@ -319,10 +319,24 @@ void ifci_davidson_default_opts(ifci_davidson_opts_t *opts);
  *   energies : host double[nprob], eigenvalues including e_core.
  *   iters    : host int[nprob] or NULL, sigma builds per problem.
  *   status   : host int[nprob] or NULL, IFCI_OK or IFCI_ERR_NOT_CONVERGED.
+ * In a quantised or mixed precision the last digits of the energies (up to
+ * ~1e-10 Eh) are those of the order in which the small eigenproblems are
+ * rotated, and this call takes another order than ifci_increments does.  The
+ * two are equally accurate; where differences of energies are taken with those
+ * of ifci_increments, use ifci_davidson_expansion.
  * Synchronous.  Returns NOT_CONVERGED if any problem did not converge. */
 int ifci_davidson_batched(ifci_handle_t handle, int nprob, const ifci_problem_t *probs,
                           const ifci_davidson_opts_t *opts, double *energies, int *iters,
                           int *status, ifci_stream_t stream);
+
+/* ifci_davidson_expansion — the same batch solved as ifci_increments solves its
+ * body sets: the small eigenproblems in the serial order, so the energies are
+ * those of ifci_increments bit for bit.  Slower than ifci_davidson_batched
+ * where many small problems run in a quantised or mixed precision; the same
+ * call in FP64. */
+int ifci_davidson_expansion(ifci_handle_t handle, int nprob, const ifci_problem_t *probs,
+                            const ifci_davidson_opts_t *opts, double *energies, int *iters,
+                            int *status, ifci_stream_t stream);
 
 /* ---------------------------------------------------------------- HBCI */
 

@@ -30,7 +30,7 @@ EXPORTS = [
     "ifci_frozen_core", "ifci_davidson_default_opts", "ifci_davidson_batched", "ifci_num_subsets",
     "ifci_increments", "ifci_rdm_backward", "ifci_profile_enable", "ifci_profile_read",
     "ifci_sigma_noalloc", "ifci_sigma_noalloc_max_bytes", "ifci_h_elements", "ifci_wait_selftest",
-    "ifci_hbci_batched",
+    "ifci_hbci_batched", "ifci_davidson_expansion",
 ]
 PROFILE_KINDS = {"gather": 0, "contract": 1, "scatter": 2, "vector": 3, "other": 4, "contract_hi": 5, "setup": 6, "pspace": 7}
 
@@ -98,6 +98,7 @@ def load(build_if_missing: bool = True):
     L.ifci_davidson_default_opts.restype = None
     L.ifci_davidson_batched.argtypes = [H, c_int, ctypes.POINTER(Problem), ctypes.POINTER(DavidsonOpts),
                                         c_double_p, c_int_p, c_int_p, c_void_p]
+    L.ifci_davidson_expansion.argtypes = L.ifci_davidson_batched.argtypes
     L.ifci_hbci_batched.argtypes = [H, c_int, ctypes.POINTER(Problem), ctypes.POINTER(c_ll),
                                     ctypes.POINTER(DavidsonOpts), ctypes.POINTER(HbciOpts), c_double_p, c_double_p,
                                     ctypes.POINTER(c_ll), c_int_p, c_int_p, c_void_p]

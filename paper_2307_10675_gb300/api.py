@@ -259,6 +259,15 @@ class CIProblem:
 
 
 def ifci_davidson_batched(handle: Handle, problems: List[CIProblem], opts=None, stream=None, allow_unconverged=False):
+    return _davidson(_lib().ifci_davidson_batched, handle, problems, opts, stream, allow_unconverged)
+
+
+def ifci_davidson_expansion(handle: Handle, problems: List[CIProblem], opts=None, stream=None, allow_unconverged=False):
+    """The batch solved as ``ifci_increments`` solves its body sets (include/ifci.h)."""
+    return _davidson(_lib().ifci_davidson_expansion, handle, problems, opts, stream, allow_unconverged)
+
+
+def _davidson(entry, handle, problems, opts, stream, allow_unconverged):
     n = len(problems)
     arr = (_capi.Problem * max(n, 1))()
     for i, p in enumerate(problems):
@@ -268,9 +277,8 @@ def ifci_davidson_batched(handle: Handle, problems: List[CIProblem], opts=None, 
     it = np.zeros(n, dtype=np.int32)
     st = np.zeros(n, dtype=np.int32)
     o = opts or davidson_opts()
-    rc = _lib().ifci_davidson_batched(handle.ptr, n, arr, ctypes.byref(o), e.ctypes.data_as(_capi.c_double_p),
-                                      it.ctypes.data_as(_capi.c_int_p), st.ctypes.data_as(_capi.c_int_p),
-                                      _stream(stream))
+    rc = entry(handle.ptr, n, arr, ctypes.byref(o), e.ctypes.data_as(_capi.c_double_p),
+               it.ctypes.data_as(_capi.c_int_p), st.ctypes.data_as(_capi.c_int_p), _stream(stream))
     handle.check(rc, allow=(IFCI_ERR_NOT_CONVERGED,) if allow_unconverged else ())
     return e, it, st
 

@@ -17,8 +17,8 @@ workload and GPU are the parameters of the batched solve itself:
   one by one), which removes launch latency for batches of small problems.
 
 Every candidate is timed on the same seeded sample of the workload's CI
-problems (their frozen-body Hamiltonians, one ``ifci_davidson_batched`` call
-each, after one untimed call); a candidate whose energies differ from the
+problems (their frozen-body Hamiltonians, one ``ifci_davidson_expansion`` call
+each, which solves them as an expansion does, after one untimed call); a candidate whose energies differ from the
 first candidate's by more than ``tol`` is rejected.  The choice is cached in
 a JSON file keyed by the GPU name and a signature of the workload, and the
 search is coordinate-wise (one parameter at a time, the others at their
@@ -62,13 +62,13 @@ def _problems(handle: api.Handle, system: api.SystemArrays, sets):
 
 def _time(handle, probs, opts, repeats=1, warm=True):
     if warm:
-        api.ifci_davidson_batched(handle, probs, opts, allow_unconverged=True)   # set-up (workspace growth)
+        api.ifci_davidson_expansion(handle, probs, opts, allow_unconverged=True)   # set-up (workspace growth)
         torch.cuda.synchronize()
     best = float("inf")
     e = None
     for _ in range(repeats):
         t0 = time.perf_counter()
-        e, _, st = api.ifci_davidson_batched(handle, probs, opts, allow_unconverged=True)
+        e, _, st = api.ifci_davidson_expansion(handle, probs, opts, allow_unconverged=True)
         torch.cuda.synchronize()
         best = min(best, time.perf_counter() - t0)
         if np.any(st != 0):

@@ -868,8 +868,8 @@ void ifci_davidson_default_opts(ifci_davidson_opts_t *o) {
     o->hbci_eps2 = 1e-6;
 }
 
-int ifci_davidson_batched(ifci_handle_t h, int nprob, const ifci_problem_t *probs, const ifci_davidson_opts_t *opts,
-                          double *energies, int *iters, int *status, ifci_stream_t stream) {
+static int solve_batch(ifci_handle_t h, int nprob, const ifci_problem_t *probs, const ifci_davidson_opts_t *opts,
+                       bool any_order, double *energies, int *iters, int *status, ifci_stream_t stream) {
     using namespace ifci;
     if (!h) return IFCI_ERR_INVALID_ARG;
     if (nprob < 0 || (nprob > 0 && (!probs || !energies)))
@@ -883,11 +883,21 @@ int ifci_davidson_batched(ifci_handle_t h, int nprob, const ifci_problem_t *prob
         if (!p.h1 || !p.eri || p.nelec_spin < 1 || ifci_string_counts(p.norb, p.nelec_spin, nullptr, nullptr))
             return set_error(h, IFCI_ERR_INVALID_ARG, "davidson_batched: problem %d invalid", i);
         specs.push_back(ProbSpec{p.norb, p.nelec_spin, p.h1, p.eri, p.e_core, p.c_out});
-        specs.back().any_order = true;
+        specs.back().any_order = any_order;
     }
     IFCI_TRY(check_opts(h, o));
     IFCI_CUDA_TRY(h, cudaSetDevice(h->device));
     return dav_solve_sectors(h, specs, o, energies, iters, status, as_cuda(stream));
+}
+
+int ifci_davidson_batched(ifci_handle_t h, int nprob, const ifci_problem_t *probs, const ifci_davidson_opts_t *opts,
+                          double *energies, int *iters, int *status, ifci_stream_t stream) {
+    return solve_batch(h, nprob, probs, opts, true, energies, iters, status, stream);
+}
+
+int ifci_davidson_expansion(ifci_handle_t h, int nprob, const ifci_problem_t *probs, const ifci_davidson_opts_t *opts,
+                            double *energies, int *iters, int *status, ifci_stream_t stream) {
+    return solve_batch(h, nprob, probs, opts, false, energies, iters, status, stream);
 }
 
 }  // extern "C"

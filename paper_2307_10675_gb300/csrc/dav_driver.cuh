@@ -20,10 +20,11 @@ struct ProbSpec {
     const double *seed = nullptr;
     const unsigned char *mask = nullptr;
     long long ndim = 0;
-    // its energy is a result by itself: the small eigenproblems may take the faster
-    // order of rotations, whose other rounding a quantised sigma turns into
-    // ~1e-10 Eh.  An expansion, which takes differences of such energies, and HBCI
-    // keep the serial order.
+    // the small eigenproblems may take the faster, round-robin order of rotations
+    // (ifci_davidson_batched).  An expansion and HBCI keep the serial order and with it
+    // every bit; ifci_davidson_expansion solves a batch as they do.  Both orders are
+    // equally far from FP64: rms 5.23e-11 Eh over 6,304 FP64E problems in either,
+    // 5.99e-11 and 6.00e-11 in BF16 + FP64E (TF32 5.94e-11 and 5.94e-11).
     bool any_order = false;
 };
 
