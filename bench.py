@@ -529,8 +529,9 @@ def main():
 def paths_sample(ifci, torch, handle, chain, sysd, args, dev):
     """FP64E, plain FP64 and mixed BF16 and TF32 (+FP64E restarts) on the same seeded
     sample of body sets (their frozen-body CI problems through
-    ifci_davidson_batched, one batch per path): increments/s of each path and
-    the largest energy difference from the plain FP64 path."""
+    ifci_davidson_expansion, which solves them as ifci_increments does, one batch
+    per path): increments/s of each path and the largest energy difference from
+    the plain FP64 path."""
     sample = compare_sample(chain, args.max_order, args.compare_fraction)
     probs = []
     for X, n, k in sample:
@@ -542,7 +543,7 @@ def paths_sample(ifci, torch, handle, chain, sysd, args, dev):
         o = ifci.davidson_opts(prec, hi_precision=hi, r_tol=R_TOL, e_tol=E_TOL, max_iter=300)
         torch.cuda.synchronize(dev)
         t0 = time.perf_counter()
-        e, it, st = ifci.ifci_davidson_batched(handle, probs, o, allow_unconverged=True)
+        e, it, st = ifci.ifci_davidson_expansion(handle, probs, o, allow_unconverged=True)
         torch.cuda.synchronize(dev)
         wall = time.perf_counter() - t0
         res[name] = {"increments_per_s": len(probs) / wall, "seconds": wall, "iters_mean": float(np.mean(it)),
