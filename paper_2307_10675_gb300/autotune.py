@@ -1,18 +1,21 @@
 """Autotuner of the batched solver's launch parameters.
 
 The kernels' tile shapes are fixed by the hardware they are written for (128
-TMEM lanes per tile, five 96-column level accumulators in the 512 TMEM
-columns, 64-pair K atoms in shared memory), so what is left to choose per
-workload and GPU are the parameters of the batched solve itself:
+TMEM lanes per tile; FP64E: two sets of five 48-column level accumulators in
+the 512 TMEM columns, and the K rows of one alpha string in shared memory), so
+what is left to choose per workload and GPU are the parameters of the batched
+solve itself:
 
 * ``max_space``: Davidson subspace size before a thick restart (fewer
   restarts and iterations against more vector traffic per iteration; on a
   sample too small to fill the GPU a small subspace looks cheaper than it is
   at full scale, where the extra sigma builds dominate, so the grid starts at
   10);
-* ``det_budget``: D elements per sigma wave (how many problems one sigma
-  launch covers: larger waves fill the GPU better, smaller ones keep the
-  intermediates in L2);
+* ``det_budget``: D elements per sigma wave of the FP32, TF32 and BF16
+  contractions (how many problems one sigma launch covers: larger waves fill
+  the GPU better, smaller ones keep the intermediates in L2).  The FP64 sigma
+  has no intermediates and the FP64E one ~3.5 elements per determinant, of
+  which 2^31 hold a batch of 130 GB of Davidson vectors: one value for those;
 * ``graph_iters``: Davidson iterations captured per CUDA graph (0 = launched
   one by one), which removes launch latency for batches of small problems.
 
@@ -43,6 +46,13 @@ DEFAULT_GRID = {
     "det_budget": [1 << 31, 1 << 30],
     "graph_iters": [0, 4],
 }
+
+
+def default_grid(precision: str) -> Dict[str, List]:
+    grid = dict(DEFAULT_GRID)
+    if precision in ("fp64", "fp64e"):
+        grid["det_budget"] = grid["det_budget"][:1]
+    return grid
 
 
 def workload_signature(system: api.SystemArrays, sets: Sequence[Sequence[int]], precision: str, r_tol: float) -> str:
@@ -83,7 +93,7 @@ def autotune(handle: api.Handle, system: api.SystemArrays, sets: Sequence[Sequen
     ``system`` (body index tuples).  Returns {"params": {...}, "table": [...],
     "cached": bool}; ``table`` lists every timed candidate (seconds, energy
     deviation from the first candidate)."""
-    grid = dict(DEFAULT_GRID if grid is None else grid)
+    grid = dict(default_grid(precision) if grid is None else grid)
     dev_name = torch.cuda.get_device_name(handle.device)
     sig = workload_signature(system, sets, precision, r_tol)
     key = f"{dev_name}|{sig}"
