@@ -297,10 +297,7 @@ __device__ void jacobi_warp(double *A, double *V, int k, int lane) {
                 const bool rot = go && !tiny;
                 __syncwarp();   // every lane has read the rotation's entries
                 if (tiny && lane == 0) A[pp * LD + q] = A[q * LD + pp] = 0.0;
-                if (!__any_sync(0xffffffffu, rot)) {
-                    __syncwarp();   // orders the zeros written above, which a vote does not
-                    continue;
-                }
+                if (!__any_sync(0xffffffffu, rot)) continue;   // a barrier follows before the zeros are read
                 double c = 1.0, sn = 0.0;
                 if (rot) jacobi_rotation(app, aqq, apq, c, sn);
                 __syncwarp();
@@ -321,6 +318,7 @@ __device__ void jacobi_warp(double *A, double *V, int k, int lane) {
                 }
                 __syncwarp();
             }
+        __syncwarp();   // the next sweep reads the zeros of a last pair that did not rotate
     }
 }
 
