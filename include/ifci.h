@@ -149,14 +149,20 @@ typedef struct {
  *   c     : device double[nstr*nstr], input vector.
  *   sigma : device double[nstr*nstr], output (must not alias c).
  *   precision : ifci_precision_t of the contraction (FP64 exact path;
- *               the others round the contraction inputs, FP32 accumulate).
+ *               the others round the contraction inputs; FP32, TF32 and BF16
+ *               accumulate the contraction in FP32 and add up its FP32 results
+ *               over the excitations of a determinant in two floats, ~48 bits,
+ *               in FP64 where such a sum leaves FP32's range).
  * Sizes: BF16 and TF32 take npair <= 256 (norb <= 22), FP64E npair <= 304
- * (norb <= 24) and nstr <= 32767, else UNSUPPORTED (OOM for more strings).  The
- * intermediates take 2 * npair * nstr^2 elements of the precision's storage
- * type; FP64E takes 28 bytes per determinant instead (digit planes of c and
- * -c, and the integer sigma), 56 without IFCI_SIGMA_SPIN_SYMMETRIC.  Its sums
- * are integer sums: the result does not depend on their order.  Workspace
- * beyond the device's memory fails with OOM.
+ * (norb <= 24) and nstr <= 32767, else UNSUPPORTED (OOM for more strings); FP64
+ * takes nstr + npair <= 28160 (OOM beyond).  FP32, TF32 and BF16 take
+ * 2 * npair * nstr^2 4-byte elements of intermediates.  FP64 has none: it takes
+ * 12 bytes per nonzero element of the string Hamiltonian, nstr * (1 + m (n - m)
+ * + C(m,2) C(n-m,2)) of them for m electrons in n orbitals.  FP64E takes 28
+ * bytes per determinant (digit planes of c and -c, and the integer sigma), 56
+ * without IFCI_SIGMA_SPIN_SYMMETRIC.  Its sums are integer sums: the result does
+ * not depend on their order.  Workspace beyond the device's memory fails with
+ * OOM.
  * Asynchronous on `stream`; uses handle workspace (grows it if needed). */
 int ifci_sigma(ifci_handle_t handle, const ifci_strings_t *str,
                const double *h1, const double *eri, const double *c, double *sigma,
@@ -255,11 +261,11 @@ typedef struct {
                             precision always finishes on exact sigmas. */
     int hi_precision;    /* mixed mode: sigma of restart vectors, IFCI_FP64 or IFCI_FP64E
                             (default IFCI_FP64E) */
-    long long det_budget;/* D elements (npair x determinants) per sigma wave, on the FP64E path
-                            8-byte elements of its intermediates (~3.5 per determinant);
-                            0 = 2^31.  A problem above it alone takes a wave of its own on the
-                            FP64E path; on the other paths it fails with OOM.  The result does
-                            not depend on it */
+    long long det_budget;/* D elements (npair x determinants) per sigma wave of the FP32, TF32
+                            and BF16 contractions; on the FP64E path 8-byte elements of its
+                            intermediates (~3.5 per determinant); 0 = 2^31.  FP64 has no
+                            intermediates and one wave.  A problem above it alone takes a wave
+                            of its own.  The result does not depend on it */
     int graph_iters;     /* > 0: Davidson iterations are captured in blocks of this
                             many into one CUDA graph, replayed on a stream of the
                             handle (event-ordered with `stream`); 0 = launched one

@@ -330,10 +330,13 @@ __device__ void jacobi_warp(double *A, double *V, int k, int lane) {
 // the next step's rotations are derived (those of step `step` in buffer step & 1).
 // The chain of a step (~1200 clk to derive, 2 x 256 to mix) bounds it: 32 problems
 // of up to 12 vectors take 62 us on average, 194 us one rotation at a time.  FP64
-// solves and direct batches take it; in expansions and HBCI with a quantised
-// sigma another rounding here turns up at the contraction's own level (energies
-// of selected spaces moved by 7e-10 of themselves), so those keep the serial
-// order and every bit.
+// solves and direct batches take it.  Expansions and HBCI with a quantised sigma
+// keep the serial order and with it every bit: another rounding here turns up at
+// the contraction's own level (energies of selected spaces moved by 7e-10 of
+// themselves).  It does not turn up as a larger error: against tight FP64 solves
+// the rms of E_X over 1,304 sets in FP64E is 4.89e-11 Eh in the serial order and
+// 4.88e-11 in this one, at most 2.26e-10 in either; of 192 selected spaces' E_var
+// 6.32e-11 and 6.26e-11.
 constexpr int kPairSolveThreads = 128;
 
 template <int LD>

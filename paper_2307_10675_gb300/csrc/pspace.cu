@@ -564,12 +564,13 @@ __device__ __forceinline__ void psp_jacobi_refined(double *A, double *V, float *
 // 20.1 ms with one rotation at a time; less after an FP32 solve) and serves the
 // whole spaces of FP64 solves, where a last-bit change of the start vector stays
 // one, and of direct batches in every precision, whose energies it moves by
-// 1e-13 (FP64E) to 3e-11 (mixed) of themselves (a batch of two-body spaces in
-// FP64E: 18.9 ms, 4.2 ms with the Rayleigh-Ritz problems in that order too).  In
-// an expansion with a quantised contraction (FP64E and the mixed modes that end
-// on it) such a change turns up at the contraction's own level, ~5e-11 Eh, in
-// increments that are differences of energies, so those and HBCI keep the order
-// of rotations, and with it every bit of their start vectors, on five warps a
+// 1e-13 (FP64E) to 3e-11 (mixed) of themselves (32 spaces CAS(4e,10o) in FP64E:
+// 27.5 ms, 8.1 ms with the Rayleigh-Ritz problems in that order too).  In an
+// expansion with a quantised contraction (FP64E and the mixed modes that end on
+// it) such a change turns up at the contraction's own level, ~5e-11 Eh, in
+// increments that are differences of energies; it moves them without taking them
+// farther from FP64 (davidson.cu, jacobi_pairs).  Those and HBCI keep the order of
+// rotations, and with it every bit of their start vectors, on five warps a
 // problem: 64 functions 20.1 ms on one warp, 13.8 ms; 298 such problems at once
 // 21.9 ms, 15.7 ms; the P-space solves of an expansion of 298 sets 58.9 ms,
 // 42.9 ms.  So do the blocks of sectored spaces (MAXP = 24), which come by the

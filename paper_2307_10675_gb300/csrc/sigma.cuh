@@ -11,7 +11,8 @@ struct SigmaProb {
     int n, nstr, nexc, np;   // active orbitals, strings, excitations per string, pairs
     int ld;                  // row stride of W (>= np)
     int sym;                 // 1: the vector is spin-flip symmetric (C = C^T); the tensor-core paths gather
-                             // alpha excitations only and return S + S^T (set by plan_sigma, needs pmap)
+                             // alpha excitations only and return S + S^T (set by plan_sigma; BF16 and TF32
+                             // need pmap, FP64E jmap)
     long long ndet;
     long long stride;
     const int32_t *exc;      // [nstr * nexc] excitation table of (n, nelec_spin)
@@ -22,7 +23,7 @@ struct SigmaProb {
     const void *Wtc;         // tensor-core operand image (BF16 path) or nullptr
     const void *Woz;         // sliced operand image of the FP64-emulating path or nullptr
     double *Wexp;            // its power-of-two scale
-    double dscale;           // power of two >= max |D| (FP64-emulating path)
+    double dscale;           // scale of the digits of c, a power of two above max |c| (twice that where sym; FP64E)
     const uint16_t *jmap;    // excitation map over the contracted pairs (FP64-emulating path) or nullptr
     int ldj;
     long long qoff;          // element offset of the quantised copies of c in their wave buffer

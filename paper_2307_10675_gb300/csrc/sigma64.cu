@@ -20,8 +20,11 @@
 // One block per alpha string Ia.  The rows c[J_B] and the integral columns of
 // kb excitations B at a time sit in shared memory (the sign s_B is taken into
 // the rows), each thread owns determinants Ib = t, t + blockDim, ...; s_A flips
-// the accumulator's sign bit instead of costing a multiplication.  56 KB per
-// block leave four blocks on an SM, whose loads overlap another's FMAs.
+// the accumulator's sign bit instead of costing a multiplication.  58.9 KB per
+// block (54 KB of rows, 2.5 KB of lists, 1 KB of the system's) leave three blocks
+// on an SM, whose loads overlap another's FMAs.  Rows cut to 53.5 KB let a fourth
+// in: CAS(12e,12o) 4.49 ms, 3.86 ms; 64 problems of CAS(4e,12o) 4 % faster; but
+// eight of CAS(6e,12o) 22.6 ms, 22.9 ms, and CAS(6e,13o) 285 us, 289 us.
 //
 // Measured: CAS(6e,13o) 240 us and 9 us for the lists (dense contraction 1634 us,
 // gather and scatter 103 us before), 1.16e8 FMAs at 0.88 of a DGEMM's rate.
@@ -37,7 +40,7 @@ namespace {
 constexpr int kMaxThreads64 = 512;
 constexpr int kList = 128;              // alpha-alpha elements staged at a time
 constexpr int kMaxExc = (kMaxNorb + 1) * (kMaxNorb + 1) / 4;   // most excitations m (n - m + 1) of a string
-constexpr int kCapSmall = 6912, kCapMid = 13824, kCapLarge = 28160;   // doubles: 4, 2 or 1 blocks per SM
+constexpr int kCapSmall = 6912, kCapMid = 13824, kCapLarge = 28160;   // doubles: 3, 2 or 1 blocks per SM
 
 // the input row and the sums are kept in shared memory too, unless the strings
 // are too many for that

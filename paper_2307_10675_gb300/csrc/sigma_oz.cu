@@ -6,7 +6,9 @@
 // Ozaki-style splitting):
 //
 //   W[A][B] = Wscale 2^-7 (w1 + 2^-8 w2 + ... + 2^-32 w5)    Wscale >= max|W|
-//   c[K]    = dscale  2^-6 (d1 + 2^-8 d2 + ... + 2^-32 d5)    dscale >= 2 max|c|
+//   c[K]    = dscale  2^-6 (d1 + 2^-8 d2 + ... + 2^-32 d5)    dscale > max|c|
+//
+// (dscale > 2 max|c| for spin-flip-symmetric c),
 //
 // with every slice an integer in [-128, 128], exact in FP16: c becomes the
 // fixed-point integer X = round(c 2^38 / dscale), whose slices are the
@@ -257,9 +259,9 @@ struct OzGeom {
     uint32_t m8, m16, m24;   // 2^8, 2^16, 2^24, in registers: one multiply-add per level instead of a shift and two adds
 };
 
-// The biased value of T from its level sums: each level as kMagic + acc, so
-// T + kBias = sum_L (kMagic + acc_L) 2^{8 (4 - L)} needs no sign handling.
-// T of levels that may reach 2^24 (levels 0 and 1 stay below 2^22 = 2 2^14 kMaxK)
+// T of levels that may reach 2^24; levels 0 and 1 (at most two products of 2^14 a
+// row) stay below 2^22 and take the biased form.
+static_assert(2 * (1 << 14) * kMaxK < (1 << 22), "levels 0 and 1 of the wide form");
 __device__ __forceinline__ unsigned long long wide_sum(float sg, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                        uint32_t a4) {
     const uint32_t h = __float_as_uint(fmaf(sg, __uint_as_float(a0), 12582912.0f)) - kMagic;
@@ -270,6 +272,8 @@ __device__ __forceinline__ unsigned long long wide_sum(float sg, uint32_t a0, ui
     T += (long long)(int)l * 16777216;
     return (unsigned long long)T + ((unsigned long long)h << 32);
 }
+// The biased value of T from its level sums: each level as kMagic + acc, so
+// T + kBias = sum_L (kMagic + acc_L) 2^{8 (4 - L)} needs no sign handling.
 constexpr unsigned long long kBias = (unsigned long long)kMagic * 0x0101010101ull;
 __device__ __forceinline__ unsigned long long biased(const uint32_t (&b)[kS], const OzGeom &g) {
     unsigned long long t = mad_wide(b[3], g.m8, b[4]);
@@ -875,9 +879,10 @@ __global__ void __launch_bounds__(256) oz_compact_maps_kernel(const OzMapDesc *_
     }
 }
 
-// A single problem is prepared in two launches around its two maxima: CAS(6e,12o)
-// takes 41 us a call, 92 us with one launch per step (fold, max W, pack, map,
-// max c, scale, quantise: 62 us of device time before the contraction).
+// A single problem is prepared in two launches around its two maxima: CAS(4e,12o)
+// takes 37 us a call (41 us with the plan's arrays copied one by one), 92 us with
+// one launch per step (fold, max W, pack, map, max c, scale, quantise: 62 us of
+// device time before the contraction).
 
 // Largest |x| of the block's values to *out (as ordered bits; NaN left out).
 __device__ __forceinline__ void block_max_bits(long long m, unsigned long long *out) {

@@ -42,7 +42,7 @@ __device__ __forceinline__ void jacobi_rotation(double app, double aqq, double a
 }
 
 // |apq| <= 1e-18 (|app| + |aqq|): decided by the exponents unless they are
-// within reach of the threshold (1e-18 > 2^-60, the sum is below 2^(e + 2))
+// within reach of the threshold (1e-18 < 2^-59, the sum is below 2^(e + 2))
 __device__ __forceinline__ bool jacobi_negligible(double app, double aqq, double apq) {
     const int em = max(dexp_field(app), dexp_field(aqq));
     if (em < 2047 && dexp_field(apq) - em >= -57) return false;
