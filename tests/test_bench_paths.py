@@ -1,5 +1,5 @@
-"""bench.paths_sample reports the solver that an expansion runs (no GPU: the
-library is a stand-in that records the calls)."""
+"""bench.py reports what runs (no GPU): the solver of the path comparison (the
+library is a stand-in that records the calls) and the operations of a sigma."""
 import os
 import sys
 from types import SimpleNamespace
@@ -29,3 +29,11 @@ def test_paths_sample_solves_as_an_expansion():
     out = bench.paths_sample(lib, torch, None, chain_24_uneven(), None, args, None)
     assert calls == ["fp64e", "fp64", "bf16", "tf32"]
     assert set(out["runs"]) == {"fp64e", "fp64", "bf16_mixed", "tf32_mixed"}
+
+
+def test_sigma_flops_of_the_fp64_path():
+    # H of CAS(6e,13o), row by row of one determinant's excitations: the diagonal, 30 singles and
+    # 135 doubles of each spin; 33 excitations (diagonal ones among them) of each spin at once
+    assert bench.sigma_flops("fp64", 13, 3, 91) == 2.0 * 286 ** 2 * (33 ** 2 + 2 * 166)
+    assert bench.sigma_flops("bf16", 13, 3, 91) == 2.0 * 286 ** 2 * 91 ** 2
+    assert bench.sigma_flops("fp64e", 13, 3, 91) == 2.0 * 286 ** 2 * 91 * 33
