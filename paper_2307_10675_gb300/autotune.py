@@ -22,7 +22,11 @@ solve itself:
 Every candidate is timed on the same seeded sample of the workload's CI
 problems (their frozen-body Hamiltonians, one ``ifci_davidson_expansion`` call
 each, which solves them as an expansion does, after one untimed call); a candidate whose energies differ from the
-first candidate's by more than ``tol`` is rejected.  The choice is cached in
+first candidate's by more than ``tol`` is rejected, and one that is not faster
+than the best so far by more than ``MARGIN`` does not replace it: a run of the
+sample differs by about 1 % from the next, and a smaller subspace that ties on
+it (2.985 s, 2.986 s on a quarter of the 40-body chain) takes 12.53 s for the
+whole expansion, the default 12.23 s.  The choice is cached in
 a JSON file keyed by the GPU name and a signature of the workload, and the
 search is coordinate-wise (one parameter at a time, the others at their
 best so far).  All arithmetic runs in the library; this module only times
@@ -46,6 +50,9 @@ DEFAULT_GRID = {
     "det_budget": [1 << 31, 1 << 30],
     "graph_iters": [0, 4],
 }
+
+
+MARGIN = 0.02
 
 
 def default_grid(precision: str) -> Dict[str, List]:
@@ -124,7 +131,7 @@ def autotune(handle: api.Handle, system: api.SystemArrays, sets: Sequence[Sequen
             dev = float(np.max(np.abs(e - ref_e))) if e is not None else float("inf")
             ok = t < float("inf") and dev <= tol
             table.append({"params": cand, "seconds": t, "max_abs_energy_deviation": dev, "accepted": ok})
-            if ok and t < best_t:
+            if ok and t < (1.0 - MARGIN) * best_t:
                 best_t = t
                 best = cand
     out = {"params": best, "table": table, "cached": False}
