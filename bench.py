@@ -37,10 +37,11 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "iFCI increments/s & sigma TFLOP/s, 1 GB300, batched+mixed vs plain FP64 @1µEh"
-# dram__bytes_read.sum + dram__bytes_write.sum of one oz_sigma_kernel launch on
-# CAS(6e,18o) per determinant (ncu capture of one FP64E sigma); set to None
-# whenever that kernel changes until it is captured again
-OZ_DRAM_BYTES_PER_DET = 19.46e6 / 665856
+# dram__bytes_read.sum + dram__bytes_write.sum of one oz_sigma_kernel launch per
+# determinant (ncu capture of a Davidson batch of 16 CAS(6e,18o) in FP64E, whose
+# digit planes and integer sigmas, 298 MB, exceed the L2 as a step's do); set to
+# None whenever that kernel changes until it is captured again
+OZ_DRAM_BYTES_PER_DET = (304.7e6 + 63.3e6) / (16 * 665856)
 UNIT = "increments/s"
 
 
