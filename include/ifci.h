@@ -336,10 +336,11 @@ int ifci_davidson_batched(ifci_handle_t handle, int nprob, const ifci_problem_t 
                           int *status, ifci_stream_t stream);
 
 /* ifci_davidson_expansion — the same batch solved as ifci_increments solves its
- * body sets: the small eigenproblems in the serial order, so the energies are
- * those of ifci_increments bit for bit.  Slower than ifci_davidson_batched
- * where many small problems run in a quantised or mixed precision; the same
- * call in FP64. */
+ * body sets: the small eigenproblems in the serial order, so the energies of
+ * the same sets are those of ifci_increments bit for bit (a set by itself too,
+ * but in FP64, where the largest space of a batch decides how sums are split).
+ * Slower than ifci_davidson_batched where small problems run in a quantised or
+ * mixed precision; the same call in FP64. */
 int ifci_davidson_expansion(ifci_handle_t handle, int nprob, const ifci_problem_t *probs,
                             const ifci_davidson_opts_t *opts, double *energies, int *iters,
                             int *status, ifci_stream_t stream);

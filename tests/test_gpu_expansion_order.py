@@ -48,3 +48,14 @@ def test_the_autotuner_times_it(monkeypatch):
     with ifci.Handle(0, 0) as h:
         out = autotune.autotune(h, _system(), [(0, 1), (1, 2, 3)], "fp64e", grid={"max_space": [12, 8]})
     assert calls == [2] * (1 + len(out["table"]))
+
+
+def test_a_set_by_itself():
+    with ifci.Handle(0, 0) as h:
+        system = _system()
+        opts = ifci.davidson_opts("fp64e")
+        out = ifci.ifci_increments(h, system, 2, opts)
+        for i, X in enumerate(ifci.body_subsets(len(SIZES), 2)):
+            h1, eri, e_core = ifci.ifci_frozen_core(h, system, list(X))
+            e, _, _ = ifci.ifci_davidson_expansion(h, [ifci.CIProblem(h1.shape[0], len(X), h1, eri, e_core)], opts)
+            assert e[0] == out["e_x"][i], X
